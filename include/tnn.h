@@ -157,11 +157,13 @@ typedef struct {
     double lag;            /* t_w >= 0 (s): valid iff t_j < t_q - lag        */
     int32_t seed_segments; /* F: the F segments of smallest bound are scanned
                               first (Algorithm 2 fetches F segments, nearest
-                              first), 1..6 (0 = default 4)                    */
+                              first), 1..6 (0 = default 4); the grid order
+                              takes them one by one and ignores it            */
     int32_t seed_window;   /* at most this many of the most recent causal
                               segments are searched for those F
                               (0 = no limit, the default)                     */
-    int32_t extra;         /* candidate slots kept beyond k, 2..32 (0 = 4)   */
+    int32_t extra;         /* candidate slots kept beyond k, 2..32 (0 = 4);
+                              the grid order's shared tiles always keep 4     */
     int32_t flags;         /* TNN_FLAG_*                                      */
     float defer_cells;     /* grid order: a query whose k-th candidate after
                               seeding is farther than defer_cells grid cells

@@ -13,14 +13,14 @@
 
 static const unsigned long long SENT = (0x7f800000ull << 32) | 0xffffffffull;
 
-// Shared-memory layout per warp of the tile kernels.
-enum { SMEM_SWEEP = 0, SMEM_LINEAR = 1, SMEM_GRID = 2 };
+// Shared-memory layout per warp of the sweep and linear kernels.
+enum { SMEM_SWEEP = 0, SMEM_LINEAR = 1 };
 
 __host__ __device__ inline size_t smem_per_warp(int L_max, int kseg_max, int mode)
 {
-    // candidate lists [L_max][32] keys, then: sweep and grid: segment chunk
+    // candidate lists [L_max][32] keys, then: sweep: segment chunk
     // [32][4] float4 | points [kseg_max] float4 | seed union [TNN_UCAP] int
-    // (| pass-1 list [TNN_WCAP] int for the sweep); linear search: points
+    // | pass-1 list [TNN_WCAP] int; linear search: points
     // [32] float4 | indices [32] int.  The FP64 settlement scratch
     // ([CMAX][32] u64 + [CMAX][32] int) reuses that area.
     size_t base = (size_t)L_max * 32 * 8;

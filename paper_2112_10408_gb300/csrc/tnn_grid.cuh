@@ -1,30 +1,47 @@
 // TNN search over the time-bucketed spatial grid of the index.
 //
-// Same tiles, candidate lists, seeds and settlement as the sweep kernel
-// (tnn_search.cuh); only the order in which segments are considered
-// changes.  A key of the grid (bucket of t_A, cell of the midpoint) has its
-// own lower bound -- distance from the query to the cell rectangle minus the
-// key's extent, plus the temporal part from the key's largest t_B -- which
-// never exceeds the cylinder bound of any member segment, so whole keys are
-// excluded at once by the exclusion criterion of Sec. 3.4.
+// One warp answers a tile of up to 32 queries, one query per lane.  A key of
+// the grid (bucket of t_A, cell of the midpoint) has its own lower bound --
+// distance from the query to the cell rectangle minus the key's extent, plus
+// the temporal part from the key's largest t_B -- which never exceeds the
+// cylinder bound of any member segment, so whole keys are excluded at once by
+// the exclusion criterion of Sec. 3.4.
 //
-//   seeds   the 3 x 3 cells around the warp in the three most recent buckets:
-//           every lane keeps its F smallest cylinder bounds there; the union
-//           of those segments is scanned first (Algorithm 2's first fetch).
+//   near    the segments of the 3 x 3 cells around the tile in the newest
+//           buckets, 32 at a time: every lane's cylinder bounds, then the
+//           segments by ascending bound (over the lanes) while some lane's
+//           bound does not exceed its pruning key (Algorithm 2 fetches the
+//           nearest first).
 //   main    buckets from the causal end backwards; a bucket is visited while
 //           the temporal bound of its running maximum of t_B does not exceed
-//           some lane's pruning key (Algorithm 2's stop rule); inside it, the
-//           cells within reach of the warp's queries, and inside a cell whose
-//           bound does not exceed a lane's key, the member segments whose
-//           cylinder bound does not exceed it are scanned for that lane.
+//           some lane's pruning key (Algorithm 2's stop rule); inside it the
+//           other cells within reach, the keys whose bound does not exceed a
+//           lane's key, and their segments as above.
+//
+// Points reach the lists 32 at a time.  A lane keeps its candidates as sorted
+// 32-bit keys in registers: the upper bits of the FP32 distance above the
+// point's slot in a per-tile table.  Every 8 points are sorted by Batcher's
+// odd-even merge network and merged with the list by a bitonic network:
+// minima and maxima only, no branch, no shared memory, every lane in step.
+// At the end the distances of the k + 4 smallest are taken again in full FP32
+// and settled as before.
+//
+// Bound: issue and latency of this arithmetic (data are L2-resident; DRAM
+// sees little more than the written lists).  A sorted 64-bit list per lane in
+// shared memory, with one insertion per candidate, spent half of the kernel
+// in chains of dependent loads and stores at a different moment in every
+// lane: 615 us for 400,000 flight samples at k = 32 and 6,774 us for
+// 4,000,000; the networks take 284 and 3,088 us, the latency of a single tile
+// (10,000 points, k = 8) falls from 170 to 80 us.  The instruction cache sets
+// the batch: straight-line code for 32 points a time executes the fewest
+// instructions but streams its code (459 us, over half of the stall cycles
+// waiting for instructions), 16 take 306 and 8 take 284 us; for the same
+// reason everything done once per tile is rolled into short loops.
 #pragma once
 #include "tnn_device.cuh"
 
-#ifndef TNN_GMAX_F
-#define TNN_GMAX_F 6
-#endif
 #ifndef TNN_SEED_BUCKETS
-#define TNN_SEED_BUCKETS 3 // newest buckets whose 3 x 3 cells seed a tile (at most 3)
+#define TNN_SEED_BUCKETS 3 // newest buckets whose 3 x 3 cells start a tile (at most 3)
 #endif
 
 // Lower bound on the cylinder bound (and so on the FP32 distance of any
@@ -70,34 +87,258 @@ __device__ __forceinline__ float warp_maxf(float v)
     return v;
 }
 
-#ifndef TNN_GRID_MINB
-#define TNN_GRID_MINB 4
-#endif
+// ------------------------------------------------- candidate keys, networks
 
-// MIRROR: also copy each finished tile's rows to KnnLaunch::mirror_idx /
-// mirror_d2 (a separate instantiation, so that the plain search compiles
-// without that code).
-template <bool MIRROR>
-__global__ void __launch_bounds__(TNN_WARPS_PER_CTA * 32, TNN_GRID_MINB)
+#define TG_SLOT_BITS 10 // point slots of a tile; 14 mantissa bits of the distance remain
+#define TG_SLOTS (1 << TG_SLOT_BITS)
+#define TG_SMASK (TG_SLOTS - 1u)
+#define TG_EMPTY 0xffffffffu // sorts after every key
+#define TG_INF 0xff000000u   // keys of infinite distances
+#define TG_EXTRA 4           // candidates kept beyond the k-th
+#define TG_NB 8        // points sorted at a time
+#define TG_INSERT 5          // batches with at most this many candidates are inserted one by one
+#define TG_MIN_GROUP 3       // smaller groups of a tile go to the warp-per-query kernel
+
+// Key of a distance (>= 0) in slot `s`: its bits without the sign, the lowest
+// replaced by the slot.  Keys of one lane order like the distances up to the
+// 2^-14 that the slot displaces.
+__device__ __forceinline__ unsigned tg_key(float d, unsigned s)
+{
+    return ((__float_as_uint(d) << 1) & ~TG_SMASK) | s;
+}
+// Smallest and largest distance a key can stand for.
+__device__ __forceinline__ float tg_lower(unsigned key) { return __uint_as_float((key & ~TG_SMASK) >> 1); }
+__device__ __forceinline__ float tg_upper(unsigned key) { return __uint_as_float((key | TG_SMASK) >> 1); }
+
+__device__ __forceinline__ void tg_cmpx(unsigned &a, unsigned &b)
+{
+    const unsigned lo = min(a, b), hi = max(a, b);
+    a = lo;
+    b = hi;
+}
+
+// Batcher's odd-even merge sort (K. E. Batcher, Sorting networks and their
+// applications, 1968): comparators of round (P, K).
+template <int N, int P, int K> __device__ __forceinline__ void tg_sort_round(unsigned (&v)[N])
+{
+#pragma unroll
+    for (int x = K % P; x + K < N; ++x)
+        if ((x - K % P) % (2 * K) < K && x / (2 * P) == (x + K) / (2 * P))
+            tg_cmpx(v[x], v[x + K]);
+    if constexpr (K > 1)
+        tg_sort_round<N, P, K / 2>(v);
+}
+template <int N, int P = 1> __device__ __forceinline__ void tg_sort(unsigned (&v)[N])
+{
+    tg_sort_round<N, P, P>(v);
+    if constexpr (2 * P < N)
+        tg_sort<N, 2 * P>(v);
+}
+// Ascending order of a bitonic sequence.
+template <int N, int H = N / 2> __device__ __forceinline__ void tg_bitonic(unsigned (&v)[N])
+{
+#pragma unroll
+    for (int x = 0; x < N; ++x)
+        if ((x & H) == 0)
+            tg_cmpx(v[x], v[x + H]);
+    if constexpr (H > 1)
+        tg_bitonic<N, H / 2>(v);
+}
+// First H values of a bitonic sequence of 2 H: its H smallest, bitonic again.
+template <int N, int H = N / 2> __device__ __forceinline__ void tg_smallest4(unsigned (&v)[N])
+{
+#pragma unroll
+    for (int x = 0; x < H; ++x)
+        v[x] = min(v[x], v[x + H]);
+    if constexpr (H > TG_EXTRA)
+        tg_smallest4<N, H / 2>(v);
+}
+
+// Merge the sorted batch b into the sorted list a (the NL smallest keys stay)
+// and what leaves it into the TG_EXTRA next ones o.
+template <int NL, int NB>
+__device__ __forceinline__ void tg_merge(unsigned (&a)[NL], unsigned (&o)[TG_EXTRA], const unsigned (&b)[NB])
+{
+    unsigned r[NB];
+#pragma unroll
+    for (int i = 0; i < NB; ++i) {
+        const unsigned x = a[NL - NB + i], y = b[NB - 1 - i];
+        a[NL - NB + i] = min(x, y);
+        r[i] = max(x, y);
+    }
+    tg_bitonic<NL>(a);
+    tg_smallest4<NB>(r);
+    unsigned e[TG_EXTRA];
+#pragma unroll
+    for (int i = 0; i < TG_EXTRA; ++i)
+        e[i] = r[i];
+    tg_bitonic<TG_EXTRA>(e);
+#pragma unroll
+    for (int i = 0; i < TG_EXTRA; ++i)
+        o[i] = min(o[i], e[TG_EXTRA - 1 - i]);
+    tg_bitonic<TG_EXTRA>(o);
+}
+
+template <int NL>
+__device__ __forceinline__ void tg_insert(unsigned (&a)[NL], unsigned (&o)[TG_EXTRA], unsigned key)
+{
+#pragma unroll
+    for (int i = 0; i < NL; ++i) {
+        const unsigned t = min(a[i], key);
+        key = max(a[i], key);
+        a[i] = t;
+    }
+#pragma unroll
+    for (int i = 0; i < TG_EXTRA; ++i) {
+        const unsigned t = min(o[i], key);
+        key = max(o[i], key);
+        o[i] = t;
+    }
+}
+
+// ------------------------------------------------------------ shared memory
+
+// Per warp.  While points are gathered: the batch's points, staged segments,
+// their bounds (upper halves of the floats), the slots in use and their
+// prefix, the key ranges' ends and offsets; the slot table behind them.  To
+// settle, the lists' 32-bit keys take the first part's place, and then the
+// 64-bit lists [NL + TG_EXTRA + 1][32] everything's.
+template <int NL> struct TileSmem {
+    union {
+        struct {
+            float4 pts[32];
+            float4 seg[32][3];
+            uint16_t lb[32][32];
+            unsigned used[32];
+            int pre[32];
+            int kend[32];
+            int krel[32];
+        };
+        unsigned raw[NL + TG_EXTRA][32];
+    };
+    int slot[TG_SLOTS];
+};
+
+template <int NL> __host__ __device__ constexpr size_t tg_smem_per_warp()
+{
+    const size_t lists = (size_t)(NL + TG_EXTRA + 1) * 256;
+    return lists > sizeof(TileSmem<NL>) ? lists : sizeof(TileSmem<NL>);
+}
+
+// Entry e of a lane's settled list: the lane's column is rotated by the entry
+// so that both a column (settlement) and a row (output) are read without bank
+// conflicts.
+__device__ __forceinline__ unsigned long long *tg_entry(unsigned long long *Kw, int e, int lane)
+{
+    return Kw + e * 32 + (lane ^ (e & 31));
+}
+
+// Settle one query whose n exact keys (list rows z ...) are not yet in certain order: sort
+// them, drop those at or above `bound` (every point outside the list lies at
+// or above it), then rank chains of close keys in FP64, in place.  Bit 0 of
+// the result: settled; the rest counts the FP64 distances.  Out of line: a
+// few per cent of the queries come here.
+static __device__ __noinline__ unsigned tg_settle(const KnnWin *W, float4 q, unsigned long long *Kw,
+                                                  int lane, int z, int n, float bound)
+{
+    for (int i = 1; i < n; ++i) {
+        const unsigned long long v = *tg_entry(Kw, z + i, lane);
+        int j = i;
+        while (j > 0) {
+            const unsigned long long u = *tg_entry(Kw, z + j - 1, lane);
+            if (u <= v)
+                break;
+            *tg_entry(Kw, z + j, lane) = u;
+            --j;
+        }
+        if (j < i)
+            *tg_entry(Kw, z + j, lane) = v;
+    }
+    const bool full = bound < INFINITY;
+    if (full) {
+        while (n > 0 && key_d(*tg_entry(Kw, z + n - 1, lane)) >= bound)
+            --n;
+        *tg_entry(Kw, z + n, lane) = pack_key(bound, 0x7fffffff); // end marker
+        ++n;
+    }
+    const int k = W->k;
+    const bool exact_all = (W->flags & TNN_FLAG_EXACT_D2) != 0;
+    unsigned nfp = 0;
+    int i = 0;
+    while (i < k && i < n) {
+        const unsigned long long ki = *tg_entry(Kw, z + i, lane);
+        if (ki == SENT)
+            break;
+        int e = i;
+        float de = key_d(ki);
+        while (e + 1 < n) {
+            const unsigned long long kn = *tg_entry(Kw, z + e + 1, lane);
+            const float dn = key_d(kn);
+            if (kn == SENT || !(dn <= fmaf(de, 0x1p-17f, de) + 0x1p-100f))
+                break;
+            ++e;
+            de = dn;
+        }
+        const int c = e - i + 1;
+        if ((full && e == n - 1) || c > CMAX)
+            return nfp << 1;
+        if (c > 1 || exact_all) {
+            double dd[CMAX];
+            int id[CMAX];
+            for (int t = 0; t < c; ++t) {
+                const int j = key_i(*tg_entry(Kw, z + i + t, lane));
+                const double d = dist64(W->sigd, q, W->pts[j]);
+                ++nfp;
+                int pos = t;
+                while (pos > 0 && (dd[pos - 1] > d || (dd[pos - 1] == d && id[pos - 1] > j))) {
+                    dd[pos] = dd[pos - 1];
+                    id[pos] = id[pos - 1];
+                    --pos;
+                }
+                dd[pos] = d;
+                id[pos] = j;
+            }
+            for (int t = 0; t < c; ++t)
+                *tg_entry(Kw, z + i + t, lane) = pack_key((float)dd[t], id[t]);
+        }
+        i = e + 1;
+    }
+    if (full && i < k)
+        return nfp << 1;
+    return (nfp << 1) | 1u;
+}
+
+// Cells of the newest buckets in the order they are staged: the tile's own
+// first, then its neighbours, by bucket age.  db * 16 + (dy + 1) * 4 + dx + 1.
+static __device__ const unsigned char tg_seed_cell[32] = {
+    5,  21, 4,  6,  1,  9,  20, 22, 17, 25, 0,  2,  8,  10, 16, 18, 24, 26, 37, 36, 38, 33, 41, 32, 34, 40, 42,
+    0,  0,  0,  0,  0};
+
+// CTAs per SM: the list's registers (list + batch) set it.
+template <int NL> struct TileCtas {
+    static constexpr int value = NL == 64 ? 3 : NL == 32 ? 4 : 6;
+};
+
+// The grid-order tile kernel for k <= NL.  A list shorter than NL keys holds
+// zeros in front (they never leave and are skipped at the end), so that its
+// last key is the k-th smallest.
+template <int NL>
+__global__ void __launch_bounds__(TNN_WARPS_PER_CTA * 32, TileCtas<NL>::value)
     k_tnn_grid_search(const __grid_constant__ KnnLaunch L)
 {
+    constexpr int NB = NL < TG_NB ? NL : TG_NB; // points per network batch
     extern __shared__ __align__(16) unsigned char smem[];
     const int lane = threadIdx.x & 31;
-    const size_t pw = smem_per_warp(L.L_max, L.kseg_max, SMEM_GRID);
-    unsigned char *ws = smem + (threadIdx.x >> 5) * pw;
-    unsigned long long *K = (unsigned long long *)ws + lane;
-    unsigned char *rest = ws + (size_t)L.L_max * 256;
-    float4 *segbuf = (float4 *)rest;                     // [32][4]
-    float4 *pbuf = (float4 *)(rest + 2048);              // [kseg_max]
-    int *ulist = (int *)(rest + 2048 + 16 * L.kseg_max); // [TNN_UCAP] seeds
-    unsigned long long *cl_d = (unsigned long long *)rest + lane;
-    int *cl_i = (int *)(rest + CMAX * 32 * 8) + lane;
+    unsigned char *ws = smem + (threadIdx.x >> 5) * tg_smem_per_warp<NL>();
+    TileSmem<NL> &S = *(TileSmem<NL> *)ws;
+    unsigned long long *Kw = (unsigned long long *)ws;
+    const int seed_cell = tg_seed_cell[lane];
 
-    LaneStats st = {0, 0, 0, 0, 0};
+    unsigned n_q = 0, n_lb = 0, n_pairs = 0, n_segs = 0, n_fp = 0;
     for (;;) {
         long long tile = 0;
         if (lane == 0)
-            tile = (long long)atomicAdd(&L.scr->tile_counter, 1ull);
+            tile = L.tile_lo + (long long)atomicAdd(&L.scr->tile_counter[L.queue], 1ull);
         tile = __shfl_sync(FULLMASK, tile, 0);
         if (tile >= L.total_tiles)
             break;
@@ -105,334 +346,513 @@ __global__ void __launch_bounds__(TNN_WARPS_PER_CTA * 32, TNN_GRID_MINB)
         int64_t qrow;
         const bool active = tile_query(W, tile, lane, qrow);
         const float4 q = active ? W->q[qrow] : make_float4(0.f, 0.f, 0.f, 0.f);
-        const QCtx c = make_qctx(W, q, active);
         const float s0 = W->sig[0], s1 = W->sig[1], s2 = W->sig[2], s3 = W->sig[3];
-        const float4 *__restrict__ seg = W->seg;
         const float4 *__restrict__ pts = W->pts;
         const GridDesc &G = W->grid;
-        const int32_t *__restrict__ goff = G.off;
-        const int Lw = W->L, F = W->F;
+        const float tau_defer = W->tau_defer;
+        const int k = W->k;
+        const float ext_max = __ldg(G.ext_max);
+        if (active)
+            n_q++;
+
+        // A tile whose queries lie far apart (the caller's own order, two
+        // flights in one tile) is answered in groups around its first query
+        // not yet taken; lanes of tiny groups get a warp of their own.
+        unsigned todo = __ballot_sync(FULLMASK, active);
+        unsigned lone = 0;
+        while (todo) {
+        unsigned grp = todo;
+        if (tau_defer < INFINITY) {
+            const int ld = __ffs(todo) - 1;
+            const float gx = W->ssq[0] * q.x, gy = W->ssq[1] * q.y;
+            const float lx = __shfl_sync(FULLMASK, gx, ld), ly = __shfl_sync(FULLMASK, gy, ld);
+            const float lt = __shfl_sync(FULLMASK, q.w, ld);
+            const bool near = fabsf(gx - lx) <= 1.5f * G.cell && fabsf(gy - ly) <= 1.5f * G.cell &&
+                              fabsf(q.w - lt) <= 1.5f * G.dt;
+            grp = __ballot_sync(FULLMASK, near) & todo;
+            grp |= 1u << ld;
+            todo &= ~grp;
+            if (__popc(grp) < TG_MIN_GROUP) {
+                lone |= grp;
+                continue;
+            }
+        } else {
+            todo = 0;
+        }
+        const bool act = (grp >> lane) & 1u;
+        const QCtx c = make_qctx(W, q, act);
 
         const float tmax = warp_maxf(c.T32);
-        const float bx0 = warp_minf(active ? c.sx : INFINITY);
-        const float bx1 = warp_maxf(active ? c.sx : -INFINITY);
-        const float by0 = warp_minf(active ? c.sy : INFINITY);
-        const float by1 = warp_maxf(active ? c.sy : -INFINITY);
-        const float dmax = warp_maxf(active ? c.delta : 0.0f);
-        const float ext_max = __ldg(G.ext_max);
+        const float bx0 = warp_minf(act ? c.sx : INFINITY);
+        const float bx1 = warp_maxf(act ? c.sx : -INFINITY);
+        const float by0 = warp_minf(act ? c.sy : INFINITY);
+        const float by1 = warp_maxf(act ? c.sy : -INFINITY);
         int bhi = -1;
         {
             const float fb = (tmax - G.t0) * G.inv_dt;
             if (fb >= 0.0f)
                 bhi = (int)fminf(floorf(fb), (float)(G.nb - 1));
         }
+        const int hx = min(max((int)floorf((0.5f * (bx0 + bx1) - G.x0) * G.inv_cell), 0), G.nx - 1);
+        const int hy = min(max((int)floorf((0.5f * (by0 + by1) - G.y0) * G.inv_cell), 0), G.ny - 1);
 
-        for (int i = 0; i < Lw; ++i)
-            K[i * 32] = SENT;
-        int nv = 0;
-        unsigned long long tauk = SENT;
+        unsigned a[NL], o[TG_EXTRA];
+#pragma unroll
+        for (int i = 0; i < NL; ++i)
+            a[i] = i < NL - k ? 0u : TG_EMPTY;
+#pragma unroll
+        for (int i = 0; i < TG_EXTRA; ++i)
+            o[i] = TG_EMPTY;
+        // Pruning key: points above it are not needed.  A little above the
+        // k-th key so that every point its FP64 settlement may involve is seen.
         float tau = INFINITY;
-        bool done = !active;
+        // what a segment's bound is compared with in the present phase
+        float lim = act ? tau_defer : -1.0f;
+        bool given_up = false; // more distinct candidates than slots (warp-uniform)
+        bool deferred = false;
 
-        auto scan_pbuf = [&](int first, int cnt, bool need) {
-            if (!need)
-                return;
-            st.segs++;
-            st.pairs += cnt;
-            if (L.dbg_seen)
-                dbg_mark_seen(L, qrow, first, cnt);
-            // newest member first: along a trajectory the members nearest a
-            // later query come last, and keys arriving in ascending order
-            // make the sorted insertion an append
-            auto consider = [&](const float4 &p, float d, int id) {
-                if (p.w < c.T32 && d <= tau) {
-                    const unsigned long long key = pack_key(d, id);
-                    if (key < tauk) {
-                        tauk = lane_push(K, Lw, nv, key);
-                        tau = key_d(tauk);
-                    }
-                }
-            };
-            int j = cnt - 1;
-            // four members per step: their loads and distance chains overlap
-            for (; j >= 3; j -= 4) {
-                const float4 pa = pbuf[j], pb = pbuf[j - 1], pc = pbuf[j - 2], pd = pbuf[j - 3];
-                const float da = dist32(c, s0, s1, s2, s3, pa), db = dist32(c, s0, s1, s2, s3, pb);
-                const float dc = dist32(c, s0, s1, s2, s3, pc), dd = dist32(c, s0, s1, s2, s3, pd);
-                consider(pa, da, first + j);
-                consider(pb, db, first + j - 1);
-                consider(pc, dc, first + j - 2);
-                consider(pd, dd, first + j - 3);
-            }
-            for (; j >= 0; --j) {
-                const float4 p = pbuf[j];
-                consider(p, dist32(c, s0, s1, s2, s3, p), first + j);
-            }
-        };
-        auto scan_chunk = [&](unsigned any, unsigned need) {
-            if (!any)
-                return;
-            SegPoints cur, nxt;
-            int i = 31 - __clz(any);
-            any &= ~(1u << i);
-            seg_points_load(cur, pts, segbuf[4 * i + 3], lane);
-            for (;;) {
-                int inx = -1;
-                if (any) {
-                    inx = 31 - __clz(any);
-                    any &= ~(1u << inx);
-                    seg_points_load(nxt, pts, segbuf[4 * inx + 3], lane);
-                }
-                __syncwarp();
-                seg_points_store(cur, pbuf, lane);
-                __syncwarp();
-                scan_pbuf(cur.first, cur.cnt, (need >> i) & 1u);
-                if (inx < 0)
-                    break;
-                cur = nxt;
-                i = inx;
-            }
-        };
+        int base = 0, fill = 0, myidx = 0; // next slot; points gathered so far, this lane's
+        int b = bhi + 1, t0 = 0, ncells = 0, cx0 = 0, cy0 = 0, wx = 1; // main phase
+        bool near_phase = true;
+        int total = 0, pos = 0; // segments of the present key group, handled so far
 
-        float bl[TNN_GMAX_F];
-        int bp[TNN_GMAX_F];
+        // The segments of up to 32 keys (lane: [klo, klo + kn) in key order)
+        // become the present group.
+        auto take_keys = [&](int klo, int kn) {
+            int inc = kn;
 #pragma unroll
-        for (int f = 0; f < TNN_GMAX_F; ++f) {
-            bl[f] = INFINITY;
-            bp[f] = -1;
-        }
-        float wF = INFINITY;
-        int nu = 0;
-
-        // Records of up to 32 segments into segbuf (lane j loads gseg[src_j]);
-        // returns this lane's segment position in the t_A order.
-        auto load_records = [&](int src, bool have) -> int {
-            __syncwarp();
-            int mypos = -1;
-            if (have) {
-                const float4 *r = G.gseg + 4 * (size_t)src;
-                segbuf[4 * lane] = __ldg(r);
-                segbuf[4 * lane + 1] = __ldg(r + 1);
-                segbuf[4 * lane + 2] = __ldg(r + 2);
-                const float4 r3 = __ldg(r + 3);
-                segbuf[4 * lane + 3] = r3;
-                mypos = __float_as_int(r3.z);
-            }
-            __syncwarp();
-            return mypos;
-        };
-        // Seed selection over the cnt staged segments: every lane keeps its F
-        // smallest cylinder bounds.
-        auto seed_pick = [&](int cnt, int mypos) {
-            for (int i = 0; i < cnt; ++i) {
-                const int pos = __shfl_sync(FULLMASK, mypos, i);
-                const float lb = seg_lb(c, s3, segbuf[4 * i], segbuf[4 * i + 1], segbuf[4 * i + 2]);
-                if (active && lb < wF) {
-                    float cur = lb;
-                    int cp = pos;
-#pragma unroll
-                    for (int f = 0; f < TNN_GMAX_F; ++f) {
-                        if (f < F && cur < bl[f]) {
-                            const float tf = bl[f];
-                            bl[f] = cur;
-                            cur = tf;
-                            const int tp = bp[f];
-                            bp[f] = cp;
-                            cp = tp;
-                        }
-                    }
-#pragma unroll
-                    for (int f = 0; f < TNN_GMAX_F; ++f)
-                        if (f == F - 1)
-                            wF = bl[f];
-                }
-            }
-            if (active)
-                st.lb += cnt;
-        };
-
-        // Main mode over the member segments [lo, hi) (key order) of one key:
-        // scan those whose bound allows.
-        auto visit = [&](int lo, int hi) {
-            for (int base = lo; base < hi; base += 32) {
-                const int cnt = min(32, hi - base);
-                const int mypos = load_records(base + lane, lane < cnt);
-                {
-                    bool sd = false;
-                    if (lane < cnt)
-                        for (int u = 0; u < nu; ++u)
-                            sd |= ulist[u] == mypos;
-                    const unsigned smask = __ballot_sync(FULLMASK, sd);
-                    unsigned need = 0;
-                    if (!done) {
-#pragma unroll 4
-                        for (int i = 0; i < cnt; ++i) {
-                            const float lb = seg_lb(c, s3, segbuf[4 * i], segbuf[4 * i + 1],
-                                                    segbuf[4 * i + 2]);
-                            if (lb <= tau)
-                                need |= 1u << i;
-                        }
-                        need &= ~smask;
-                        st.lb += cnt;
-                    }
-                    scan_chunk(__reduce_or_sync(FULLMASK, need), need);
-                }
-            }
-        };
-
-        // ---- seeds: 3 x 3 cells around the warp, two most recent buckets
-        if (bhi >= 0) {
-            const int hx = min(max((int)floorf((0.5f * (bx0 + bx1) - G.x0) * G.inv_cell), 0), G.nx - 1);
-            const int hy = min(max((int)floorf((0.5f * (by0 + by1) - G.y0) * G.inv_cell), 0), G.ny - 1);
-            // lanes 0..9 TNN_SEED_BUCKETS - 1 hold the 3 x 3 cells of the
-            // newest buckets bhi, bhi - 1, ...; the member segments of all
-            // those keys are staged 32 at a time
-            const int bq = bhi - lane / 9, cl = lane % 9;
-            const int cx = hx + cl % 3 - 1, cy = hy + cl / 3 - 1;
-            const bool ok = lane < 9 * TNN_SEED_BUCKETS && bq >= 0 && cx >= 0 && cx < G.nx && cy >= 0 &&
-                            cy < G.ny;
-            int lo = 0, n = 0;
-            if (ok) {
-                const int key = bq * G.ncell + cy * G.nx + cx;
-                lo = __ldg(goff + key);
-                n = __ldg(goff + key + 1) - lo;
-            }
-            int inc = n;
-#pragma unroll
-            for (int o = 1; o < 32; o <<= 1) {
-                const int v = __shfl_up_sync(FULLMASK, inc, o);
-                if (lane >= o)
+            for (int s = 1; s < 32; s <<= 1) {
+                const int v = __shfl_up_sync(FULLMASK, inc, s);
+                if (lane >= s)
                     inc += v;
             }
-            const int total = __shfl_sync(FULLMASK, inc, 31);
-            const int rel = lo - (inc - n); // record index = rel_j + position in the batch
-            for (int base = 0; base < total; base += 32) {
-                const int t = base + lane;
-                int src = 0;
-#pragma unroll
-                for (int j = 0; j < 9 * TNN_SEED_BUCKETS; ++j) {
-                    const int ij = __shfl_sync(FULLMASK, inc, j);
-                    const int rj = __shfl_sync(FULLMASK, rel, j);
-                    if (src == 0 && t < ij)
-                        src = rj + t + 1; // +1 keeps 0 as "unset"
-                }
-                const int cnt = min(32, total - base);
-                const int mypos = load_records(src - 1, lane < cnt);
-                seed_pick(cnt, mypos);
-            }
-        }
-
-        // ---- scan the union of the seeds (highest position first)
+            __syncwarp();
+            S.kend[lane] = inc;
+            S.krel[lane] = klo - (inc - kn); // record = krel[j] + position in the group
+            total = __shfl_sync(FULLMASK, inc, 31);
+            pos = 0;
+            __syncwarp();
+        };
         {
-            auto next_seed = [&]() {
-                int mm = -1;
-#pragma unroll
-                for (int f = 0; f < TNN_GMAX_F; ++f)
-                    mm = max(mm, bp[f]);
-                return __reduce_max_sync(FULLMASK, mm);
-            };
-            int pos = next_seed();
-            SegPoints cur, nxt;
-            if (pos >= 0)
-                seg_points_load(cur, pts, __ldg(seg + 4 * (size_t)pos + 3), lane);
-            while (pos >= 0 && nu < TNN_UCAP) {
-#pragma unroll
-                for (int f = 0; f < TNN_GMAX_F; ++f)
-                    if (bp[f] == pos)
-                        bp[f] = -1;
-                if (lane == 0)
-                    ulist[nu] = pos;
-                ++nu;
-                const int npos = nu < TNN_UCAP ? next_seed() : -1;
-                if (npos >= 0)
-                    seg_points_load(nxt, pts, __ldg(seg + 4 * (size_t)npos + 3), lane);
-                __syncwarp();
-                seg_points_store(cur, pbuf, lane);
-                __syncwarp();
-                scan_pbuf(cur.first, cur.cnt, active);
-                cur = nxt;
-                pos = npos;
+            const int bq = bhi - (seed_cell >> 4);
+            const int cx = hx + (seed_cell & 3) - 1, cy = hy + ((seed_cell >> 2) & 3) - 1;
+            int klo = 0, kn = 0;
+            if (lane < 9 * TNN_SEED_BUCKETS && bq >= 0 && cx >= 0 && cx < G.nx && cy >= 0 && cy < G.ny) {
+                const int key = bq * G.ncell + cy * G.nx + cx;
+                klo = __ldg(G.off + key);
+                kn = __ldg(G.off + key + 1) - klo;
             }
+            take_keys(klo, kn);
         }
-        __syncwarp();
 
-        // ---- a lane whose key is still above the deferral threshold (far
-        // neighbours, or a list not yet full) would make the whole tile visit
-        // a wide region: it is handed to the warp-per-query kernel instead
-        const bool deferred = active && !(tau <= W->tau_defer);
+        for (;;) {
+            const int cnt = min(32, total - pos);
+            bool flush = false;
+            if (cnt <= 0) {
+                // the group is done: next one, or first what is gathered
+                if (near_phase) {
+                    if (fill > 0) {
+                        flush = true;
+                    } else {
+                        // a lane whose key is still above the deferral
+                        // threshold (far neighbours, or a list not yet full)
+                        // would make the whole tile visit a wide region
+                        near_phase = false;
+                        deferred = act && !(tau <= tau_defer);
+                        continue;
+                    }
+                } else if (t0 >= ncells) {
+                    if (fill > 0) {
+                        flush = true;
+                    } else {
+                        if (--b < 0)
+                            break;
+                        const bool done =
+                            !act || deferred || !(time_lb(c, s3, __ldg(G.bpm + b)) <= tau);
+                        if (__all_sync(FULLMASK, done))
+                            break;
+                        lim = done ? -1.0f : tau;
+                        const float tmx = warp_maxf(done ? 0.0f : tau);
+                        int cx1 = G.nx - 1, cy1 = G.ny - 1;
+                        cx0 = 0;
+                        cy0 = 0;
+                        if (tmx < INFINITY) {
+                            // any key outside this reach has a bound above every key
+                            const float R = sqrtf(tmx) * (1.0f + 0x1p-18f) + ext_max +
+                                            warp_maxf(act ? c.delta : 0.0f);
+                            reach_cells(bx0, bx1, R, G.x0, G.inv_cell, G.nx, cx0, cx1);
+                            reach_cells(by0, by1, R, G.y0, G.inv_cell, G.ny, cy0, cy1);
+                        }
+                        wx = cx1 - cx0 + 1;
+                        ncells = wx * (cy1 - cy0 + 1);
+                        t0 = 0;
+                        continue;
+                    }
+                } else {
+                    // up to 32 cells of bucket b: the keys some lane needs
+                    const int t = t0 + lane;
+                    t0 += 32;
+                    int klo = 0, kn = 0, cx = 0, cy = 0;
+                    float ex = 0.f, tk = 0.f;
+                    if (t < ncells) {
+                        cx = cx0 + t % wx;
+                        cy = cy0 + t / wx;
+                        const bool staged = b > bhi - TNN_SEED_BUCKETS && abs(cx - hx) <= 1 && abs(cy - hy) <= 1;
+                        if (!staged) {
+                            const int4 kr = __ldg(G.krec + (b * G.ncell + cy * G.nx + cx));
+                            klo = kr.x;
+                            kn = kr.y - kr.x;
+                            ex = __int_as_float(kr.z);
+                            tk = __int_as_float(kr.w);
+                        }
+                    }
+                    unsigned m = __ballot_sync(FULLMASK, kn > 0), want = 0;
+                    while (m) {
+                        const int j = __ffs(m) - 1;
+                        m &= m - 1;
+                        const int jx = __shfl_sync(FULLMASK, cx, j), jy = __shfl_sync(FULLMASK, cy, j);
+                        const float jex = __shfl_sync(FULLMASK, ex, j), jtk = __shfl_sync(FULLMASK, tk, j);
+                        const float rx0 = G.x0 + (float)jx * G.cell, ry0 = G.y0 + (float)jy * G.cell;
+                        if (__any_sync(FULLMASK, cell_lb(c, s3, rx0, rx0 + G.cell, ry0, ry0 + G.cell, jex,
+                                                         jtk) <= lim))
+                            want |= 1u << j;
+                    }
+                    if (want)
+                        take_keys(klo, (want >> lane) & 1u ? kn : 0);
+                    continue;
+                }
+            }
+
+            // ---- the next (up to 32) segments of the group: bounds of every lane
+            int sfirst = 0, scnt = 0;
+            unsigned score = TG_EMPTY; // lane j: smallest bound of segment j over the lanes
+            if (cnt > 0) {
+                __syncwarp();
+                if (lane < cnt) {
+                    const int g = pos + lane;
+                    int lo = 0, hi = 31; // smallest key with kend > g
+#pragma unroll
+                    for (int s = 0; s < 5; ++s) {
+                        const int mid = (lo + hi) >> 1;
+                        if (S.kend[mid] > g)
+                            hi = mid;
+                        else
+                            lo = mid + 1;
+                    }
+                    const float4 *r = G.gseg + 4 * (size_t)(S.krel[lo] + g);
+                    S.seg[lane][0] = __ldg(r);
+                    S.seg[lane][1] = __ldg(r + 1);
+                    S.seg[lane][2] = __ldg(r + 2);
+                    const float4 r3 = __ldg(r + 3);
+                    sfirst = __float_as_int(r3.x);
+                    scnt = __float_as_int(r3.y);
+                }
+                pos += cnt;
+                __syncwarp();
+                // two per step (their chains overlap); an odd count's last
+                // partner is a stale record whose bound is not used
+#pragma unroll 1
+                for (int i = 0; i < cnt; i += 2) {
+#pragma unroll
+                    for (int u = 0; u < 2; ++u) {
+                        const float lb = seg_lb(c, s3, S.seg[i + u][0], S.seg[i + u][1], S.seg[i + u][2]);
+                        // the upper half of a non-negative float is a lower bound of it
+                        const unsigned h = __float_as_uint(lb) >> 16;
+                        S.lb[i + u][lane] = (uint16_t)h;
+                        const unsigned m = __reduce_min_sync(FULLMASK, lb <= lim ? h : 0xffffu);
+                        if (lane == i + u && lane < cnt && m != 0xffffu)
+                            score = (m << 5) | (unsigned)lane;
+                    }
+                }
+                if (act)
+                    n_lb += cnt;
+                __syncwarp();
+            }
+
+            // ---- their points, 32 at a time, nearest segments first
+            int lf = 0, lc = 0; // points left of the segment taken last
+            for (;;) {
+                while (fill < 32) {
+                    if (lc == 0) {
+                        const unsigned best = __reduce_min_sync(FULLMASK, score);
+                        if (best == TG_EMPTY)
+                            break;
+                        const int j = best & 31u;
+                        if (lane == j)
+                            score = TG_EMPTY;
+                        if (!__any_sync(FULLMASK, __uint_as_float((unsigned)S.lb[j][lane] << 16) <= lim))
+                            continue;
+                        lf = __shfl_sync(FULLMASK, sfirst, j);
+                        lc = __shfl_sync(FULLMASK, scnt, j);
+                        n_segs += act;
+                    }
+                    const int take = min(lc, 32 - fill);
+                    if (lane >= fill && lane < fill + take)
+                        myidx = lf + lc - 1 - (lane - fill); // newest member first
+                    lc -= take;
+                    fill += take;
+                }
+                if (fill == 0 || (fill < 32 && !flush))
+                    break;
+                if (base > TG_SLOTS - 32) {
+                    // renumber the slots that some list still holds
+                    __syncwarp();
+                    S.used[lane] = 0;
+                    __syncwarp();
+                    unsigned t[NL + TG_EXTRA]; // in local memory: this is rare
+#pragma unroll
+                    for (int i = 0; i < NL; ++i)
+                        t[i] = a[i];
+#pragma unroll
+                    for (int i = 0; i < TG_EXTRA; ++i)
+                        t[NL + i] = o[i];
+#pragma unroll 1
+                    for (int i = 0; i < NL + TG_EXTRA; ++i)
+                        if (t[i] != TG_EMPTY)
+                            atomicOr(&S.used[(t[i] & TG_SMASK) >> 5], 1u << (t[i] & 31u));
+                    __syncwarp();
+                    const unsigned u = S.used[lane];
+                    int inc = __popc(u);
+#pragma unroll
+                    for (int s = 1; s < 32; s <<= 1) {
+                        const int v = __shfl_up_sync(FULLMASK, inc, s);
+                        if (lane >= s)
+                            inc += v;
+                    }
+                    S.pre[lane] = inc - __popc(u);
+                    base = __shfl_sync(FULLMASK, inc, 31);
+                    __syncwarp();
+#pragma unroll 1
+                    for (int i = 0; i < NL + TG_EXTRA; ++i) {
+                        const unsigned v = t[i], s = v & TG_SMASK;
+                        if (v != TG_EMPTY)
+                            t[i] = (v & ~TG_SMASK) |
+                                   (unsigned)(S.pre[s >> 5] + __popc(S.used[s >> 5] & ((1u << (s & 31u)) - 1u)));
+                    }
+#pragma unroll
+                    for (int i = 0; i < NL; ++i)
+                        a[i] = t[i];
+#pragma unroll
+                    for (int i = 0; i < TG_EXTRA; ++i)
+                        o[i] = t[NL + i];
+#pragma unroll 1
+                    for (int w = 0; w < 32; ++w) {
+                        const unsigned uw = S.used[w];
+                        const int id = S.slot[w * 32 + lane];
+                        __syncwarp();
+                        if ((uw >> lane) & 1u)
+                            S.slot[S.pre[w] + __popc(uw & ((1u << lane) - 1u))] = id;
+                        __syncwarp();
+                    }
+                    if (base > TG_SLOTS - 32) {
+                        given_up = true;
+                        break;
+                    }
+                }
+                __syncwarp();
+                {
+                    const bool have = lane < fill;
+                    float4 p = make_float4(0.f, 0.f, 0.f, INFINITY); // never causal
+                    if (have) {
+                        p = __ldg(pts + myidx);
+                        S.slot[base + lane] = myidx;
+                    }
+                    S.pts[lane] = p;
+                }
+                __syncwarp();
+                if (act) {
+                    n_pairs += fill;
+                    if (L.dbg_seen)
+#pragma unroll 1
+                        for (int i = 0; i < fill; ++i)
+                            dbg_mark_seen(L, qrow, S.slot[base + i], 1);
+                }
+                unsigned kept = 0;
+#pragma unroll 1
+                for (int s = 0; s < fill; s += NB) {
+                    unsigned v[NB], mine = 0;
+#pragma unroll
+                    for (int i = 0; i < NB; ++i) {
+                        const float4 p = S.pts[s + i];
+                        const float d = dist32(c, s0, s1, s2, s3, p);
+                        const bool in = p.w < c.T32 && d <= tau;
+                        v[i] = in ? tg_key(d, (unsigned)(base + s + i)) : TG_EMPTY;
+                        mine |= in ? 1u << i : 0u;
+                    }
+                    unsigned any = __reduce_or_sync(FULLMASK, mine);
+                    if (!any)
+                        continue;
+                    kept = 1;
+                    if (__popc(any) <= TG_INSERT) {
+#pragma unroll 1
+                        while (any) {
+                            const int i = __ffs(any) - 1;
+                            any &= any - 1;
+                            const float4 p = S.pts[s + i];
+                            const float d = dist32(c, s0, s1, s2, s3, p);
+                            const unsigned key = (mine >> i) & 1u ? tg_key(d, (unsigned)(base + s + i)) : TG_EMPTY;
+                            tg_insert<NL>(a, o, key);
+                        }
+                    } else {
+                        tg_sort<NB>(v);
+                        tg_merge<NL, NB>(a, o, v);
+                    }
+                    if (a[NL - 1] < TG_INF)
+                        tau = fmaf(tg_upper(a[NL - 1]), 0x1p-12f, tg_upper(a[NL - 1])) + 0x1p-98f;
+                    lim = fminf(lim, tau);
+                }
+                base += kept ? 32 : 0;
+                fill = 0;
+            }
+            if (given_up)
+                break;
+        }
+
+        // ---- hand-over of deferred lanes, with a pruning key when the list
+        // is as long as the warp-per-query kernel's
+        if (given_up)
+            deferred = act;
         if (deferred) {
+            const float hand = !given_up && W->L <= k + TG_EXTRA && o[TG_EXTRA - 1] != TG_EMPTY
+                                   ? tg_upper(o[TG_EXTRA - 1])
+                                   : INFINITY;
             const unsigned slot = atomicAdd(&L.scr->n_fallback, 1u);
             if (slot < (unsigned long long)L.fb_cap) {
                 L.fb_list[slot] = make_int2(window_id(L, W), (int)qrow);
-                L.fb_tau[slot] = tau;
+                L.fb_tau[slot] = hand;
             } else
                 atomicOr(&L.scr->status, 1u);
         }
 
-        // ---- main: buckets backwards, cells within reach, keys by bound
-        for (int b = bhi; b >= 0; --b) {
-            done = !active || deferred || !(time_lb(c, s3, __ldg(G.bpm + b)) <= tau);
-            if (__all_sync(FULLMASK, done))
-                break;
-            const float tmx = warp_maxf(done ? 0.0f : tau);
-            int cx0 = 0, cx1 = G.nx - 1, cy0 = 0, cy1 = G.ny - 1;
-            if (tmx < INFINITY) {
-                // any key outside this reach has a bound above every key
-                const float R = sqrtf(tmx) * (1.0f + 0x1p-18f) + ext_max + dmax;
-                reach_cells(bx0, bx1, R, G.x0, G.inv_cell, G.nx, cx0, cx1);
-                reach_cells(by0, by1, R, G.y0, G.inv_cell, G.ny, cy0, cy1);
+        // ---- settle: exact keys of the k + TG_EXTRA smallest.  Every point
+        // outside them lies at or above `bound`.
+        const bool settle = act && !deferred;
+        float bound = INFINITY;
+        bool ok = a[NL - 1] < TG_INF || a[NL - 1] == TG_EMPTY; // else distances overflowed
+        if (a[NL - 1] < TG_INF)
+            bound = o[TG_EXTRA - 1] != TG_EMPTY ? fminf(tg_lower(o[TG_EXTRA - 1]), tau) : tau;
+        __syncwarp();
+#pragma unroll
+        for (int i = 0; i < NL; ++i)
+            S.raw[i][lane] = a[i];
+#pragma unroll
+        for (int i = 0; i < TG_EXTRA; ++i)
+            S.raw[NL + i][lane] = o[i];
+        // slots to point indices (each lane its own column)
+        const int z = NL - k; // rows below hold the leading zeros
+#pragma unroll 4
+        for (int e = z; e < NL + TG_EXTRA; ++e) {
+            const unsigned v = S.raw[e][lane];
+            S.raw[e][lane] = settle && v != TG_EMPTY ? (unsigned)S.slot[v & TG_SMASK] : TG_EMPTY;
+        }
+        {
+            // Exact keys, from the last row down: 64-bit row e covers 32-bit
+            // rows 2 e and 2 e + 1, which every lane has read by then.
+            bool slow = (W->flags & TNN_FLAG_EXACT_D2) != 0;
+            unsigned long long next = SENT;
+#pragma unroll 1
+            for (int e = NL + TG_EXTRA - 1; e >= z; e -= 2) {
+                // two rows per step; row z - 1 is a zero row or absent (e0 = z)
+                const int e1 = max(e - 1, z);
+                const unsigned i0 = S.raw[e][lane], i1 = S.raw[e1][lane];
+                __syncwarp();
+                const float4 p0 = __ldg(pts + (i0 != TG_EMPTY ? i0 : 0u));
+                const float4 p1 = __ldg(pts + (i1 != TG_EMPTY ? i1 : 0u));
+                const unsigned long long k0 =
+                    i0 != TG_EMPTY ? pack_key(dist32(c, s0, s1, s2, s3, p0), (int)i0) : SENT;
+                const unsigned long long k1 =
+                    i1 != TG_EMPTY ? pack_key(dist32(c, s0, s1, s2, s3, p1), (int)i1) : SENT;
+                *tg_entry(Kw, e, lane) = k0;
+                *tg_entry(Kw, e1, lane) = k1;
+                slow |= next < k0 || (e1 < e && k0 < k1);
+                const float d0 = key_d(k0), d1 = key_d(k1);
+                if (e < NL && next != SENT)
+                    slow |= key_d(next) <= fmaf(d0, 0x1p-17f, d0) + 0x1p-100f;
+                if (e1 < NL && e1 < e && k0 != SENT)
+                    slow |= d0 <= fmaf(d1, 0x1p-17f, d1) + 0x1p-100f;
+                if (e1 == NL - 1 || e == NL - 1) {
+                    const float dk = e == NL - 1 ? d0 : d1;
+                    if (dk < INFINITY)
+                        slow |= bound <= fmaf(dk, 0x1p-17f, dk) + 0x1p-100f;
+                }
+                next = k1;
             }
-            const int kb = b * G.ncell;
-            for (int cy = cy0; cy <= cy1; ++cy) {
-                const float ry0 = G.y0 + (float)cy * G.cell, ry1 = ry0 + G.cell;
-                for (int cxb = cx0; cxb <= cx1; cxb += 32) {
-                    const int cx = cxb + lane;
-                    int lo = 0, hi = 0;
-                    float ex = 0.f, tk = 0.f;
-                    if (cx <= cx1) {
-                        const int key = kb + cy * G.nx + cx;
-                        const int4 kr = __ldg(G.krec + key);
-                        lo = kr.x;
-                        hi = kr.y;
-                        ex = __int_as_float(kr.z);
-                        tk = __int_as_float(kr.w);
+            if (settle && ok && slow) {
+                const unsigned r = tg_settle(W, q, Kw, lane, z, k + TG_EXTRA, bound);
+                ok = r & 1u;
+                n_fp += r >> 1;
+            }
+        }
+        if (settle && !ok) {
+            const unsigned slot = atomicAdd(&L.scr->n_fallback, 1u);
+            if (slot < (unsigned long long)L.fb_cap) // unsettled: -1 - window
+                L.fb_list[slot] = make_int2(-1 - window_id(L, W), (int)qrow);
+            else
+                atomicOr(&L.scr->status, 1u);
+        }
+        // ---- write the settled rows: consecutive words across the lanes (a
+        // store per lane of its own row would touch 32 lines), to the mapped
+        // host lists when the call has them
+        const unsigned wmask = __ballot_sync(FULLMASK, settle && ok);
+        if (wmask) {
+            const int64_t off0 = __shfl_sync(FULLMASK, qrow, 0) * k;
+            int32_t *oi = (L.mirror_idx ? L.mirror_idx : W->out_idx) + off0;
+            float *od = (L.mirror_d2 ? L.mirror_d2 : W->out_d2) + off0;
+            if (((k & 3) | (int)(((uintptr_t)oi | (uintptr_t)od) & 15)) == 0) {
+                const int kq = k >> 2;
+                int row = lane / kq, e = lane % kq;
+                const int drow = 32 / kq, de = 32 % kq;
+                while (row < 32) {
+                    if ((wmask >> row) & 1u) {
+                        int ri[4];
+                        float rd[4];
+#pragma unroll
+                        for (int u = 0; u < 4; ++u) {
+                            const unsigned long long key = *tg_entry(Kw, z + 4 * e + u, row);
+                            ri[u] = key == SENT ? -1 : key_i(key);
+                            rd[u] = key == SENT ? INFINITY : key_d(key);
+                        }
+                        const int64_t w = (int64_t)row * kq + e;
+                        ((int4 *)oi)[w] = make_int4(ri[0], ri[1], ri[2], ri[3]);
+                        ((float4 *)od)[w] = make_float4(rd[0], rd[1], rd[2], rd[3]);
                     }
-                    unsigned m = __ballot_sync(FULLMASK, hi > lo);
-                    while (m) {
-                        const int j = __ffs(m) - 1;
-                        m &= m - 1;
-                        const int jlo = __shfl_sync(FULLMASK, lo, j);
-                        const int jhi = __shfl_sync(FULLMASK, hi, j);
-                        const float jex = __shfl_sync(FULLMASK, ex, j);
-                        const float jtk = __shfl_sync(FULLMASK, tk, j);
-                        const float rx0 = G.x0 + (float)(cxb + j) * G.cell, rx1 = rx0 + G.cell;
-                        const bool want = !done && cell_lb(c, s3, rx0, rx1, ry0, ry1, jex, jtk) <= tau;
-                        if (__any_sync(FULLMASK, want))
-                            visit(jlo, jhi);
+                    row += drow;
+                    e += de;
+                    if (e >= kq) {
+                        e -= kq;
+                        ++row;
+                    }
+                }
+            } else {
+                int row = lane / k, e = lane % k;
+                const int drow = 32 / k, de = 32 % k;
+                while (row < 32) {
+                    if ((wmask >> row) & 1u) {
+                        const unsigned long long key = *tg_entry(Kw, z + e, row);
+                        oi[(int64_t)row * k + e] = key == SENT ? -1 : key_i(key);
+                        od[(int64_t)row * k + e] = key == SENT ? INFINITY : key_d(key);
+                    }
+                    row += drow;
+                    e += de;
+                    if (e >= k) {
+                        e -= k;
+                        ++row;
                     }
                 }
             }
         }
-
-        // ---- settle and write
         __syncwarp();
-        if (active)
-            st.q++;
-        if (active && !deferred) {
-            if (!finalize_query(W, q, K, Lw, cl_d, cl_i, qrow, st)) {
-                const unsigned slot = atomicAdd(&L.scr->n_fallback, 1u);
-                if (slot < (unsigned long long)L.fb_cap) // unsettled: -1 - window
-                    L.fb_list[slot] = make_int2(-1 - window_id(L, W), (int)qrow);
-                else
-                    atomicOr(&L.scr->status, 1u);
-            }
+        }
+        if ((lone >> lane) & 1u) {
+            const unsigned slot = atomicAdd(&L.scr->n_fallback, 1u);
+            if (slot < (unsigned long long)L.fb_cap) {
+                L.fb_list[slot] = make_int2(window_id(L, W), (int)qrow);
+                L.fb_tau[slot] = INFINITY;
+            } else
+                atomicOr(&L.scr->status, 1u);
         }
         __syncwarp();
-        if (MIRROR) {
-            const int cnt = __popc(__ballot_sync(FULLMASK, active));
-            if (cnt > 0)
-                mirror_tile(L, W, __shfl_sync(FULLMASK, qrow, 0), cnt, lane);
-        }
     }
+    LaneStats st = {n_q, n_lb, n_pairs, n_segs, n_fp};
     flush_stats(L.scr, st);
 }

@@ -148,8 +148,12 @@ struct KnnWin {
 
 #define TNN_MAX_WINDOWS_PARAM 1
 
+// Tile kernels by list length: k <= 8, 16, 32, 64.
+#define TNN_CLASSES 4
+inline int tnn_k_class(int k) { return k <= 8 ? 0 : k <= 16 ? 1 : k <= 32 ? 2 : 3; }
+
 struct KnnScratch {
-    unsigned long long tile_counter;
+    unsigned long long tile_counter[TNN_CLASSES]; // one queue per tile kernel of the launch
     unsigned long long stats[8]; // queries, lb, pairs, segs, fp64, fallback
     unsigned int n_fallback;  // queries handed to the FP32 warp scan
     unsigned int status;
@@ -167,6 +171,9 @@ struct KnnLaunch {
     int32_t kseg_max;     // largest segment length over the windows
     int32_t pad_;
     int64_t total_tiles;
+    int64_t tile_lo; // grid order: this launch's tiles [tile_lo, total_tiles)
+    int32_t queue;   // and their queue (KnnScratch::tile_counter)
+    int32_t pad3_;
     KnnScratch *scr;
     int2 *fb_list;        // (window, query) for the FP32 warp scan
     int2 *fb_list3;       // (window, query) for the exact FP64 warp scan
@@ -181,10 +188,10 @@ struct KnnLaunch {
     uint32_t *dbg_seen;   // tests only (tnn_knn_trace), else NULL: bit j of
                           // row q = point j's distance to query q was taken
     int64_t dbg_words;    // 32-bit words per row of dbg_seen
-    // When set (one window), a grid or sweep tile kernel copies the rows of
-    // each finished tile, handed-over rows included as they stand, from
-    // out_idx / out_d2 to the same rows of these: mapped page-locked host
-    // lists, written with coalesced stores.
+    // When set (one window): mapped page-locked host lists.  The grid tile
+    // kernel writes the rows it settles there instead of out_idx / out_d2;
+    // the sweep tile kernel copies each finished tile's rows there,
+    // handed-over rows included as they stand.
     int32_t *mirror_idx;
     float *mirror_d2;
     int32_t mirror_vec; // k % 4 == 0 and all four lists 16-byte aligned

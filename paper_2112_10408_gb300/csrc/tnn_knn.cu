@@ -9,16 +9,16 @@
 // left; a finished warp immediately takes new work, which is the GPU form of
 // Algorithm 2's "put completed lines at the end of the batch".
 //
-// TNN per query (lane):
-//   1. seed: among the W0 most recent causally valid segments, the F with
-//      the smallest lower bound are scanned first (Algorithm 2 fetches F
-//      segments at a time, nearest first);
-//   2. sweep: segments are visited from the most recent t_A backwards in
-//      chunks of 32; a segment's points are scanned only if its lower bound
-//      does not exceed the current k-th candidate (exclusion criterion of
-//      Sec. 3.4); the sweep stops once the time-only bound of every remaining
-//      segment, taken from the running maximum of t_B, exceeds it (the stop
-//      rule of Algorithm 2 with the temporal part of the bound).
+// TNN per query (lane; the grid order of tnn_grid.cuh is the default, the
+// sweep of tnn_search.cuh the alternative):
+//   1. nearest first: the segments around the query of smallest lower bound
+//      are scanned before any other (Algorithm 2 fetches F segments at a
+//      time, nearest first);
+//   2. then backwards in time: a segment's points are scanned only if its
+//      lower bound does not exceed the current k-th candidate (exclusion
+//      criterion of Sec. 3.4), until the time-only bound of every remaining
+//      segment, from the running maximum of t_B, exceeds it (the stop rule of
+//      Algorithm 2 with the temporal part of the bound).
 //   3. settle: rank ties the FP32 values cannot separate are re-ranked in
 //      FP64 (the canonical formula of the oracle), output sorted by
 //      (d2, index).
@@ -40,8 +40,8 @@
 //       t_q - t_j for a valid point (t_j <= t_B, t_j < T32);
 //     - the sum is multiplied by (1 - 2^-19), which covers the roundings of
 //       the bound itself and the 8u of d32.
-//   A candidate is inserted iff its key (d32, index) is below the largest
-//   key kept, so a segment whose bound exceeds that key cannot contribute.
+//   A candidate enters a list iff its distance does not exceed the list's
+//   pruning key, so a segment whose bound exceeds that key cannot contribute.
 //   Settlement: if d32(b) > d32(a)(1 + 2^-17) + 2^-100 then d2(b) > d2(a);
 //   maximal chains of keys closer than that are re-ranked in FP64.  When the
 //   chain holding rank k reaches the last kept slot of a full candidate
@@ -110,6 +110,20 @@ static cudaError_t prof_begin(cudaStream_t st, ProfEv *pr)
     return cudaEventRecord(pr->e[0], st);
 }
 
+typedef void (*TileKernel)(const KnnLaunch);
+static TileKernel grid_kernel(int cls)
+{
+    static const TileKernel t[TNN_CLASSES] = {k_tnn_grid_search<8>, k_tnn_grid_search<16>,
+                                              k_tnn_grid_search<32>, k_tnn_grid_search<64>};
+    return t[cls];
+}
+static size_t grid_smem(int cls) // per CTA
+{
+    static const size_t t[TNN_CLASSES] = {tg_smem_per_warp<8>(), tg_smem_per_warp<16>(),
+                                          tg_smem_per_warp<32>(), tg_smem_per_warp<64>()};
+    return t[cls] * TNN_WARPS_PER_CTA;
+}
+
 static tnn_status device_setup()
 {
     int dev = 0;
@@ -136,8 +150,8 @@ static tnn_status device_setup()
         const int maxs = 227 * 1024;
         TNN_CUDA_TRY(cudaFuncSetAttribute(k_tnn_search<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, maxs));
         TNN_CUDA_TRY(cudaFuncSetAttribute(k_tnn_search<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, maxs));
-        TNN_CUDA_TRY(cudaFuncSetAttribute(k_tnn_grid_search<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, maxs));
-        TNN_CUDA_TRY(cudaFuncSetAttribute(k_tnn_grid_search<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, maxs));
+        for (int c = 0; c < TNN_CLASSES; ++c)
+            TNN_CUDA_TRY(cudaFuncSetAttribute(grid_kernel(c), cudaFuncAttributeMaxDynamicSharedMemorySize, maxs));
         TNN_CUDA_TRY(cudaFuncSetAttribute(k_linear_search, cudaFuncAttributeMaxDynamicSharedMemorySize, maxs));
         TNN_CUDA_TRY(cudaFuncSetAttribute(k_linear_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, maxs));
         TNN_CUDA_TRY(cudaFuncSetAttribute(k_tnn_warp, cudaFuncAttributeMaxDynamicSharedMemorySize, maxs));
@@ -281,15 +295,38 @@ static tnn_status finish_search(const KnnLaunch &L, cudaStream_t st, bool prof, 
     return TNN_OK;
 }
 
-// The grid- or sweep-order tile kernel.
+// The grid-order tile kernel of class `cls` over tiles [L.tile_lo,
+// L.total_tiles), all of windows whose k is in that class.
+static tnn_status launch_grid_tiles(const KnnLaunch &L, int cls, cudaStream_t st)
+{
+    const TileKernel kern = grid_kernel(cls);
+    const size_t smem = grid_smem(cls);
+    int nb = 0;
+    TNN_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, kern, TNN_WARPS_PER_CTA * 32, smem));
+    if (nb < 1) {
+        tnn_set_error("search kernel does not fit on an SM (%zu B shared memory)", smem);
+        return TNN_ERR_UNSUPPORTED;
+    }
+    const long long tiles = std::max<long long>(L.total_tiles - L.tile_lo, 0);
+    const long long need = (tiles + TNN_WARPS_PER_CTA - 1) / TNN_WARPS_PER_CTA;
+    const long long grid = std::max<long long>(std::min<long long>(need, (long long)nb * g_num_sms), 1);
+    kern<<<(unsigned)grid, TNN_WARPS_PER_CTA * 32, smem, st>>>(L);
+    TNN_CUDA_TRY(cudaGetLastError());
+    return TNN_OK;
+}
+
+// The grid- or sweep-order tile kernel of a single window.
 static tnn_status launch_tiles(const KnnLaunch &L, cudaStream_t st)
 {
-    const bool sweep = (L.w0.flags & TNN_FLAG_SWEEP) != 0;
-    const size_t smem = smem_per_warp(L.L_max, L.kseg_max, sweep ? SMEM_SWEEP : SMEM_GRID) *
-                        TNN_WARPS_PER_CTA;
+    if ((L.w0.flags & TNN_FLAG_SWEEP) == 0) {
+        KnnLaunch G = L;
+        G.tile_lo = 0;
+        G.queue = 0;
+        return launch_grid_tiles(G, tnn_k_class(L.w0.k), st);
+    }
+    const size_t smem = smem_per_warp(L.L_max, L.kseg_max, SMEM_SWEEP) * TNN_WARPS_PER_CTA;
     const bool mirror = L.mirror_idx != nullptr;
-    const void *kern = sweep ? (mirror ? (const void *)k_tnn_search<true> : (const void *)k_tnn_search<false>)
-                             : (mirror ? (const void *)k_tnn_grid_search<true> : (const void *)k_tnn_grid_search<false>);
+    const TileKernel kern = mirror ? k_tnn_search<true> : k_tnn_search<false>;
     int nb = 0;
     TNN_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, kern, TNN_WARPS_PER_CTA * 32, smem));
     if (nb < 1) {
@@ -297,17 +334,8 @@ static tnn_status launch_tiles(const KnnLaunch &L, cudaStream_t st)
         return TNN_ERR_UNSUPPORTED;
     }
     const long long need = (L.total_tiles + TNN_WARPS_PER_CTA - 1) / TNN_WARPS_PER_CTA;
-    long long grid = std::min<long long>(need, (long long)nb * g_num_sms);
-    if (grid < 1)
-        grid = 1;
-    if (sweep && mirror)
-        k_tnn_search<true><<<(unsigned)grid, TNN_WARPS_PER_CTA * 32, smem, st>>>(L);
-    else if (sweep)
-        k_tnn_search<false><<<(unsigned)grid, TNN_WARPS_PER_CTA * 32, smem, st>>>(L);
-    else if (mirror)
-        k_tnn_grid_search<true><<<(unsigned)grid, TNN_WARPS_PER_CTA * 32, smem, st>>>(L);
-    else
-        k_tnn_grid_search<false><<<(unsigned)grid, TNN_WARPS_PER_CTA * 32, smem, st>>>(L);
+    const long long grid = std::max<long long>(std::min<long long>(need, (long long)nb * g_num_sms), 1);
+    kern<<<(unsigned)grid, TNN_WARPS_PER_CTA * 32, smem, st>>>(L);
     TNN_CUDA_TRY(cudaGetLastError());
     return TNN_OK;
 }
@@ -669,6 +697,54 @@ struct tnn_batch {
     cudaGraphExec_t exec;
 };
 
+// The tile kernels of the classes present as parallel branches of the graph
+// being captured on `cs` (a class's tail is filled by the next one's tiles),
+// then the per-query kernels over what they handed over.
+static tnn_status capture_grid_classes(const KnnLaunch &L, const long long *cls_tile, cudaStream_t cs)
+{
+    cudaStream_t side[TNN_CLASSES] = {nullptr};
+    cudaEvent_t fork = nullptr, join[TNN_CLASSES] = {nullptr};
+    cudaError_t e = cudaEventCreateWithFlags(&fork, cudaEventDisableTiming);
+    if (e == cudaSuccess)
+        e = cudaEventRecord(fork, cs);
+    tnn_status s = TNN_OK;
+    // the longest lists first: their tiles cost most
+    for (int c = TNN_CLASSES - 1; c >= 0 && s == TNN_OK && e == cudaSuccess; --c) {
+        if (cls_tile[c + 1] == cls_tile[c])
+            continue;
+        e = cudaStreamCreateWithFlags(&side[c], cudaStreamNonBlocking);
+        if (e == cudaSuccess)
+            e = cudaEventCreateWithFlags(&join[c], cudaEventDisableTiming);
+        if (e == cudaSuccess)
+            e = cudaStreamWaitEvent(side[c], fork, 0);
+        if (e != cudaSuccess)
+            break;
+        KnnLaunch G = L;
+        G.tile_lo = cls_tile[c];
+        G.total_tiles = cls_tile[c + 1];
+        G.queue = c;
+        s = launch_grid_tiles(G, c, side[c]);
+        // joined even after a failure, so that the capture can end
+        e = cudaEventRecord(join[c], side[c]);
+        if (e == cudaSuccess)
+            e = cudaStreamWaitEvent(cs, join[c], 0);
+    }
+    if (s == TNN_OK && e == cudaSuccess) {
+        ProfEv pr;
+        s = finish_search(L, cs, false, pr);
+    }
+    for (int c = 0; c < TNN_CLASSES; ++c) {
+        if (side[c])
+            cudaStreamDestroy(side[c]);
+        if (join[c])
+            cudaEventDestroy(join[c]);
+    }
+    if (fork)
+        cudaEventDestroy(fork);
+    TNN_CUDA_TRY(e);
+    return s;
+}
+
 extern "C" void tnn_batch_destroy(tnn_batch *b)
 {
     if (!b)
@@ -699,9 +775,19 @@ extern "C" tnn_status tnn_batch_create(const tnn_index *const *indexes,
     std::vector<KnnWin> wins(n_windows);
     long long tiles = 0, fb = 0;
     int L_max = 0, kseg = 0;
-    for (int w = 0; w < n_windows; ++w) {
+    // windows by the tile kernel that takes their k; tiles of class c:
+    // [cls_tile[c], cls_tile[c + 1])
+    std::vector<int> order(n_windows);
+    for (int w = 0; w < n_windows; ++w)
+        order[w] = w;
+    std::stable_sort(order.begin(), order.end(), [&](int x, int y) {
+        return tnn_k_class(params[x].k) < tnn_k_class(params[y].k);
+    });
+    long long cls_tile[TNN_CLASSES + 1] = {0};
+    for (int i = 0; i < n_windows; ++i) {
+        const int w = order[i];
         s = tnn_fill_window(indexes[w], d_q ? d_q[w] : nullptr, m[w], &params[w],
-                            d_idx[w], d_d2[w], &wins[w]);
+                            d_idx[w], d_d2[w], &wins[i]);
         if (s != TNN_OK)
             return s;
         TNN_ARG_CHECK(m[w] == 0 || (d_idx[w] != nullptr && d_d2[w] != nullptr),
@@ -711,12 +797,15 @@ extern "C" tnn_status tnn_batch_create(const tnn_index *const *indexes,
         TNN_ARG_CHECK((params[w].flags & TNN_FLAG_SWEEP) == (params[0].flags & TNN_FLAG_SWEEP),
                       "all windows of a batch take the same segment order (TNN_FLAG_SWEEP; window %d "
                       "differs from window 0)", w);
-        wins[w].tile_begin = tiles;
-        tiles += tnn_window_tiles(indexes[w], &wins[w]);
+        wins[i].tile_begin = tiles;
+        tiles += tnn_window_tiles(indexes[w], &wins[i]);
         fb += m[w];
-        L_max = std::max(L_max, wins[w].L);
+        L_max = std::max(L_max, wins[i].L);
+        cls_tile[tnn_k_class(wins[i].k) + 1] = tiles;
         kseg = std::max(kseg, (int)indexes[w]->K);
     }
+    for (int c = 0; c < TNN_CLASSES; ++c) // classes without windows are empty
+        cls_tile[c + 1] = std::max(cls_tile[c + 1], cls_tile[c]);
     tnn_batch *b = new tnn_batch();
     memset(b, 0, sizeof(*b));
     cudaGetDevice(&b->device);
@@ -753,7 +842,10 @@ extern "C" tnn_status tnn_batch_create(const tnn_index *const *indexes,
         e = cudaStreamBeginCapture(cs, cudaStreamCaptureModeThreadLocal);
         if (e == cudaSuccess) {
             cudaMemsetAsync(b->scratch, 0, sizeof(KnnScratch), cs);
-            s = tnn_launch_search(L, false, cs);
+            if (n_windows == 1 || (L.w0.flags & TNN_FLAG_SWEEP))
+                s = tnn_launch_search(L, false, cs);
+            else
+                s = capture_grid_classes(L, cls_tile, cs);
             cudaError_t e2 = cudaStreamEndCapture(cs, &b->graph);
             if (s == TNN_OK && e2 == cudaSuccess)
                 e = cudaGraphInstantiate(&b->exec, b->graph, 0);
@@ -834,17 +926,16 @@ extern "C" tnn_status tnn_autotune(const tnn_index *ix, tnn_knn_params *params,
         tnn_set_error("autotune setup failed: %s", cudaGetErrorString(e));
         s = TNN_ERR_CUDA;
     }
-    // Candidates: the grid order over seed count F, spare slots and the
-    // deferral threshold, plus the sweep order with two seed counts.
+    // Candidates: the grid order over spare slots and the deferral threshold
+    // (it has no seed count), plus the sweep order with two seed counts.
     struct Cand {
         int F, E, flags;
         float defer;
     };
     std::vector<Cand> cands;
-    for (int F : {2, 3, 4})
-        for (int E : {4, 8})
-            for (float dfr : {0.6f, 0.75f, 1.0f, 1.5f, 2.0f, 3.0f, 6.0f})
-                cands.push_back({F, E, 0, dfr});
+    for (int E : {4, 8})
+        for (float dfr : {0.6f, 0.75f, 1.0f, 1.5f, 2.0f, 3.0f, 6.0f})
+            cands.push_back({4, E, 0, dfr});
     for (int F : {3, 4})
         cands.push_back({F, 4, TNN_FLAG_SWEEP, 0.0f});
     float best = 1e30f;

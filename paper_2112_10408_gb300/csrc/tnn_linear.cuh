@@ -25,7 +25,7 @@ __global__ void __launch_bounds__(TNN_WARPS_PER_CTA * 32)
     for (;;) {
         long long tile = 0;
         if (lane == 0)
-            tile = (long long)atomicAdd(&L.scr->tile_counter, 1ull);
+            tile = (long long)atomicAdd(L.scr->tile_counter, 1ull);
         tile = __shfl_sync(FULLMASK, tile, 0);
         if (tile >= L.total_tiles)
             break;

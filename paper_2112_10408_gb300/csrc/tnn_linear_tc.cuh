@@ -199,7 +199,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_linear_tc(const __grid_consta
 
     for (;;) {
         if (t == 0)
-            *s_tile = (long long)atomicAdd(&L.scr->tile_counter, 1ull);
+            *s_tile = (long long)atomicAdd(L.scr->tile_counter, 1ull);
         __syncthreads();
         const long long tile = *s_tile;
         if (tile >= L.total_tiles || *s_err)

@@ -33,6 +33,10 @@
 #include "tnn_grid.cuh"
 #include "tnn_tc.cuh"
 
+#ifndef TNN_GMAX_F
+#define TNN_GMAX_F 6 // largest seed count
+#endif
+
 #define TT_Q 128
 #define TT_P 128
 #define TT_S 8         // ring slots
@@ -153,7 +157,7 @@ __global__ void __launch_bounds__(TT_THREADS, 1) k_tnn_tc(const __grid_constant_
 
     for (;;) {
         if (t == 0)
-            *s_tile = (long long)atomicAdd(&L.scr->tile_counter, 1ull);
+            *s_tile = (long long)atomicAdd(L.scr->tile_counter, 1ull);
         __syncthreads();
         const long long tile = *s_tile;
         if (tile >= L.total_tiles || *s_err)
