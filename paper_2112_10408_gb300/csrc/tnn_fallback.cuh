@@ -5,57 +5,62 @@
 //     aside and carries on with the others -- they are finished here, where
 //     the whole warp works on one query (list of k + extra candidates);
 //   - unsettled (window id stored as -1 - w): the chain of FP32 keys that FP32
-//     cannot order reached the last candidate slot; here the list keeps
-//     k + 32 candidates (a deferred query that ends the same way is run
-//     again at once with k + 32).
+//     cannot order reached the last candidate; here the pruning key is that
+//     of a later rank (a deferred query that ends the same way is run again
+//     at once like that).
 //
 // k_tnn_warp: the 32 lanes split the grid keys, the member segments and the
-// member points of one query.  Candidates below the pruning key are sorted
-// across the warp (bitonic) and merged into a sorted list in shared memory
-// (merge path).  Seeding visits cubes of keys of growing radius around the
-// query's own key (cells in the plane, buckets backwards in time) until the
-// list is full; inside a chunk of segments, while the list is not full, the
-// segment of smallest bound is scanned first (Algorithm 2's nearest-first
-// fetch), so the pruning key is tight as soon as it exists.  The main phase
+// member points of one query.  Its candidates are sorted 32-bit keys (the
+// tile kernel's: the distance's upper bits above a slot), entry r * 32 + lane
+// of the list in register r of a lane.  Up to 32 points at a time: the few
+// that pass are inserted by ballot and shift, many are sorted across the warp
+// and merged by a bitonic network of shuffles.  The next points are fetched
+// while the present ones are merged.  Seeding visits cubes of keys of growing
+// radius around the query's own key (cells in the plane, buckets backwards in
+// time) until the list is full; inside a chunk of segments the nearest is
+// always scanned first (Algorithm 2's nearest-first fetch).  The main phase
 // is the exclusion criterion and stop rule of Algorithm 2 over the other
-// keys, scanning the needed segments of a chunk 32 points at a time.
+// keys.  To settle, the list's distances are taken again in FP32 and put in
+// order, and chains of close keys are ranked by their FP64 distances, a lane
+// per entry, however long a chain is.
+// What bounds it is latency: one query is a chain of dependent L2 reads and
+// merges.  64-bit lists in shared memory (sorted and merge-path merged per 32
+// points), one key per lane and round and a queue ticket for every idle warp
+// took 52 us for the 170 handed-over queries of 10,000 points, 72 us for the
+// 4,400 of 400,000, 584 us for the 56,600 of 4,000,000 and 267 us for the
+// 47,000 of a half-hour-lag nowcast; register lists 52 / 67 / 463 / 215, four
+// keys per lane and round 32 / 49 / 355 / 199, the first entry per warp
+// without a ticket 28 / 45 / 350 / 199.
 // A query still unsettled goes to k_fallback_exact: the definition, with the
 // FP64 distance taken only for the points that FP32 cannot rule out.
 #pragma once
 #include "tnn_device.cuh"
 #include "tnn_grid.cuh"
 
-#define FB_EXTRA 32
-#define WQ_CMAX (64 + FB_EXTRA)
+#define WQ_MORE 28 // ranks beyond k that set the pruning key of an unsettled query
+#define WQ_KEYS 4   // keys per lane and round
+#define WQ_INSERT 4 // at most this many passing points are inserted one by one
 #ifndef WQ_RSEED
 #define WQ_RSEED 4 // largest radius of the seeding shells
 #endif
 
-__host__ __device__ inline size_t wq_smem_per_warp()
-{
-    // list [WQ_CMAX] + merge output [WQ_CMAX] + batch [32] (u64), packed
-    // segment starts and firsts, packed key starts and ranges [4][32] (int),
-    // and the settlement scratch
-    // ([CMAX][32] u64 + [CMAX][32] int) after them
-    return (size_t)(2 * WQ_CMAX + 32) * 8 + 128 * 4 + (size_t)CMAX * 32 * 12;
-}
+struct WarpSmem {
+    union {
+        int slot[TG_SLOTS]; // point index of every slot
+        struct {            // to settle:
+            unsigned long long key[128]; // exact keys
+            double d64[128];
+        };
+    };
+    unsigned used[32]; // renumbering
+    int pre[32];
+    int kend[32 * WQ_KEYS]; // key ranges of the present round: ends and offsets
+    int krel[32 * WQ_KEYS];
+};
 
 __host__ __device__ inline size_t fb_exact_smem_per_warp(int k_max)
 {
     return (size_t)k_max * 32 * 12;
-}
-
-// The settlement of the warp-per-query kernel, out of line (lane 0 only,
-// and only for queries with close ranks): bit 0 = settled, the rest the
-// FP64 rechecks made.  Keeps its body out of the kernel's hot loop code.
-static __device__ __noinline__ unsigned finalize_query_ool(const KnnWin *W, float4 q,
-                                                          const unsigned long long *K, int L,
-                                                          unsigned long long *cl_d, int *cl_i,
-                                                          int64_t qrow)
-{
-    LaneStats st = {0, 0, 0, 0, 0};
-    const bool ok = finalize_query(W, q, K, L, cl_d, cl_i, qrow, st, 1);
-    return ((unsigned)st.fp64 << 1) | (ok ? 1u : 0u);
 }
 
 __device__ __forceinline__ unsigned long long shfl_xor_u64(unsigned long long v, int m)
@@ -63,116 +68,99 @@ __device__ __forceinline__ unsigned long long shfl_xor_u64(unsigned long long v,
     return __shfl_xor_sync(FULLMASK, v, m);
 }
 
-// Ascending bitonic sort of one key per lane across the warp.
-__device__ __forceinline__ unsigned long long warp_sort_u64(unsigned long long v, int lane)
+__device__ __forceinline__ int warp_incl_sum(int v, int lane)
 {
 #pragma unroll
-    for (int k = 2; k <= 32; k <<= 1) {
+    for (int o = 1; o < 32; o <<= 1) {
+        const int t = __shfl_up_sync(FULLMASK, v, o);
+        if (lane >= o)
+            v += t;
+    }
+    return v;
+}
+
+// Ascending order of one key per lane.
+__device__ __forceinline__ unsigned wq_sort(unsigned v, int lane)
+{
+#pragma unroll
+    for (int k = 2; k <= 32; k <<= 1)
 #pragma unroll
         for (int j = k >> 1; j > 0; j >>= 1) {
-            const unsigned long long o = shfl_xor_u64(v, j);
-            const bool up = (lane & k) == 0;
-            const bool lower = (lane & j) == 0;
-            const unsigned long long mn = o < v ? o : v, mx = o < v ? v : o;
-            v = (lower == up) ? mn : mx;
+            const unsigned o = __shfl_xor_sync(FULLMASK, v, j);
+            v = ((lane & k) == 0) == ((lane & j) == 0) ? min(v, o) : max(v, o);
         }
-    }
     return v;
 }
 
-__device__ __forceinline__ unsigned long long warp_min_u64(unsigned long long v)
+// Merge a sorted key per lane into the list: the 32 NR smallest stay.
+template <int NR> __device__ __forceinline__ void wq_merge(unsigned (&a)[NR], unsigned b, int lane)
 {
-    for (int o = 16; o > 0; o >>= 1) {
-        const unsigned long long w = shfl_xor_u64(v, o);
-        v = w < v ? w : v;
-    }
-    return v;
+    a[NR - 1] = min(a[NR - 1], __shfl_xor_sync(FULLMASK, b, 31));
+#pragma unroll
+    for (int h = NR / 2; h > 0; h >>= 1)
+#pragma unroll
+        for (int r = 0; r < NR; ++r)
+            if ((r & h) == 0)
+                tg_cmpx(a[r], a[r + h]);
+#pragma unroll
+    for (int j = 16; j > 0; j >>= 1)
+#pragma unroll
+        for (int r = 0; r < NR; ++r) {
+            const unsigned o = __shfl_xor_sync(FULLMASK, a[r], j);
+            a[r] = (lane & j) == 0 ? min(a[r], o) : max(a[r], o);
+        }
 }
 
-struct WarpList {
-    unsigned long long *L;   // [C] sorted keys, SENT beyond nv
-    unsigned long long *tmp; // [C]
-    unsigned long long *B;   // [32]
-    int C, nv;
-    unsigned long long tauk; // largest key kept once full, else bound0
-    unsigned long long bound0; // no key above it can enter the list
-};
-
-// Merge the keys below the pruning key (at most one per lane) into the list.
-__device__ __forceinline__ void wl_merge(WarpList &w, unsigned long long ck, int lane)
+// Insert one key (the same in every lane).
+template <int NR> __device__ __forceinline__ void wq_insert(unsigned (&a)[NR], unsigned key, int lane)
 {
-    const bool take = ck < w.tauk;
-    const unsigned m = __ballot_sync(FULLMASK, take);
-    if (!m)
-        return;
-    const int nb = __popc(m);
-    const unsigned long long v = warp_sort_u64(take ? ck : SENT, lane);
-    w.B[lane] = v;
-    __syncwarp();
-    const int na = w.nv;
-    for (int p = lane; p < w.C; p += 32) {
-        int lo = max(0, p - nb), hi = min(p, na);
-        while (lo < hi) {
-            const int mid = (lo + hi) >> 1;
-            if (w.L[mid] < w.B[p - mid - 1])
-                lo = mid + 1;
-            else
-                hi = mid;
+    int pos = 0;
+#pragma unroll
+    for (int r = 0; r < NR; ++r)
+        pos += __popc(__ballot_sync(FULLMASK, a[r] < key));
+#pragma unroll
+    for (int r = NR - 1; r >= 0; --r) {
+        unsigned prev = __shfl_up_sync(FULLMASK, a[r], 1);
+        if (r > 0) {
+            const unsigned last = __shfl_sync(FULLMASK, a[r > 0 ? r - 1 : 0], 31);
+            prev = lane == 0 ? last : prev;
         }
-        const int i = lo, j = p - lo;
-        unsigned long long out = SENT;
-        if (i < na && (j >= nb || w.L[i] < w.B[j]))
-            out = w.L[i];
-        else if (j < nb)
-            out = w.B[j];
-        w.tmp[p] = out;
+        const int g = r * 32 + lane;
+        a[r] = g < pos ? a[r] : g == pos ? key : prev;
     }
-    __syncwarp();
-    for (int p = lane; p < w.C; p += 32)
-        w.L[p] = w.tmp[p];
-    __syncwarp();
-    w.nv = min(na + nb, w.C);
-    w.tauk = w.nv == w.C ? w.L[w.C - 1] : w.bound0;
 }
 
 #ifndef TNN_WARP_MINB
-#define TNN_WARP_MINB 7 // 7 CTAs (28 warps, 73 registers) per SM: fewer spills than 8 at 64 registers
+#define TNN_WARP_MINB 6 // CTAs per SM (4 M points: 5 368 us, 6 350, 7 353; fewer spill less when few queries come)
 #endif
+// NR list registers per lane: 32 NR candidates, for k <= 32 NR - 16.
+template <int NR>
 __global__ void __launch_bounds__(TNN_WARPS_PER_CTA * 32, TNN_WARP_MINB)
     k_tnn_warp(const __grid_constant__ KnnLaunch L)
 {
-    extern __shared__ __align__(16) unsigned char smem[];
+    __shared__ __align__(16) WarpSmem smem[TNN_WARPS_PER_CTA];
     const int lane = threadIdx.x & 31;
-    unsigned char *ws = smem + (threadIdx.x >> 5) * wq_smem_per_warp();
-    WarpList wl;
-    wl.L = (unsigned long long *)ws;
-    wl.tmp = wl.L + WQ_CMAX;
-    wl.B = wl.tmp + WQ_CMAX;
-    int *Sstart = (int *)(wl.B + 32);
-    int *Sfirst = Sstart + 32;
-    int *Kstart = Sfirst + 32;
-    int *Klo = Kstart + 32;
-    unsigned long long *cl_d = (unsigned long long *)(Klo + 32);
-    int *cl_i = (int *)((unsigned char *)cl_d + CMAX * 32 * 8);
+    WarpSmem &S = smem[threadIdx.x >> 5];
 
     unsigned nfb = *(volatile unsigned *)&L.scr->n_fallback;
     if ((long long)nfb > L.fb_cap)
         nfb = (unsigned)L.fb_cap;
-    const int gw = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const int nw = (gridDim.x * blockDim.x) >> 5;
-    (void)gw;
-    (void)nw;
-    LaneStats st = {0, 0, 0, 0, 0};
+    unsigned n_lb = 0, n_pairs = 0, n_segs = 0, n_fp = 0;
     int2 ent = make_int2(0, 0);
     bool retry = false; // the same query again with the larger list
     float tau0 = INFINITY;
-    for (;;) {
+    // Dynamic queue (query costs differ by orders of magnitude) behind one
+    // entry per warp, dealt out over the CTAs: thousands of warps asking the
+    // counter at once, most of them in vain when few queries were handed
+    // over, would wait on one another.
+    unsigned e = (threadIdx.x >> 5) * gridDim.x + blockIdx.x;
+    for (bool first = true;; first = false) {
         if (!retry) {
-            // dynamic queue: query costs differ by orders of magnitude
-            unsigned e = 0;
-            if (lane == 0)
-                e = atomicAdd(&L.scr->fb_next, 1u);
-            e = __shfl_sync(FULLMASK, e, 0);
+            if (!first) {
+                if (lane == 0)
+                    e = atomicAdd(&L.scr->fb_next, 1u) + gridDim.x * TNN_WARPS_PER_CTA;
+                e = __shfl_sync(FULLMASK, e, 0);
+            }
             if (e >= nfb)
                 break;
             ent = L.fb_list[e];
@@ -184,144 +172,178 @@ __global__ void __launch_bounds__(TNN_WARPS_PER_CTA * 32, TNN_WARP_MINB)
         const float4 q = W->q[ent.y];
         const QCtx c = make_qctx(W, q, true);
         const float s0 = W->sig[0], s1 = W->sig[1], s2 = W->sig[2], s3 = W->sig[3];
-        const float4 *__restrict__ seg = W->seg;
         const float4 *__restrict__ pts = W->pts;
         const GridDesc &G = W->grid;
-        wl.C = unsettled ? W->k + FB_EXTRA : W->L;
-        wl.nv = 0;
-        // A deferred query arrives with the pruning key tau0 of the tile
-        // kernel's list of the same length (the same FP32 keys): its final
-        // list holds no key with a distance above tau0.
-        wl.bound0 = (unsettled || !(tau0 < INFINITY))
-                        ? SENT
-                        : (((unsigned long long)__float_as_uint(tau0) << 32) | 0xffffffffull);
-        wl.tauk = wl.bound0;
-        for (int p = lane; p < wl.C; p += 32)
-            wl.L[p] = SENT;
-        __syncwarp();
+        const int k = W->k;
+        // rank whose key prunes: every point up to a little above it is seen
+        const int C = unsettled ? min(k + WQ_MORE, 32 * NR - 1) : k;
+        unsigned a[NR];
+#pragma unroll
+        for (int r = 0; r < NR; ++r)
+            a[r] = TG_EMPTY;
+        // A deferred query may arrive with a pruning key: at least k + 4
+        // points lie at or below it.
+        float tau = unsettled ? INFINITY : tau0;
+        bool filled = false; // the list has its C-th key
+        int base = 0;
 
-        // all points of one segment, 32 at a time
-        auto scan_seg = [&](int first, int cnt) {
-            if (lane == 0)
-                st.segs++;
-            if (L.dbg_seen && lane == 0)
-                dbg_mark_seen(L, ent.y, first, cnt);
-            for (int o = 0; o < cnt; o += 32) {
-                const int j = o + lane;
-                unsigned long long ck = SENT;
-                if (j < cnt) {
-                    const float4 p = __ldg(pts + first + j);
-                    const float d = dist32(c, s0, s1, s2, s3, p);
-                    if (p.w < c.T32)
-                        ck = pack_key(d, first + j);
-                    st.pairs++;
-                }
-                wl_merge(wl, ck, lane);
-            }
-        };
-        // the points of every lane's segment with `need`, packed 32 per step
-        auto scan_packed = [&](bool need, float4 meta) {
-            const unsigned m = __ballot_sync(FULLMASK, need);
-            const int cnt = need ? __float_as_int(meta.y) : 0;
-            int incl = cnt;
-            for (int o = 1; o < 32; o <<= 1) {
-                const int t = __shfl_up_sync(FULLMASK, incl, o);
-                if (lane >= o)
-                    incl += t;
-            }
-            const int total = __shfl_sync(FULLMASK, incl, 31);
-            const int nseg = __popc(m);
-            if (need) {
-                const int rank = __popc(m & ((1u << lane) - 1u));
-                Sstart[rank] = incl - cnt;
-                Sfirst[rank] = __float_as_int(meta.x);
-                if (L.dbg_seen)
-                    dbg_mark_seen(L, ent.y, __float_as_int(meta.x), cnt);
-            }
-            if (lane == 0)
-                st.segs += nseg;
-            __syncwarp();
-            for (int s = 0; s < total; s += 32) {
-                const int g = s + lane;
-                unsigned long long ck = SENT;
-                if (g < total) {
-                    int lo = 0, hi = nseg - 1; // largest r with Sstart[r] <= g
-                    while (lo < hi) {
-                        const int mid = (lo + hi + 1) >> 1;
-                        if (Sstart[mid] <= g)
-                            lo = mid;
-                        else
-                            hi = mid - 1;
-                    }
-                    const int j = Sfirst[lo] + (g - Sstart[lo]);
-                    const float4 p = __ldg(pts + j);
-                    const float d = dist32(c, s0, s1, s2, s3, p);
-                    if (p.w < c.T32)
-                        ck = pack_key(d, j);
-                    st.pairs++;
-                }
-                wl_merge(wl, ck, lane);
-            }
-            __syncwarp();
-        };
-        // the member segments of one key whose cylinder bound does not exceed
-        // the pruning key; nearest first while the list is not full
-        // The member segments of every lane's key (key < 0: none; [klo, khi)
-        // its range of G.ids) are handled together, 32 segments per step
-        // whatever key they belong to.
-        auto visit_keys = [&](bool has, int klo, int khi) {
-            const unsigned km = __ballot_sync(FULLMASK, has);
-            if (!km)
+        // one point per lane (j < 0: none), loaded as p
+        auto consider = [&](int j, const float4 &p) {
+            const float d = dist32(c, s0, s1, s2, s3, p);
+            const bool in = j >= 0 && p.w < c.T32 && d <= tau;
+            unsigned m = __ballot_sync(FULLMASK, in);
+            n_pairs += j >= 0;
+            if (!m)
                 return;
-            const int kc = has ? khi - klo : 0;
-            int incl = kc;
-            for (int o = 1; o < 32; o <<= 1) {
-                const int t = __shfl_up_sync(FULLMASK, incl, o);
-                if (lane >= o)
-                    incl += t;
+            if (base > TG_SLOTS - 32) {
+                // renumber the slots the list still holds (at most 32 NR)
+                __syncwarp();
+                S.used[lane] = 0;
+                __syncwarp();
+#pragma unroll
+                for (int r = 0; r < NR; ++r)
+                    if (a[r] != TG_EMPTY)
+                        atomicOr(&S.used[(a[r] & TG_SMASK) >> 5], 1u << (a[r] & 31u));
+                __syncwarp();
+                const unsigned u = S.used[lane];
+                const int inc = warp_incl_sum(__popc(u), lane);
+                S.pre[lane] = inc - __popc(u);
+                base = __shfl_sync(FULLMASK, inc, 31);
+                __syncwarp();
+#pragma unroll
+                for (int r = 0; r < NR; ++r) {
+                    const unsigned s = a[r] & TG_SMASK;
+                    if (a[r] != TG_EMPTY)
+                        a[r] = (a[r] & ~TG_SMASK) |
+                               (unsigned)(S.pre[s >> 5] + __popc(S.used[s >> 5] & ((1u << (s & 31u)) - 1u)));
+                }
+#pragma unroll 1
+                for (int w = 0; w < 32; ++w) {
+                    const unsigned uw = S.used[w];
+                    const int id = S.slot[w * 32 + lane];
+                    __syncwarp();
+                    if ((uw >> lane) & 1u)
+                        S.slot[S.pre[w] + __popc(uw & ((1u << lane) - 1u))] = id;
+                    __syncwarp();
+                }
             }
-            const int total = __shfl_sync(FULLMASK, incl, 31);
-            const int nk = __popc(km);
+            const int slot = base + __popc(m & ((1u << lane) - 1u));
+            if (in)
+                S.slot[slot] = j;
+            base += __popc(m);
+            const unsigned key = in ? tg_key(d, (unsigned)slot) : TG_EMPTY;
+            if (__popc(m) <= WQ_INSERT) {
+#pragma unroll 1
+                do {
+                    const int src = __ffs(m) - 1;
+                    m &= m - 1;
+                    wq_insert<NR>(a, __shfl_sync(FULLMASK, key, src), lane);
+                } while (m);
+            } else {
+                wq_merge<NR>(a, wq_sort(key, lane), lane);
+            }
+            unsigned kc = a[0];
+#pragma unroll
+            for (int r = 1; r < NR; ++r)
+                kc = (C - 1) >> 5 == r ? a[r] : kc;
+            kc = __shfl_sync(FULLMASK, kc, (C - 1) & 31);
+            filled = kc != TG_EMPTY;
+            if (kc < TG_INF)
+                tau = fminf(tau, fmaf(tg_upper(kc), 0x1p-12f, tg_upper(kc)) + 0x1p-98f);
+        };
+        // The member segments of every lane's keys ([klo, klo + kn) in key
+        // order), 32 segments per step whatever key they belong to.
+        auto visit_keys = [&](const int (&klo)[WQ_KEYS], const int (&kn)[WQ_KEYS]) {
+            int sum = 0;
+#pragma unroll
+            for (int u = 0; u < WQ_KEYS; ++u)
+                sum += kn[u];
+            if (!__any_sync(FULLMASK, sum > 0))
+                return;
+            const int inc = warp_incl_sum(sum, lane);
+            const int total = __shfl_sync(FULLMASK, inc, 31);
             __syncwarp();
-            if (has) {
-                const int rank = __popc(km & ((1u << lane) - 1u));
-                Kstart[rank] = incl - kc;
-                Klo[rank] = klo;
+            int at = inc - sum;
+#pragma unroll
+            for (int u = 0; u < WQ_KEYS; ++u) {
+                S.krel[lane * WQ_KEYS + u] = klo[u] - at;
+                at += kn[u];
+                S.kend[lane * WQ_KEYS + u] = at;
             }
             __syncwarp();
-            for (int base = 0; base < total; base += 32) {
-                const int g = base + lane;
-                float lb = __int_as_float(0x7fffffff);
-                float4 meta = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll 1
+            for (int b0 = 0; b0 < total; b0 += 32) {
+                const int g = b0 + lane;
+                unsigned score = TG_EMPTY; // bound above the lane
+                int first = 0, cnt = 0;
                 if (g < total) {
-                    int a = 0, z = nk - 1; // largest r with Kstart[r] <= g
-                    while (a < z) {
-                        const int mid = (a + z + 1) >> 1;
-                        if (Kstart[mid] <= g)
-                            a = mid;
+                    int lo = 0, hi = 32 * WQ_KEYS - 1; // smallest range with kend > g
+#pragma unroll 1
+                    while (lo < hi) {
+                        const int mid = (lo + hi) >> 1;
+                        if (S.kend[mid] > g)
+                            hi = mid;
                         else
-                            z = mid - 1;
+                            lo = mid + 1;
                     }
-                    const float4 *src = G.gseg + 4 * (size_t)(Klo[a] + (g - Kstart[a]));
-                    meta = __ldg(src + 3);
-                    lb = seg_lb(c, s3, __ldg(src), __ldg(src + 1), __ldg(src + 2));
-                    st.lb++;
+                    const float4 *src = G.gseg + 4 * (size_t)(S.krel[lo] + g);
+                    const float4 r3 = __ldg(src + 3);
+                    const float lb = seg_lb(c, s3, __ldg(src), __ldg(src + 1), __ldg(src + 2));
+                    first = __float_as_int(r3.x);
+                    cnt = __float_as_int(r3.y);
+                    // truncated towards zero: still a lower bound
+                    if (lb <= tau)
+                        score = (__float_as_uint(lb) & ~31u) | (unsigned)lane;
+                    n_lb++;
                 }
-                while (wl.nv < wl.C) {
-                    const bool need = lb <= key_d(wl.tauk);
-                    const unsigned long long arg = warp_min_u64(
-                        need ? (((unsigned long long)__float_as_uint(lb) << 32) | (unsigned)lane) : ~0ull);
-                    if (arg == ~0ull)
-                        break;
-                    const int who = (int)(arg & 31u);
-                    scan_seg(__float_as_int(__shfl_sync(FULLMASK, meta.x, who)),
-                             __float_as_int(__shfl_sync(FULLMASK, meta.y, who)));
-                    if (lane == who)
-                        lb = __int_as_float(0x7fffffff);
-                }
-                const bool need = lb <= key_d(wl.tauk);
-                if (__any_sync(FULLMASK, need))
-                    scan_packed(need, meta);
+                // up to 32 points of the nearest segments: this lane's index
+                int lf = 0, lc = 0;
+                auto gather = [&](int &j) -> bool {
+                    int fill = 0;
+                    j = -1;
+#pragma unroll 1
+                    while (fill < 32) {
+                        if (lc == 0) {
+                            const unsigned best = __reduce_min_sync(FULLMASK, score);
+                            if (best == TG_EMPTY || !(__uint_as_float(best & ~31u) <= tau))
+                                break;
+                            const int w = best & 31u;
+                            if (lane == w)
+                                score = TG_EMPTY;
+                            lf = __shfl_sync(FULLMASK, first, w);
+                            lc = __shfl_sync(FULLMASK, cnt, w);
+                            if (lane == 0) {
+                                n_segs++;
+                                if (L.dbg_seen)
+                                    dbg_mark_seen(L, ent.y, lf, lc);
+                            }
+                        }
+                        const int take = min(lc, 32 - fill);
+                        if (lane >= fill && lane < fill + take)
+                            j = lf + lane - fill;
+                        lf += take;
+                        lc -= take;
+                        fill += take;
+                    }
+                    return fill > 0;
+                };
+                int j = -1;
+                bool have = false;
+                float4 p = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll 1
+                do {
+                    // the next points are on their way while these are merged
+                    int jn;
+                    const bool more = gather(jn);
+                    float4 pn = make_float4(0.f, 0.f, 0.f, 0.f);
+                    if (jn >= 0)
+                        pn = __ldg(pts + jn);
+                    if (have)
+                        consider(j, p);
+                    j = jn;
+                    p = pn;
+                    have = more;
+                } while (have);
             }
         };
 
@@ -336,127 +358,212 @@ __global__ void __launch_bounds__(TNN_WARPS_PER_CTA * 32, TNN_WARP_MINB)
             const int hy = min(max((int)floorf((c.sy - G.y0) * G.inv_cell), 0), G.ny - 1);
             const int rcover = max(max(max(hx, G.nx - 1 - hx), max(hy, G.ny - 1 - hy)), bhi);
             const float ext_max = __ldg(G.ext_max);
-            // One loop hands visit_keys the keys of both phases, up to 32 per
-            // round (a single inlined copy of the visit and its merges):
-            // ---- seeding: shells of growing radius around the query's key, at
-            // most WQ_RSEED + 1 of them (a query with fewer than C valid points
-            // would otherwise grow the cube over the whole grid; the main
-            // phase visits each causal bucket once instead);
-            // ---- main: buckets backwards, keys within reach, by bound.
+            // One loop hands visit_keys the keys of both phases, up to 128 per
+            // round -- a round is a chain of dependent reads, so it takes as
+            // many keys as four reads in flight per lane bring:
+            // ---- seeding: cubes of growing radius around the query's key, the
+            // first one whole, then shells up to radius WQ_RSEED (a query with
+            // fewer than C valid points would otherwise grow the cube over the
+            // whole grid; the main phase visits each causal bucket once
+            // instead);
+            // ---- main: buckets backwards, keys within reach, by bound, as
+            // many buckets per round as fit.
             bool seeding = true;
-            int rs = -1, side = 1, nk = 0, t0 = 0; // shell rs of side x side x (rs + 1) positions
-            int b = bhi + 1, cx0 = 0, cy0 = 0, wx = 1; // main: bucket b, its reach rectangle
-            bool bseed = false;
-            float bpm_next = 0.0f;
+            int rs = 0, nk = 0, t0 = 0;                // shell rs of side x side x (rs + 1) positions
+            int b = bhi, cx0 = 0, cy0 = 0, wx = 1, nc = 1; // main: next bucket, the reach rectangle
+            float inv_nc = 1.0f, inv_wx = 1.0f;        // positions per bucket (or age) and per row
+#pragma unroll 1
             for (;;) {
-                int klo = 0, khi = 0;
-                if (seeding) {
-                    if (t0 >= nk) {
-                        if (!(wl.nv < wl.C && rs < rcover && rs < WQ_RSEED)) {
-                            seeding = false;
-                            if (rs >= rcover)
-                                break; // the shells covered every causal key
-                            bpm_next = __ldg(G.bpm + bhi); // one bucket ahead
-                            nk = 0;
-                            t0 = 0;
-                            continue;
-                        }
+                if (t0 >= nk) {
+                    t0 = 0;
+                    if (seeding && rs > 0 && (filled || rs >= rcover || rs >= WQ_RSEED)) {
+                        seeding = false;
+                        if (rs >= rcover)
+                            break; // the shells covered every causal key
+                    }
+                    if (seeding) {
                         ++rs;
-                        side = 2 * rs + 1;
-                        nk = side * side * (rs + 1);
-                        t0 = 0;
-                    }
-                    const int t = t0 + lane, r = rs;
-                    if (t < nk) {
-                        const int db = t / (side * side), rem = t % (side * side);
-                        const int dy = rem / side - r, dx = rem % side - r;
-                        const int bk = bhi - db, cx = hx + dx, cy = hy + dy;
-                        const bool shell = max(max(abs(dx), abs(dy)), db) == r;
-                        if (shell && bk >= 0 && cx >= 0 && cx < G.nx && cy >= 0 && cy < G.ny) {
-                            const int k2 = bk * G.ncell + cy * G.nx + cx;
-                            klo = __ldg(G.off + k2);
-                            khi = __ldg(G.off + k2 + 1);
-                        }
-                    }
-                } else {
-                    if (t0 >= nk) {
-                        if (--b < 0)
-                            break;
-                        const float tau = key_d(wl.tauk);
-                        const float bpm_b = bpm_next;
-                        if (b > 0)
-                            bpm_next = __ldg(G.bpm + b - 1);
-                        if (!(time_lb(c, s3, bpm_b) <= tau))
+                        wx = 2 * rs + 1;
+                        nc = wx * wx;
+                        nk = nc * (rs + 1);
+                        cx0 = hx - rs;
+                        cy0 = hy - rs;
+                        b = bhi;
+                    } else {
+                        // buckets the temporal bound still allows (a prefix)
+                        const unsigned bm = __ballot_sync(
+                            FULLMASK, b - lane >= 0 && time_lb(c, s3, __ldg(G.bpm + max(b - lane, 0))) <= tau);
+                        const int nbk = bm == FULLMASK ? 32 : __ffs(~bm) - 1;
+                        if (nbk == 0)
                             break;
                         const float R = sqrtf(tau) * (1.0f + 0x1p-18f) + ext_max + c.delta;
                         int cx1, cy1;
                         reach_cells(c.sx, c.sx, R, G.x0, G.inv_cell, G.nx, cx0, cx1);
                         reach_cells(c.sy, c.sy, R, G.y0, G.inv_cell, G.ny, cy0, cy1);
                         wx = cx1 - cx0 + 1;
-                        nk = wx * (cy1 - cy0 + 1);
-                        bseed = bhi - b <= rs;
-                        t0 = 0;
+                        nc = max(wx, 0) * max(cy1 - cy0 + 1, 0);
+                        if (nc == 0)
+                            break; // no cell within reach
+                        nk = nc * max(1, min(nbk, 32 * WQ_KEYS / nc));
                     }
-                    const int t = t0 + lane;
-                    if (t < nk) {
-                        const int cx = cx0 + t % wx, cy = cy0 + t / wx;
-                        const bool seeded = bseed && abs(cx - hx) <= rs && abs(cy - hy) <= rs;
-                        if (!seeded) {
-                            const int k2 = b * G.ncell + cy * G.nx + cx;
-                            const int4 kr = __ldg(G.krec + k2);
-                            const int a0 = kr.x, a1 = kr.y;
-                            if (a1 > a0) {
-                                const float rx0 = G.x0 + (float)cx * G.cell;
-                                const float ry0 = G.y0 + (float)cy * G.cell;
-                                if (cell_lb(c, s3, rx0, rx0 + G.cell, ry0, ry0 + G.cell,
-                                            __int_as_float(kr.z), __int_as_float(kr.w)) <= key_d(wl.tauk)) {
-                                    klo = a0;
-                                    khi = a1;
-                                }
-                            }
+                    inv_nc = 1.0f / (float)nc;
+                    inv_wx = 1.0f / (float)wx;
+                }
+                int klo[WQ_KEYS], kn[WQ_KEYS];
+                int4 kr[WQ_KEYS];
+                int kx[WQ_KEYS], ky[WQ_KEYS];
+#pragma unroll
+                for (int u = 0; u < WQ_KEYS; ++u) {
+                    const int t = t0 + u * 32 + lane;
+                    // quotients of integers below 2^21: exact
+                    const int db = (int)(((float)t + 0.5f) * inv_nc), rem = t - db * nc;
+                    const int dy = (int)(((float)rem + 0.5f) * inv_wx);
+                    const int cx = cx0 + rem - dy * wx, cy = cy0 + dy, bk = b - db;
+                    bool in = t < nk && bk >= 0 && cx >= 0 && cx < G.nx && cy >= 0 && cy < G.ny;
+                    // what the seeding has visited (or, shell by shell, visits)
+                    const int cheb = max(max(abs(cx - hx), abs(cy - hy)), bhi - bk);
+                    in = in && (seeding ? (rs == 1 || cheb == rs) : cheb > rs);
+                    kr[u] = in ? __ldg(G.krec + (bk * G.ncell + cy * G.nx + cx)) : make_int4(0, 0, 0, 0);
+                    kx[u] = cx;
+                    ky[u] = cy;
+                }
+#pragma unroll
+                for (int u = 0; u < WQ_KEYS; ++u) {
+                    klo[u] = kr[u].x;
+                    kn[u] = kr[u].y - kr[u].x;
+                    const float rx0 = G.x0 + (float)kx[u] * G.cell, ry0 = G.y0 + (float)ky[u] * G.cell;
+                    if (!(cell_lb(c, s3, rx0, rx0 + G.cell, ry0, ry0 + G.cell, __int_as_float(kr[u].z),
+                                  __int_as_float(kr[u].w)) <= tau))
+                        kn[u] = 0;
+                }
+                t0 += 32 * WQ_KEYS;
+                if (!seeding && t0 >= nk)
+                    b -= nk / nc;
+                visit_keys(klo, kn);
+            }
+        }
+        // ---- settle
+        __syncwarp();
+        bool ok;
+        {
+            // Points outside the list lie at or above `bound` (none when the
+            // pruning key never took effect and nothing left the list).
+            float bound = tau;
+            const unsigned last = __shfl_sync(FULLMASK, a[NR - 1], 31);
+            if (last != TG_EMPTY)
+                bound = fminf(bound, tg_lower(last));
+            int id[NR], n = 0;
+#pragma unroll
+            for (int r = 0; r < NR; ++r) {
+                id[r] = a[r] != TG_EMPTY ? S.slot[a[r] & TG_SMASK] : -1;
+                n += __popc(__ballot_sync(FULLMASK, id[r] >= 0));
+            }
+            __syncwarp();
+#pragma unroll
+            for (int r = 0; r < NR; ++r) {
+                unsigned long long key = SENT;
+                if (id[r] >= 0)
+                    key = pack_key(dist32(c, s0, s1, s2, s3, __ldg(pts + id[r])), id[r]);
+                S.key[r * 32 + lane] = key;
+            }
+            __syncwarp();
+            // the truncated keys had them almost in order: odd-even exchanges
+            bool swapped;
+#pragma unroll 1
+            do {
+                swapped = false;
+#pragma unroll 1
+                for (int ph = 0; ph < 2; ++ph) {
+                    for (int i = 2 * lane + ph; i + 1 < n; i += 64) {
+                        const unsigned long long x = S.key[i], y = S.key[i + 1];
+                        if (y < x) {
+                            S.key[i] = y;
+                            S.key[i + 1] = x;
+                            swapped = true;
                         }
                     }
+                    __syncwarp();
                 }
-                t0 += 32;
-                visit_keys(khi > klo, klo, khi);
+            } while (__any_sync(FULLMASK, swapped));
+            // entries certainly below every point outside; which are close to
+            // their successor (or to the bound)
+            int ne = 0;
+#pragma unroll
+            for (int r = 0; r < NR; ++r) {
+                const int i = r * 32 + lane;
+                ne += __popc(__ballot_sync(FULLMASK, i < n && !(key_d(S.key[i]) >= bound)));
             }
-        }
-        __syncwarp();
-        // Settle.  When no two of the first k keys are close enough to need
-        // FP64 (no chain), the answer is the first k keys as they are and the
-        // warp writes it; otherwise lane 0 settles the chains.
-        bool ok = true;
-        {
-            const int k = W->k;
-            bool chain = (W->flags & TNN_FLAG_EXACT_D2) != 0;
-            for (int i = lane; i < k; i += 32) {
-                const unsigned long long ki = wl.L[i];
-                if (ki != SENT && i + 1 < wl.C) {
-                    const unsigned long long kn = wl.L[i + 1];
-                    const float de = key_d(ki);
-                    chain |= kn != SENT && key_d(kn) <= fmaf(de, 0x1p-17f, de) + 0x1p-100f;
+            const bool full = bound < INFINITY;
+            unsigned cl[NR];
+#pragma unroll
+            for (int r = 0; r < NR; ++r) {
+                const int i = r * 32 + lane;
+                bool close = false;
+                if (i < ne) {
+                    const float d = key_d(S.key[i]), lim = fmaf(d, 0x1p-17f, d) + 0x1p-100f;
+                    close = i + 1 < ne ? key_d(S.key[i + 1]) <= lim : full && bound <= lim;
                 }
+                cl[r] = __ballot_sync(FULLMASK, close);
             }
-            if (!__any_sync(FULLMASK, chain)) {
+            auto is_close = [&](int i) {
+                unsigned w = cl[0];
+#pragma unroll
+                for (int r = 1; r < NR; ++r)
+                    w = (i >> 5) == r ? cl[r] : w;
+                return ((w >> (i & 31)) & 1u) != 0;
+            };
+            const bool exact_all = (W->flags & TNN_FLAG_EXACT_D2) != 0;
+            // end of the chain that holds rank k
+            int end = min(k, ne) - 1;
+#pragma unroll 1
+            while (end >= 0 && end < ne && is_close(end))
+                ++end;
+            // overflowed distances cannot be ranked here
+            const bool over = n > 0 && !(key_d(S.key[n > 0 ? n - 1 : 0]) < INFINITY);
+            ok = !over && !(full && ne < k) && end < ne;
+            if (ok) {
                 int32_t *oi = W->out_idx + (int64_t)ent.y * k;
                 float *od = W->out_d2 + (int64_t)ent.y * k;
-                for (int i = lane; i < k; i += 32) {
-                    const unsigned long long ki = wl.L[i];
-                    oi[i] = ki == SENT ? -1 : key_i(ki);
-                    od[i] = ki == SENT ? INFINITY : key_d(ki);
+#pragma unroll 1
+                for (int i = lane; i <= end; i += 32)
+                    if (exact_all || is_close(i) || (i > 0 && is_close(i - 1))) {
+                        S.d64[i] = dist64(W->sigd, q, __ldg(pts + key_i(S.key[i])));
+                        n_fp++;
+                    }
+                __syncwarp();
+#pragma unroll 1
+                for (int i = lane; i < max(end + 1, k); i += 32) {
+                    if (i > end) { // fewer than k valid points
+                        oi[i] = -1;
+                        od[i] = INFINITY;
+                        continue;
+                    }
+                    const unsigned long long key = S.key[i];
+                    const bool chain = is_close(i) || (i > 0 && is_close(i - 1));
+                    int rank = i;
+                    if (chain) {
+                        int t = i;
+                        while (t > 0 && is_close(t - 1))
+                            --t;
+                        rank = t;
+                        const double d = S.d64[i];
+                        for (;; ++t) {
+                            const double o = S.d64[t];
+                            rank += o < d || (o == d && key_i(S.key[t]) < key_i(key));
+                            if (!is_close(t))
+                                break;
+                        }
+                    }
+                    if (rank < k) {
+                        oi[rank] = key_i(key);
+                        od[rank] = chain || exact_all ? (float)S.d64[i] : key_d(key);
+                    }
                 }
-            } else {
-                if (lane == 0) {
-                    const unsigned r = finalize_query_ool(W, q, wl.L, wl.C, cl_d, cl_i, ent.y);
-                    ok = (r & 1u) != 0;
-                    st.fp64 += r >> 1;
-                }
-                ok = __shfl_sync(FULLMASK, ok, 0);
             }
         }
-        // a tie chain ran past the end of a k + extra list: once more with
-        // k + FB_EXTRA slots before the FP64 definition is used
-        retry = !ok && wl.C < W->k + FB_EXTRA;
+        // a chain ran past the pruning key of rank k: once more with that of a
+        // later rank before the FP64 definition is used
+        retry = !ok && !unsettled;
         if (!ok && !retry && lane == 0) {
             const unsigned slot = atomicAdd(&L.scr->n_fallback3, 1u);
             if (slot < (unsigned long long)L.fb_cap)
@@ -466,7 +573,7 @@ __global__ void __launch_bounds__(TNN_WARPS_PER_CTA * 32, TNN_WARP_MINB)
         }
         __syncwarp();
     }
-    unsigned long long v[4] = {st.lb, st.pairs, st.segs, st.fp64};
+    unsigned v[4] = {n_lb, n_pairs, n_segs, n_fp};
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
         unsigned long long x = v[i];
@@ -505,17 +612,16 @@ __global__ void __launch_bounds__(TNN_WARPS_PER_CTA * 32)
     unsigned nfb = *(volatile unsigned *)&L.scr->n_fallback3;
     if ((long long)nfb > L.fb_cap)
         nfb = (unsigned)L.fb_cap;
-    const int gw = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const int nw = (gridDim.x * blockDim.x) >> 5;
     const unsigned long long INF64 = 0x7ff0000000000000ull;
     unsigned long long nfp = 0;
-    (void)gw;
-    (void)nw;
-    for (;;) {
-        unsigned e = 0;
-        if (lane == 0)
-            e = atomicAdd(&L.scr->fb_next3, 1u);
-        e = __shfl_sync(FULLMASK, e, 0);
+    // one entry per warp, then the queue (as k_tnn_warp)
+    unsigned e = (threadIdx.x >> 5) * gridDim.x + blockIdx.x;
+    for (bool first = true;; first = false) {
+        if (!first) {
+            if (lane == 0)
+                e = atomicAdd(&L.scr->fb_next3, 1u) + gridDim.x * TNN_WARPS_PER_CTA;
+            e = __shfl_sync(FULLMASK, e, 0);
+        }
         if (e >= nfb)
             break;
         const int2 ent = L.fb_list3[e];

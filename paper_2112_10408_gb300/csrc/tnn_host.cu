@@ -169,6 +169,7 @@ static tnn_status run_mapped(tnn_index *ix, int64_t n, const tnn_knn_params *kp,
         return s;
     L.nwin = 1;
     L.L_max = L.w0.L;
+    L.k_max = L.w0.k;
     L.kseg_max = ix->K;
     L.total_tiles = tnn_window_tiles(ix, &L.w0);
     L.fb_cap = n;

@@ -173,7 +173,7 @@ struct KnnLaunch {
     int64_t total_tiles;
     int64_t tile_lo; // grid order: this launch's tiles [tile_lo, total_tiles)
     int32_t queue;   // and their queue (KnnScratch::tile_counter)
-    int32_t pad3_;
+    int32_t k_max;   // largest k over the windows
     KnnScratch *scr;
     int2 *fb_list;        // (window, query) for the FP32 warp scan
     int2 *fb_list3;       // (window, query) for the exact FP64 warp scan

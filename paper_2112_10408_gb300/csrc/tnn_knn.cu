@@ -154,7 +154,6 @@ static tnn_status device_setup()
             TNN_CUDA_TRY(cudaFuncSetAttribute(grid_kernel(c), cudaFuncAttributeMaxDynamicSharedMemorySize, maxs));
         TNN_CUDA_TRY(cudaFuncSetAttribute(k_linear_search, cudaFuncAttributeMaxDynamicSharedMemorySize, maxs));
         TNN_CUDA_TRY(cudaFuncSetAttribute(k_linear_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, maxs));
-        TNN_CUDA_TRY(cudaFuncSetAttribute(k_tnn_warp, cudaFuncAttributeMaxDynamicSharedMemorySize, maxs));
         TNN_CUDA_TRY(cudaFuncSetAttribute(k_fallback_exact, cudaFuncAttributeMaxDynamicSharedMemorySize, maxs));
         TNN_CUDA_TRY(cudaFuncSetAttribute(k_tnn_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, maxs));
         attrs[dev] = true;
@@ -277,10 +276,11 @@ static tnn_status finish_search(const KnnLaunch &L, cudaStream_t st, bool prof, 
     if (prof)
         TNN_CUDA_TRY(cudaEventRecord(pr.e[1], st));
     {
-        const size_t wsm = wq_smem_per_warp() * TNN_WARPS_PER_CTA;
+        // list registers by the largest k of the launch
+        const TileKernel kern = L.k_max <= 16 ? k_tnn_warp<1> : L.k_max <= 32 ? k_tnn_warp<2> : k_tnn_warp<4>;
         int nbw = 0;
-        TNN_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nbw, k_tnn_warp, TNN_WARPS_PER_CTA * 32, wsm));
-        k_tnn_warp<<<(unsigned)(std::max(nbw, 1) * g_num_sms), TNN_WARPS_PER_CTA * 32, wsm, st>>>(L);
+        TNN_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nbw, kern, TNN_WARPS_PER_CTA * 32, 0));
+        kern<<<(unsigned)(std::max(nbw, 1) * g_num_sms), TNN_WARPS_PER_CTA * 32, 0, st>>>(L);
     }
     TNN_CUDA_TRY(cudaGetLastError());
     if (prof)
@@ -572,6 +572,7 @@ static tnn_status run_single(const tnn_index *ix, const float *d_q, int64_t m,
     cudaStream_t st = (cudaStream_t)stream;
     L.nwin = 1;
     L.L_max = L.w0.L;
+    L.k_max = L.w0.k;
     L.kseg_max = ix->K;
     if (brute)
         L.w0.tile_rows = nullptr; // the linear search gains nothing from trajectory tiles
@@ -774,7 +775,7 @@ extern "C" tnn_status tnn_batch_create(const tnn_index *const *indexes,
         return s;
     std::vector<KnnWin> wins(n_windows);
     long long tiles = 0, fb = 0;
-    int L_max = 0, kseg = 0;
+    int L_max = 0, k_max = 0, kseg = 0;
     // windows by the tile kernel that takes their k; tiles of class c:
     // [cls_tile[c], cls_tile[c + 1])
     std::vector<int> order(n_windows);
@@ -801,6 +802,7 @@ extern "C" tnn_status tnn_batch_create(const tnn_index *const *indexes,
         tiles += tnn_window_tiles(indexes[w], &wins[i]);
         fb += m[w];
         L_max = std::max(L_max, wins[i].L);
+        k_max = std::max(k_max, wins[i].k);
         cls_tile[tnn_k_class(wins[i].k) + 1] = tiles;
         kseg = std::max(kseg, (int)indexes[w]->K);
     }
@@ -825,6 +827,7 @@ extern "C" tnn_status tnn_batch_create(const tnn_index *const *indexes,
     L.wins = b->d_wins;
     L.nwin = n_windows;
     L.L_max = L_max;
+    L.k_max = k_max;
     L.kseg_max = kseg;
     L.total_tiles = tiles;
     L.scr = (KnnScratch *)b->scratch;

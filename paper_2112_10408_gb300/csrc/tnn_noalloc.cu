@@ -75,6 +75,7 @@ extern "C" tnn_status tnn_knn_noalloc(const tnn_index *index, const float *d_q, 
     cudaStream_t st = (cudaStream_t)stream;
     L.nwin = 1;
     L.L_max = L.w0.L;
+    L.k_max = L.w0.k;
     L.kseg_max = index->K;
     L.total_tiles = tnn_window_tiles(index, &L.w0);
     L.fb_cap = m;
