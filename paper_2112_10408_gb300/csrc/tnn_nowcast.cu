@@ -41,61 +41,224 @@ struct FeatNorm {
     float ssq[4];
 };
 
-// One warp per query; lane r handles neighbour ranks r, r + 32.
-__global__ void k_context_features(const float4 *__restrict__ pts,
-                                   const float2 *__restrict__ wind,
-                                   const float4 *__restrict__ q, int64_t m,
-                                   const int32_t *__restrict__ idx,
-                                   const float *__restrict__ d2, int k,
-                                   const __grid_constant__ FeatNorm nrm, float eps,
-                                   uint16_t *__restrict__ feat, float *__restrict__ idw)
+// A warp takes 128 neighbours' worth of queries.  What must be moved is 44 k +
+// 32 B per query of HBM traffic; what kept the kernel from that rate were
+// the passes through the load/store data path: with one query per warp, 15
+// shuffles per query and three 4-byte stores with a 12-byte stride (each
+// sector written in three parts).
+//   k > 16  lane = rank, so a gather instruction reads the neighbours of one
+//           query (runs of consecutive samples of few flights) and the lists
+//           are read in whole lines; 4 queries (2 for k > 32) in flight and
+//           reduced together, each step of the butterfly halving the values
+//           a lane carries (18 shuffles instead of 60); each CTA answers one
+//           run of queries, the next lists on their way meanwhile.
+//   k <= 16 2^lg lanes per query, up to four ranks each.
+// The features leave through shared memory as whole 16-byte words (VEC: k a
+// multiple of 4 and 16-byte aligned features) or 4-byte words of consecutive
+// lanes.  1,000,000 contexts of k = 32: 283 us before, 180 us with 2^lg
+// lanes per query for every k, 169 us now (4.0 TB/s of what must be moved; 3
+// CTAs per SM hold the pipeline's registers, 4 take 173 us and 5 spill).
+#define CF_WARPS 8
+#define CF_CTAS 3 // per SM
+
+// One neighbour: its weight and weighted wind added up, its features as
+// three packed words (zeros for a missing neighbour).
+__device__ __forceinline__ void cf_neighbour(const FeatNorm &nrm, bool on, const float4 &p, const float2 &w,
+                                             const float4 &q, float d2, float eps, float &nu, float &nv,
+                                             float &den, uint32_t (&h)[3])
 {
-    const int64_t qi = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const int lane = threadIdx.x & 31;
-    if (qi >= m)
+    float f[TNN_N_FEAT];
+    if (on) {
+        const float wt = 1.0f / (d2 + eps);
+        nu = fmaf(wt, w.x, nu);
+        nv = fmaf(wt, w.y, nv);
+        den += wt;
+        f[0] = nrm.ssq[0] * (p.x - q.x);
+        f[1] = nrm.ssq[1] * (p.y - q.y);
+        f[2] = nrm.ssq[2] * (p.z - q.z);
+        f[3] = nrm.ssq[3] * (p.w - q.w);
+        f[4] = w.x;
+        f[5] = w.y;
+#pragma unroll
+        for (int c = 0; c < TNN_N_FEAT; ++c)
+            f[c] = (f[c] - nrm.mean[c]) * nrm.inv_std[c];
+    } else {
+#pragma unroll
+        for (int c = 0; c < TNN_N_FEAT; ++c)
+            f[c] = 0.f;
+    }
+#pragma unroll
+    for (int c = 0; c < 3; ++c)
+        h[c] = (uint32_t)f2bf(f[2 * c]) | ((uint32_t)f2bf(f[2 * c + 1]) << 16);
+}
+
+// A warp's feature words from shared memory to its rows.
+template <bool VEC>
+__device__ __forceinline__ void cf_store(const uint32_t *sw, uint32_t *out, int nw, int lane)
+{
+    __syncwarp();
+    if (VEC) {
+        for (int i = lane; i < nw / 4; i += 32)
+            ((uint4 *)out)[i] = ((const uint4 *)sw)[i];
+    } else {
+        for (int i = lane; i < nw; i += 32)
+            out[i] = sw[i];
+    }
+}
+
+__device__ __forceinline__ void cf_idw(float *idw, int64_t qi, float nu, float nv, float den)
+{
+    idw[2 * qi] = den > 0.f ? nu / den : __int_as_float(0x7fffffff);
+    idw[2 * qi + 1] = den > 0.f ? nv / den : __int_as_float(0x7fffffff);
+}
+
+// 16 < k <= 32 R: lane = rank (and rank + 32), 4 / R queries per warp.
+template <int R, bool VEC>
+__global__ void __launch_bounds__(CF_WARPS * 32, CF_CTAS)
+    k_context_features(const float4 *__restrict__ pts, const float2 *__restrict__ wind,
+                       const float4 *__restrict__ q, int64_t m, const int32_t *__restrict__ idx,
+                       const float *__restrict__ d2, int k, const __grid_constant__ FeatNorm nrm, float eps,
+                       uint16_t *__restrict__ feat, float *__restrict__ idw)
+{
+    constexpr int Q = 4 / R;
+    __shared__ __align__(16) uint32_t s_feat[CF_WARPS][128 * 3];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    // A CTA answers one run of consecutive queries, whose neighbours overlap.
+    constexpr int step = CF_WARPS * Q;
+    const int64_t per = (m + (int64_t)gridDim.x * step - 1) / ((int64_t)gridDim.x * step) * step;
+    const int64_t end = min(m, (blockIdx.x + 1) * per);
+    int64_t q0 = blockIdx.x * per + warp * Q;
+    uint32_t *sw = s_feat[warp];
+    int nid[4];
+    float ndd[4];
+    auto fetch = [&](int64_t qa) { // the lists of the queries from qa on
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            const int rank = lane + 32 * (j % R);
+            const bool in = qa + j / R < end && rank < k;
+            nid[j] = in ? __ldg(idx + (qa + j / R) * k + rank) : -1;
+            ndd[j] = in ? __ldg(d2 + (qa + j / R) * k + rank) : 0.f;
+        }
+    };
+    fetch(q0);
+    for (; q0 < end; q0 += step) { // the same for the whole warp
+        const int nq = end - q0 < Q ? (int)(end - q0) : Q;
+        int id[4];
+        float dd[4];
+        float4 p[4];
+        float2 w[4];
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            id[j] = nid[j];
+            dd[j] = ndd[j];
+            if (id[j] >= 0) {
+                p[j] = __ldg(pts + id[j]);
+                w[j] = __ldg(wind + id[j]);
+            }
+        }
+        fetch(q0 + step); // on their way while these are worked on
+        float v[3 * Q];
+#pragma unroll
+        for (int i = 0; i < 3 * Q; ++i)
+            v[i] = 0.f;
+        __syncwarp(); // the previous rows have left shared memory
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            const int qj = j / R, rank = lane + 32 * (j % R);
+            const float4 qq = __ldg(q + (qj < nq ? q0 + qj : q0));
+            uint32_t h[3];
+            cf_neighbour(nrm, id[j] >= 0, p[j], w[j], qq, dd[j], eps, v[3 * qj], v[3 * qj + 1], v[3 * qj + 2],
+                         h);
+            if (feat && rank < k)
+#pragma unroll
+                for (int c = 0; c < 3; ++c)
+                    sw[(qj * k + rank) * 3 + c] = h[c];
+        }
+        if (idw) {
+            // halve the queries a lane carries until one is left, then its sums
+            int mine = 0; // query of this lane's sums
+            int o = 16;
+#pragma unroll
+            for (int hq = Q / 2; hq > 0; hq >>= 1, o >>= 1) {
+                const bool up = (lane & o) != 0;
+#pragma unroll
+                for (int i = 0; i < 3 * hq; ++i) {
+                    const float send = up ? v[i] : v[3 * hq + i], keep = up ? v[3 * hq + i] : v[i];
+                    v[i] = keep + __shfl_xor_sync(FULLMASK, send, o);
+                }
+                mine += up ? hq : 0;
+            }
+#pragma unroll
+            for (; o > 0; o >>= 1)
+#pragma unroll
+                for (int i = 0; i < 3; ++i)
+                    v[i] += __shfl_xor_sync(FULLMASK, v[i], o);
+            if ((lane & (32 / Q - 1)) == 0 && mine < nq)
+                cf_idw(idw, q0 + mine, v[0], v[1], v[2]);
+        }
+        if (feat)
+            cf_store<VEC>(sw, (uint32_t *)(feat + q0 * k * TNN_N_FEAT), nq * k * 3, lane);
+    }
+}
+
+// k <= 16: 2^lg lanes per query, ranks r0 + u 2^lg.
+template <bool VEC>
+__global__ void __launch_bounds__(CF_WARPS * 32, 5)
+    k_context_features_small(const float4 *__restrict__ pts, const float2 *__restrict__ wind,
+                             const float4 *__restrict__ q, int64_t m, const int32_t *__restrict__ idx,
+                             const float *__restrict__ d2, int k, int lg,
+                             const __grid_constant__ FeatNorm nrm, float eps, uint16_t *__restrict__ feat,
+                             float *__restrict__ idw)
+{
+    // (32 >> lg) queries x k neighbours x 3 words, at most 128 neighbours
+    __shared__ __align__(16) uint32_t s_feat[CF_WARPS][128 * 3];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int G = 1 << lg, nq = 32 >> lg, ql = lane >> lg, r0 = lane & (G - 1);
+    const int64_t q0 = ((int64_t)blockIdx.x * CF_WARPS + warp) * nq;
+    if (q0 >= m) // the same for the whole warp
         return;
-    const float4 qq = q[qi];
+    const int64_t qi = q0 + ql;
+    const bool on = qi < m;
+    int id[4] = {-1, -1, -1, -1};
+    float dd[4] = {0.f, 0.f, 0.f, 0.f};
+    const float4 qq = __ldg(q + (on ? qi : q0));
+#pragma unroll
+    for (int u = 0; u < 4; ++u)
+        if (on && r0 + u * G < k) {
+            id[u] = __ldcs(idx + qi * k + r0 + u * G);
+            dd[u] = __ldcs(d2 + qi * k + r0 + u * G);
+        }
+    float4 p[4];
+    float2 w[4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u)
+        if (id[u] >= 0) {
+            p[u] = __ldg(pts + id[u]);
+            w[u] = __ldg(wind + id[u]);
+        }
     float nu = 0.f, nv = 0.f, den = 0.f;
-    for (int r = lane; r < k; r += 32) {
-        const int j = idx[qi * k + r];
-        float f[TNN_N_FEAT];
-        if (j >= 0) {
-            const float4 p = pts[j];
-            const float2 w = wind[j];
-            const float wt = 1.0f / (d2[qi * k + r] + eps);
-            nu = fmaf(wt, w.x, nu);
-            nv = fmaf(wt, w.y, nv);
-            den += wt;
-            f[0] = nrm.ssq[0] * (p.x - qq.x);
-            f[1] = nrm.ssq[1] * (p.y - qq.y);
-            f[2] = nrm.ssq[2] * (p.z - qq.z);
-            f[3] = nrm.ssq[3] * (p.w - qq.w);
-            f[4] = w.x;
-            f[5] = w.y;
+    uint32_t *sw = s_feat[warp];
 #pragma unroll
-            for (int c = 0; c < TNN_N_FEAT; ++c)
-                f[c] = (f[c] - nrm.mean[c]) * nrm.inv_std[c];
-        } else {
+    for (int u = 0; u < 4; ++u) {
+        uint32_t h[3];
+        cf_neighbour(nrm, id[u] >= 0, p[u], w[u], qq, dd[u], eps, nu, nv, den, h);
+        if (feat && r0 + u * G < k)
 #pragma unroll
-            for (int c = 0; c < TNN_N_FEAT; ++c)
-                f[c] = 0.f;
+            for (int c = 0; c < 3; ++c)
+                sw[(ql * k + r0 + u * G) * 3 + c] = h[c];
+    }
+    if (idw) {
+        for (int o = G >> 1; o > 0; o >>= 1) {
+            nu += __shfl_xor_sync(FULLMASK, nu, o);
+            nv += __shfl_xor_sync(FULLMASK, nv, o);
+            den += __shfl_xor_sync(FULLMASK, den, o);
         }
-        if (feat) {
-            uint32_t *o = reinterpret_cast<uint32_t *>(feat + (qi * k + r) * TNN_N_FEAT);
-#pragma unroll
-            for (int c = 0; c < TNN_N_FEAT; c += 2)
-                o[c / 2] = (uint32_t)f2bf(f[c]) | ((uint32_t)f2bf(f[c + 1]) << 16);
-        }
+        if (r0 == 0 && on)
+            cf_idw(idw, qi, nu, nv, den);
     }
-    for (int o = 16; o > 0; o >>= 1) {
-        nu += __shfl_xor_sync(FULLMASK, nu, o);
-        nv += __shfl_xor_sync(FULLMASK, nv, o);
-        den += __shfl_xor_sync(FULLMASK, den, o);
-    }
-    if (lane == 0 && idw) {
-        idw[2 * qi] = den > 0.f ? nu / den : __int_as_float(0x7fffffff);
-        idw[2 * qi + 1] = den > 0.f ? nv / den : __int_as_float(0x7fffffff);
-    }
+    if (feat)
+        cf_store<VEC>(sw, (uint32_t *)(feat + q0 * k * TNN_N_FEAT), (int)(m - q0 < nq ? m - q0 : nq) * k * 3,
+                      lane);
 }
 
 extern "C" tnn_status tnn_context_features(const tnn_index *ix, const float *d_wind,
@@ -126,9 +289,27 @@ extern "C" tnn_status tnn_context_features(const tnn_index *ix, const float *d_w
     for (int i = 0; i < 4; ++i)
         nrm.ssq[i] = (float)sqrt(ix->sigma[i]);
     const float4 *q = d_q ? (const float4 *)d_q : ix->pts;
-    const int64_t threads = m * 32;
-    k_context_features<<<(unsigned)((threads + 255) / 256), 256, 0, (cudaStream_t)stream>>>(
-        ix->pts, (const float2 *)d_wind, q, m, d_idx, d_d2, k, nrm, idw_eps, d_feat, d_idw);
+    const bool vec = k % 4 == 0 && ((uintptr_t)d_feat & 15) == 0;
+    int lg = 0; // k <= 16: 2^lg lanes per query, four neighbours each
+    while (k <= 16 && (4 << lg) < k)
+        ++lg;
+    const int64_t per_cta = (int64_t)CF_WARPS * (k > 32 ? 2 : k > 16 ? 4 : 32 >> lg);
+    int64_t grid = (m + per_cta - 1) / per_cta;
+    if (k > 16) { // persistent: CF_CTAS CTAs per SM
+        int nsm = 0;
+        TNN_CUDA_TRY(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, ix->device));
+        grid = std::min<int64_t>(grid, (int64_t)CF_CTAS * nsm);
+    }
+    const float2 *wind = (const float2 *)d_wind;
+    cudaStream_t st = (cudaStream_t)stream;
+    if (k <= 16) {
+        const auto kern = vec ? k_context_features_small<true> : k_context_features_small<false>;
+        kern<<<(unsigned)grid, CF_WARPS * 32, 0, st>>>(ix->pts, wind, q, m, d_idx, d_d2, k, lg, nrm, idw_eps, d_feat, d_idw);
+    } else {
+        const auto kern = k > 32 ? (vec ? k_context_features<2, true> : k_context_features<2, false>)
+                                 : (vec ? k_context_features<1, true> : k_context_features<1, false>);
+        kern<<<(unsigned)grid, CF_WARPS * 32, 0, st>>>(ix->pts, wind, q, m, d_idx, d_d2, k, nrm, idw_eps, d_feat, d_idw);
+    }
     TNN_CUDA_TRY(cudaGetLastError());
     return TNN_OK;
 }
