@@ -44,9 +44,11 @@
 #define WQ_RSEED 4 // largest radius of the seeding shells
 #endif
 
+typedef Slots<9> WqSlots; // a list holds at most 128 points
+
 struct WarpSmem {
     union {
-        int slot[TG_SLOTS]; // point index of every slot
+        int slot[WqSlots::n]; // point index of every slot
         struct {            // to settle:
             unsigned long long key[128]; // exact keys
             double d64[128];
@@ -195,7 +197,7 @@ __global__ void __launch_bounds__(TNN_WARPS_PER_CTA * 32, TNN_WARP_MINB)
             n_pairs += j >= 0;
             if (!m)
                 return;
-            if (base > TG_SLOTS - 32) {
+            if (base > WqSlots::n - 32) {
                 // renumber the slots the list still holds (at most 32 NR)
                 __syncwarp();
                 S.used[lane] = 0;
@@ -203,7 +205,7 @@ __global__ void __launch_bounds__(TNN_WARPS_PER_CTA * 32, TNN_WARP_MINB)
 #pragma unroll
                 for (int r = 0; r < NR; ++r)
                     if (a[r] != TG_EMPTY)
-                        atomicOr(&S.used[(a[r] & TG_SMASK) >> 5], 1u << (a[r] & 31u));
+                        atomicOr(&S.used[(a[r] & WqSlots::mask) >> 5], 1u << (a[r] & 31u));
                 __syncwarp();
                 const unsigned u = S.used[lane];
                 const int inc = warp_incl_sum(__popc(u), lane);
@@ -212,13 +214,13 @@ __global__ void __launch_bounds__(TNN_WARPS_PER_CTA * 32, TNN_WARP_MINB)
                 __syncwarp();
 #pragma unroll
                 for (int r = 0; r < NR; ++r) {
-                    const unsigned s = a[r] & TG_SMASK;
+                    const unsigned s = a[r] & WqSlots::mask;
                     if (a[r] != TG_EMPTY)
-                        a[r] = (a[r] & ~TG_SMASK) |
+                        a[r] = (a[r] & ~WqSlots::mask) |
                                (unsigned)(S.pre[s >> 5] + __popc(S.used[s >> 5] & ((1u << (s & 31u)) - 1u)));
                 }
 #pragma unroll 1
-                for (int w = 0; w < 32; ++w) {
+                for (int w = 0; w < WqSlots::n / 32; ++w) {
                     const unsigned uw = S.used[w];
                     const int id = S.slot[w * 32 + lane];
                     __syncwarp();
@@ -231,7 +233,7 @@ __global__ void __launch_bounds__(TNN_WARPS_PER_CTA * 32, TNN_WARP_MINB)
             if (in)
                 S.slot[slot] = j;
             base += __popc(m);
-            const unsigned key = in ? tg_key(d, (unsigned)slot) : TG_EMPTY;
+            const unsigned key = in ? WqSlots::key(d, (unsigned)slot) : TG_EMPTY;
             if (__popc(m) <= WQ_INSERT) {
 #pragma unroll 1
                 do {
@@ -249,7 +251,7 @@ __global__ void __launch_bounds__(TNN_WARPS_PER_CTA * 32, TNN_WARP_MINB)
             kc = __shfl_sync(FULLMASK, kc, (C - 1) & 31);
             filled = kc != TG_EMPTY;
             if (kc < TG_INF)
-                tau = fminf(tau, fmaf(tg_upper(kc), 0x1p-12f, tg_upper(kc)) + 0x1p-98f);
+                tau = fminf(tau, fmaf(WqSlots::upper(kc), 0x1p-12f, WqSlots::upper(kc)) + 0x1p-98f);
         };
         // The member segments of every lane's keys ([klo, klo + kn) in key
         // order), 32 segments per step whatever key they belong to.
@@ -451,11 +453,11 @@ __global__ void __launch_bounds__(TNN_WARPS_PER_CTA * 32, TNN_WARP_MINB)
             float bound = tau;
             const unsigned last = __shfl_sync(FULLMASK, a[NR - 1], 31);
             if (last != TG_EMPTY)
-                bound = fminf(bound, tg_lower(last));
+                bound = fminf(bound, WqSlots::lower(last));
             int id[NR], n = 0;
 #pragma unroll
             for (int r = 0; r < NR; ++r) {
-                id[r] = a[r] != TG_EMPTY ? S.slot[a[r] & TG_SMASK] : -1;
+                id[r] = a[r] != TG_EMPTY ? S.slot[a[r] & WqSlots::mask] : -1;
                 n += __popc(__ballot_sync(FULLMASK, id[r] >= 0));
             }
             __syncwarp();

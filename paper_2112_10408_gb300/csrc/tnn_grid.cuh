@@ -8,9 +8,10 @@
 // the exclusion criterion of Sec. 3.4.
 //
 //   near    the segments of the 3 x 3 cells around the tile in the newest
-//           buckets, 32 at a time: every lane's cylinder bounds, then the
-//           segments by ascending bound (over the lanes) while some lane's
-//           bound does not exceed its pruning key (Algorithm 2 fetches the
+//           buckets, 32 at a time, one per lane: by ascending bound over the
+//           whole tile, as far as some lane's pruning key reaches, every
+//           lane's own cylinder bound, and the segment's points if one of
+//           them does not exceed its lane's key (Algorithm 2 fetches the
 //           nearest first).
 //   main    buckets from the causal end backwards; a bucket is visited while
 //           the temporal bound of its running maximum of t_B does not exceed
@@ -74,42 +75,66 @@ __device__ __forceinline__ void reach_cells(float s0, float s1, float R, float o
     c1 = min((int)floorf(fminf(fmaf(s1 + R - o, inv_cell, slack), (float)n)), n - 1);
 }
 
+// Smallest and largest of the warp (NaN only if every lane's is).
 __device__ __forceinline__ float warp_minf(float v)
 {
-    for (int o = 16; o > 0; o >>= 1)
-        v = fminf(v, __shfl_xor_sync(FULLMASK, v, o));
-    return v;
+    float r;
+    asm volatile("redux.sync.min.f32 %0, %1, %2;" : "=f"(r) : "f"(v), "n"(0xffffffff));
+    return r;
 }
 __device__ __forceinline__ float warp_maxf(float v)
 {
-    for (int o = 16; o > 0; o >>= 1)
-        v = fmaxf(v, __shfl_xor_sync(FULLMASK, v, o));
-    return v;
+    float r;
+    asm volatile("redux.sync.max.f32 %0, %1, %2;" : "=f"(r) : "f"(v), "n"(0xffffffff));
+    return r;
+}
+
+// Lower bound on seg_lb of one segment over a group of queries whose scaled
+// x, y lie in [bx0, bx1] x [by0, by1], whose times are at least qt, whose
+// thresholds are at most T32 and lie at least `gap` before them: distance of
+// the two rectangles instead of point and line.
+struct GroupBox {
+    float bx0, bx1, by0, by1, qt, T32, gap, delta;
+};
+__device__ __forceinline__ float box_lb(const GroupBox &g, float st, float4 a, float4 u, float4 b)
+{
+    const float ex = a.x + b.x, ey = a.y + b.y;
+    const float dx = fmaxf(fmaxf(fminf(a.x, ex) - g.bx1, g.bx0 - fmaxf(a.x, ex)), 0.0f);
+    const float dy = fmaxf(fmaxf(fminf(a.y, ey) - g.by1, g.by0 - fmaxf(a.y, ey)), 0.0f);
+    const float a2 = fmaf(dy, dy, dx * dx);
+    const float dist = a2 * rsqrtf(fmaxf(a2, 1e-37f));
+    const float sp = fmaxf(fmaf(dist, 1.0f - 0x1p-20f, -(b.w + g.delta)), 0.0f);
+    const float et = fmaxf(fmaxf(__fsub_rd(g.qt, u.w), g.gap), 0.0f);
+    const float lb = fmaf(sp, sp, (st * et) * et) * (1.0f - 0x1p-18f);
+    return (a.w < g.T32) ? lb : INFINITY;
 }
 
 // ------------------------------------------------- candidate keys, networks
 
-#define TG_SLOT_BITS 10 // point slots of a tile; 14 mantissa bits of the distance remain
-#define TG_SLOTS (1 << TG_SLOT_BITS)
-#define TG_SMASK (TG_SLOTS - 1u)
 #define TG_EMPTY 0xffffffffu // sorts after every key
-#define TG_INF 0xff000000u   // keys of infinite distances
+#define TG_INF 0x7f800000u   // keys of infinite distances
 #define TG_EXTRA 4           // candidates kept beyond the k-th
 #define TG_NB 8        // points sorted at a time
 #define TG_INSERT 1    // batches with at most this many candidates are inserted one by one
                        // (400,000 points: 1 279.8 us, 2 280.0, 3 281.3, 5 285.2)
 #define TG_MIN_GROUP 3       // smaller groups of a tile go to the warp-per-query kernel
 
-// Key of a distance (>= 0) in slot `s`: its bits without the sign, the lowest
-// replaced by the slot.  Keys of one lane order like the distances up to the
-// 2^-14 that the slot displaces.
-__device__ __forceinline__ unsigned tg_key(float d, unsigned s)
-{
-    return ((__float_as_uint(d) << 1) & ~TG_SMASK) | s;
-}
-// Smallest and largest distance a key can stand for.
-__device__ __forceinline__ float tg_lower(unsigned key) { return __uint_as_float((key & ~TG_SMASK) >> 1); }
-__device__ __forceinline__ float tg_upper(unsigned key) { return __uint_as_float((key | TG_SMASK) >> 1); }
+// Key of a distance (>= 0) in a slot: its bits, the lowest SB replaced by the
+// slot.  Keys of one lane order like the distances up to the 2^(SB - 23) that
+// the slot displaces.
+template <int SB> struct Slots {
+    static constexpr int n = 1 << SB;
+    static constexpr unsigned mask = n - 1u;
+    static __device__ __forceinline__ unsigned key(float d, unsigned s)
+    {
+        return (__float_as_uint(d) & ~mask) | s;
+    }
+    // smallest and largest distance a key can stand for
+    static __device__ __forceinline__ float lower(unsigned key) { return __uint_as_float(key & ~mask); }
+    static __device__ __forceinline__ float upper(unsigned key) { return __uint_as_float(key | mask); }
+};
+// 512 slots; 1024 for the longest lists, whose tiles hold more points
+template <int NL> using TileSlots = Slots<(NL > 32 ? 10 : 9)>;
 
 __device__ __forceinline__ void tg_cmpx(unsigned &a, unsigned &b)
 {
@@ -200,8 +225,8 @@ __device__ __forceinline__ void tg_insert(unsigned (&a)[NL], unsigned (&o)[TG_EX
 // ------------------------------------------------------------ shared memory
 
 // Per warp.  While points are gathered: the batch's points, staged segments,
-// their bounds (upper halves of the floats), the slots in use and their
-// prefix, the key ranges' ends and offsets; the slot table behind them.  To
+// the slots in use and their prefix, the key ranges' ends and offsets; the
+// slot table behind them.  To
 // settle, the lists' 32-bit keys take the first part's place, and then the
 // 64-bit lists [NL + TG_EXTRA + 1][32] everything's.
 template <int NL> struct TileSmem {
@@ -209,15 +234,14 @@ template <int NL> struct TileSmem {
         struct {
             float4 pts[32];
             float4 seg[32][3];
-            uint16_t lb[32][32];
-            unsigned used[32];
+            unsigned used[32]; // one word per 32 slots
             int pre[32];
             int kend[32];
             int krel[32];
         };
         unsigned raw[NL + TG_EXTRA][32];
     };
-    int slot[TG_SLOTS];
+    int slot[TileSlots<NL>::n];
 };
 
 template <int NL> __host__ __device__ constexpr size_t tg_smem_per_warp()
@@ -327,6 +351,7 @@ template <int NL>
 __global__ void __launch_bounds__(TNN_WARPS_PER_CTA * 32, TileCtas<NL>::value)
     k_tnn_grid_search(const __grid_constant__ KnnLaunch L)
 {
+    using SL = TileSlots<NL>;
     constexpr int NB = NL < TG_NB ? NL : TG_NB; // points per network batch
     extern __shared__ __align__(16) unsigned char smem[];
     const int lane = threadIdx.x & 31;
@@ -388,6 +413,9 @@ __global__ void __launch_bounds__(TNN_WARPS_PER_CTA * 32, TileCtas<NL>::value)
         const float bx1 = warp_maxf(act ? c.sx : -INFINITY);
         const float by0 = warp_minf(act ? c.sy : INFINITY);
         const float by1 = warp_maxf(act ? c.sy : -INFINITY);
+        const GroupBox box = {bx0, bx1, by0, by1, warp_minf(act ? c.qt : INFINITY), tmax,
+                              warp_minf(act ? __fsub_rd(c.qt, c.T32) : INFINITY),
+                              warp_maxf(act ? c.delta : 0.0f)};
         int bhi = -1;
         {
             const float fb = (tmax - G.t0) * G.inv_dt;
@@ -413,7 +441,8 @@ __global__ void __launch_bounds__(TNN_WARPS_PER_CTA * 32, TileCtas<NL>::value)
         bool deferred = false;
 
         int base = 0, fill = 0, myidx = 0; // next slot; points gathered so far, this lane's
-        int b = bhi + 1, t0 = 0, ncells = 0, cx0 = 0, cy0 = 0, wx = 1; // main phase
+        // main phase: next bucket, buckets of the present group, their cells
+        int b = bhi, gb = 0, t0 = 0, ncells = 0, cx0 = 0, cy0 = 0, wx = 1, nc = 1;
         bool near_phase = true;
         int total = 0, pos = 0; // segments of the present key group, handled so far
 
@@ -466,10 +495,14 @@ __global__ void __launch_bounds__(TNN_WARPS_PER_CTA * 32, TileCtas<NL>::value)
                     if (fill > 0) {
                         flush = true;
                     } else {
-                        if (--b < 0)
+                        // the next buckets, as many as give 32 cells: their
+                        // records are one round of reads
+                        b -= gb;
+                        if (b < 0)
                             break;
-                        const bool done =
-                            !act || deferred || !(time_lb(c, s3, __ldg(G.bpm + b)) <= tau);
+                        const float bp = __ldg(G.bpm + max(b - lane, 0));
+                        const float tl = time_lb(c, s3, __shfl_sync(FULLMASK, bp, 0));
+                        const bool done = !act || deferred || !(tl <= tau);
                         if (__all_sync(FULLMASK, done))
                             break;
                         lim = done ? -1.0f : tau;
@@ -479,28 +512,40 @@ __global__ void __launch_bounds__(TNN_WARPS_PER_CTA * 32, TileCtas<NL>::value)
                         cy0 = 0;
                         if (tmx < INFINITY) {
                             // any key outside this reach has a bound above every key
-                            const float R = sqrtf(tmx) * (1.0f + 0x1p-18f) + ext_max +
-                                            warp_maxf(act ? c.delta : 0.0f);
+                            const float R = sqrtf(tmx) * (1.0f + 0x1p-18f) + ext_max + box.delta;
                             reach_cells(bx0, bx1, R, G.x0, G.inv_cell, G.nx, cx0, cx1);
                             reach_cells(by0, by1, R, G.y0, G.inv_cell, G.ny, cy0, cy1);
                         }
                         wx = cx1 - cx0 + 1;
-                        ncells = wx * (cy1 - cy0 + 1);
+                        nc = max(wx, 0) * max(cy1 - cy0 + 1, 0);
+                        if (nc == 0)
+                            break; // no cell within reach
+                        const int most = min(b + 1, 32 / nc);
+#pragma unroll 1
+                        for (gb = 1; gb < most; ++gb) {
+                            const float tg = time_lb(c, s3, __shfl_sync(FULLMASK, bp, gb));
+                            if (!__any_sync(FULLMASK, !done && tg <= tau))
+                                break;
+                        }
+                        ncells = nc * gb;
                         t0 = 0;
                         continue;
                     }
                 } else {
-                    // up to 32 cells of bucket b: the keys some lane needs
+                    // up to 32 cells of the group: the keys some lane needs
                     const int t = t0 + lane;
                     t0 += 32;
                     int klo = 0, kn = 0, cx = 0, cy = 0;
                     float ex = 0.f, tk = 0.f;
                     if (t < ncells) {
-                        cx = cx0 + t % wx;
-                        cy = cy0 + t / wx;
-                        const bool staged = b > bhi - TNN_SEED_BUCKETS && abs(cx - hx) <= 1 && abs(cy - hy) <= 1;
+                        // quotients of integers below 2^21: exact
+                        const int db = (int)(((float)t + 0.5f) * (1.0f / (float)nc)), rem = t - db * nc;
+                        const int dy = (int)(((float)rem + 0.5f) * (1.0f / (float)wx));
+                        cx = cx0 + rem - dy * wx;
+                        cy = cy0 + dy;
+                        const bool staged = b - db > bhi - TNN_SEED_BUCKETS && abs(cx - hx) <= 1 && abs(cy - hy) <= 1;
                         if (!staged) {
-                            const int4 kr = __ldg(G.krec + (b * G.ncell + cy * G.nx + cx));
+                            const int4 kr = __ldg(G.krec + ((b - db) * G.ncell + cy * G.nx + cx));
                             klo = kr.x;
                             kn = kr.y - kr.x;
                             ex = __int_as_float(kr.z);
@@ -524,9 +569,10 @@ __global__ void __launch_bounds__(TNN_WARPS_PER_CTA * 32, TileCtas<NL>::value)
                 }
             }
 
-            // ---- the next (up to 32) segments of the group: bounds of every lane
+            // ---- the next (up to 32) segments of the key group, one per lane,
+            // by their bound over the whole query group
             int sfirst = 0, scnt = 0;
-            unsigned score = TG_EMPTY; // lane j: smallest bound of segment j over the lanes
+            unsigned score = TG_EMPTY; // that bound above the lane
             if (cnt > 0) {
                 __syncwarp();
                 if (lane < cnt) {
@@ -541,47 +587,36 @@ __global__ void __launch_bounds__(TNN_WARPS_PER_CTA * 32, TileCtas<NL>::value)
                             lo = mid + 1;
                     }
                     const float4 *r = G.gseg + 4 * (size_t)(S.krel[lo] + g);
-                    S.seg[lane][0] = __ldg(r);
-                    S.seg[lane][1] = __ldg(r + 1);
-                    S.seg[lane][2] = __ldg(r + 2);
-                    const float4 r3 = __ldg(r + 3);
+                    const float4 ra = __ldg(r), ru = __ldg(r + 1), rb = __ldg(r + 2), r3 = __ldg(r + 3);
+                    S.seg[lane][0] = ra;
+                    S.seg[lane][1] = ru;
+                    S.seg[lane][2] = rb;
                     sfirst = __float_as_int(r3.x);
                     scnt = __float_as_int(r3.y);
+                    const float lb = box_lb(box, s3, ra, ru, rb);
+                    if (lb < INFINITY) // truncated towards zero: still a bound
+                        score = (__float_as_uint(lb) & ~31u) | (unsigned)lane;
                 }
                 pos += cnt;
                 __syncwarp();
-                // two per step (their chains overlap); an odd count's last
-                // partner is a stale record whose bound is not used
-#pragma unroll 1
-                for (int i = 0; i < cnt; i += 2) {
-#pragma unroll
-                    for (int u = 0; u < 2; ++u) {
-                        const float lb = seg_lb(c, s3, S.seg[i + u][0], S.seg[i + u][1], S.seg[i + u][2]);
-                        // the upper half of a non-negative float is a lower bound of it
-                        const unsigned h = __float_as_uint(lb) >> 16;
-                        S.lb[i + u][lane] = (uint16_t)h;
-                        const unsigned m = __reduce_min_sync(FULLMASK, lb <= lim ? h : 0xffffu);
-                        if (lane == i + u && lane < cnt && m != 0xffffu)
-                            score = (m << 5) | (unsigned)lane;
-                    }
-                }
-                if (act)
-                    n_lb += cnt;
-                __syncwarp();
             }
 
-            // ---- their points, 32 at a time, nearest segments first
+            // ---- their points, 32 at a time: nearest segments first, while
+            // some query's own bound allows
             int lf = 0, lc = 0; // points left of the segment taken last
+            float most = warp_maxf(lim);
             for (;;) {
                 while (fill < 32) {
                     if (lc == 0) {
                         const unsigned best = __reduce_min_sync(FULLMASK, score);
-                        if (best == TG_EMPTY)
+                        if (best == TG_EMPTY || !(__uint_as_float(best & ~31u) <= most))
                             break;
                         const int j = best & 31u;
                         if (lane == j)
                             score = TG_EMPTY;
-                        if (!__any_sync(FULLMASK, __uint_as_float((unsigned)S.lb[j][lane] << 16) <= lim))
+                        const float lb = seg_lb(c, s3, S.seg[j][0], S.seg[j][1], S.seg[j][2]);
+                        n_lb += act;
+                        if (!__any_sync(FULLMASK, lb <= lim))
                             continue;
                         lf = __shfl_sync(FULLMASK, sfirst, j);
                         lc = __shfl_sync(FULLMASK, scnt, j);
@@ -595,7 +630,7 @@ __global__ void __launch_bounds__(TNN_WARPS_PER_CTA * 32, TileCtas<NL>::value)
                 }
                 if (fill == 0 || (fill < 32 && !flush))
                     break;
-                if (base > TG_SLOTS - 32) {
+                if (base > SL::n - 32) {
                     // renumber the slots that some list still holds
                     __syncwarp();
                     S.used[lane] = 0;
@@ -610,7 +645,7 @@ __global__ void __launch_bounds__(TNN_WARPS_PER_CTA * 32, TileCtas<NL>::value)
 #pragma unroll 1
                     for (int i = 0; i < NL + TG_EXTRA; ++i)
                         if (t[i] != TG_EMPTY)
-                            atomicOr(&S.used[(t[i] & TG_SMASK) >> 5], 1u << (t[i] & 31u));
+                            atomicOr(&S.used[(t[i] & SL::mask) >> 5], 1u << (t[i] & 31u));
                     __syncwarp();
                     const unsigned u = S.used[lane];
                     int inc = __popc(u);
@@ -625,9 +660,9 @@ __global__ void __launch_bounds__(TNN_WARPS_PER_CTA * 32, TileCtas<NL>::value)
                     __syncwarp();
 #pragma unroll 1
                     for (int i = 0; i < NL + TG_EXTRA; ++i) {
-                        const unsigned v = t[i], s = v & TG_SMASK;
+                        const unsigned v = t[i], s = v & SL::mask;
                         if (v != TG_EMPTY)
-                            t[i] = (v & ~TG_SMASK) |
+                            t[i] = (v & ~SL::mask) |
                                    (unsigned)(S.pre[s >> 5] + __popc(S.used[s >> 5] & ((1u << (s & 31u)) - 1u)));
                     }
 #pragma unroll
@@ -637,7 +672,7 @@ __global__ void __launch_bounds__(TNN_WARPS_PER_CTA * 32, TileCtas<NL>::value)
                     for (int i = 0; i < TG_EXTRA; ++i)
                         o[i] = t[NL + i];
 #pragma unroll 1
-                    for (int w = 0; w < 32; ++w) {
+                    for (int w = 0; w < SL::n / 32; ++w) {
                         const unsigned uw = S.used[w];
                         const int id = S.slot[w * 32 + lane];
                         __syncwarp();
@@ -645,7 +680,7 @@ __global__ void __launch_bounds__(TNN_WARPS_PER_CTA * 32, TileCtas<NL>::value)
                             S.slot[S.pre[w] + __popc(uw & ((1u << lane) - 1u))] = id;
                         __syncwarp();
                     }
-                    if (base > TG_SLOTS - 32) {
+                    if (base > SL::n - 32) {
                         given_up = true;
                         break;
                     }
@@ -677,7 +712,7 @@ __global__ void __launch_bounds__(TNN_WARPS_PER_CTA * 32, TileCtas<NL>::value)
                         const float4 p = S.pts[s + i];
                         const float d = dist32(c, s0, s1, s2, s3, p);
                         const bool in = p.w < c.T32 && d <= tau;
-                        v[i] = in ? tg_key(d, (unsigned)(base + s + i)) : TG_EMPTY;
+                        v[i] = in ? SL::key(d, (unsigned)(base + s + i)) : TG_EMPTY;
                         mine |= in ? 1u << i : 0u;
                     }
                     unsigned any = __reduce_or_sync(FULLMASK, mine);
@@ -691,7 +726,7 @@ __global__ void __launch_bounds__(TNN_WARPS_PER_CTA * 32, TileCtas<NL>::value)
                             any &= any - 1;
                             const float4 p = S.pts[s + i];
                             const float d = dist32(c, s0, s1, s2, s3, p);
-                            const unsigned key = (mine >> i) & 1u ? tg_key(d, (unsigned)(base + s + i)) : TG_EMPTY;
+                            const unsigned key = (mine >> i) & 1u ? SL::key(d, (unsigned)(base + s + i)) : TG_EMPTY;
                             tg_insert<NL>(a, o, key);
                         }
                     } else {
@@ -699,11 +734,12 @@ __global__ void __launch_bounds__(TNN_WARPS_PER_CTA * 32, TileCtas<NL>::value)
                         tg_merge<NL, NB>(a, o, v);
                     }
                     if (a[NL - 1] < TG_INF)
-                        tau = fmaf(tg_upper(a[NL - 1]), 0x1p-12f, tg_upper(a[NL - 1])) + 0x1p-98f;
+                        tau = fmaf(SL::upper(a[NL - 1]), 0x1p-12f, SL::upper(a[NL - 1])) + 0x1p-98f;
                     lim = fminf(lim, tau);
                 }
                 base += kept ? 32 : 0;
                 fill = 0;
+                most = warp_maxf(lim);
             }
             if (given_up)
                 break;
@@ -715,7 +751,7 @@ __global__ void __launch_bounds__(TNN_WARPS_PER_CTA * 32, TileCtas<NL>::value)
             deferred = act;
         if (deferred) {
             const float hand = !given_up && W->L <= k + TG_EXTRA && o[TG_EXTRA - 1] != TG_EMPTY
-                                   ? tg_upper(o[TG_EXTRA - 1])
+                                   ? SL::upper(o[TG_EXTRA - 1])
                                    : INFINITY;
             const unsigned slot = atomicAdd(&L.scr->n_fallback, 1u);
             if (slot < (unsigned long long)L.fb_cap) {
@@ -731,7 +767,7 @@ __global__ void __launch_bounds__(TNN_WARPS_PER_CTA * 32, TileCtas<NL>::value)
         float bound = INFINITY;
         bool ok = a[NL - 1] < TG_INF || a[NL - 1] == TG_EMPTY; // else distances overflowed
         if (a[NL - 1] < TG_INF)
-            bound = o[TG_EXTRA - 1] != TG_EMPTY ? fminf(tg_lower(o[TG_EXTRA - 1]), tau) : tau;
+            bound = o[TG_EXTRA - 1] != TG_EMPTY ? fminf(SL::lower(o[TG_EXTRA - 1]), tau) : tau;
         __syncwarp();
 #pragma unroll
         for (int i = 0; i < NL; ++i)
@@ -744,40 +780,33 @@ __global__ void __launch_bounds__(TNN_WARPS_PER_CTA * 32, TileCtas<NL>::value)
 #pragma unroll 4
         for (int e = z; e < NL + TG_EXTRA; ++e) {
             const unsigned v = S.raw[e][lane];
-            S.raw[e][lane] = settle && v != TG_EMPTY ? (unsigned)S.slot[v & TG_SMASK] : TG_EMPTY;
+            S.raw[e][lane] = settle && v != TG_EMPTY ? (unsigned)S.slot[v & SL::mask] : TG_EMPTY;
         }
         {
             // Exact keys, from the last row down: 64-bit row e covers 32-bit
             // rows 2 e and 2 e + 1, which every lane has read by then.
+            // `slow`: some entry is not certainly below its successor (a little
+            // more than the margin of the settlement, so that a plain
+            // comparison will do: missing entries are infinite).
             bool slow = (W->flags & TNN_FLAG_EXACT_D2) != 0;
-            unsigned long long next = SENT;
+            float dn = INFINITY;
 #pragma unroll 1
             for (int e = NL + TG_EXTRA - 1; e >= z; e -= 2) {
-                // two rows per step; row z - 1 is a zero row or absent (e0 = z)
-                const int e1 = max(e - 1, z);
+                const int e1 = max(e - 1, z); // two rows per step, the last may be one
                 const unsigned i0 = S.raw[e][lane], i1 = S.raw[e1][lane];
                 __syncwarp();
                 const float4 p0 = __ldg(pts + (i0 != TG_EMPTY ? i0 : 0u));
                 const float4 p1 = __ldg(pts + (i1 != TG_EMPTY ? i1 : 0u));
-                const unsigned long long k0 =
-                    i0 != TG_EMPTY ? pack_key(dist32(c, s0, s1, s2, s3, p0), (int)i0) : SENT;
-                const unsigned long long k1 =
-                    i1 != TG_EMPTY ? pack_key(dist32(c, s0, s1, s2, s3, p1), (int)i1) : SENT;
-                *tg_entry(Kw, e, lane) = k0;
-                *tg_entry(Kw, e1, lane) = k1;
-                slow |= next < k0 || (e1 < e && k0 < k1);
-                const float d0 = key_d(k0), d1 = key_d(k1);
-                if (e < NL && next != SENT)
-                    slow |= key_d(next) <= fmaf(d0, 0x1p-17f, d0) + 0x1p-100f;
-                if (e1 < NL && e1 < e && k0 != SENT)
-                    slow |= d0 <= fmaf(d1, 0x1p-17f, d1) + 0x1p-100f;
-                if (e1 == NL - 1 || e == NL - 1) {
-                    const float dk = e == NL - 1 ? d0 : d1;
-                    if (dk < INFINITY)
-                        slow |= bound <= fmaf(dk, 0x1p-17f, dk) + 0x1p-100f;
-                }
-                next = k1;
+                const float d0 = i0 != TG_EMPTY ? dist32(c, s0, s1, s2, s3, p0) : INFINITY;
+                const float d1 = i1 != TG_EMPTY ? dist32(c, s0, s1, s2, s3, p1) : INFINITY;
+                *tg_entry(Kw, e, lane) = pack_key(d0, (int)i0); // (infinity, -1) is SENT
+                *tg_entry(Kw, e1, lane) = pack_key(d1, (int)i1);
+                slow |= dn < fmaf(d0, 0x1.1p-17f, d0) + 0x1p-99f;
+                slow |= e1 < e && d0 < fmaf(d1, 0x1.1p-17f, d1) + 0x1p-99f;
+                dn = d1;
             }
+            const float dk = key_d(*tg_entry(Kw, NL - 1, lane));
+            slow |= bound < fmaf(dk, 0x1.1p-17f, dk) + 0x1p-99f;
             if (settle && ok && slow) {
                 const unsigned r = tg_settle(W, q, Kw, lane, z, k + TG_EXTRA, bound);
                 ok = r & 1u;
