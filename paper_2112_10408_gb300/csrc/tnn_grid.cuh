@@ -37,7 +37,14 @@
 // the batch: straight-line code for 32 points a time executes the fewest
 // instructions but streams its code (459 us, over half of the stall cycles
 // waiting for instructions), 16 take 306 and 8 take 284 us; for the same
-// reason everything done once per tile is rolled into short loops.
+// reason everything done once per tile is rolled into short loops.  Bounding a
+// segment over the whole tile first, one segment per lane, and per lane only
+// when its turn comes (every lane's bound of every staged segment before: 47
+// of them per query at 400,000 points), and reading the key records of as many
+// buckets as fill a warp took these three figures from 280, 3,016 and 79 us to
+// 232, 2,669 and 44 us.  (Dropping single points by their distance to the
+// tile's rectangle before the lanes score them costs more than it saves: 251
+// against 234 us.)
 #pragma once
 #include "tnn_device.cuh"
 
@@ -339,9 +346,11 @@ static __device__ const unsigned char tg_seed_cell[32] = {
     5,  21, 4,  6,  1,  9,  20, 22, 17, 25, 0,  2,  8,  10, 16, 18, 24, 26, 37, 36, 38, 33, 41, 32, 34, 40, 42,
     0,  0,  0,  0,  0};
 
-// CTAs per SM: the list's registers (list + batch) set it.
+// CTAs per SM: the list's registers (list + batch) set it.  400,000 points, k
+// = 32: 3 CTAs 244.5 us, 4 234.2, 5 263.2 (spills); 10,000 points, k = 8: 5
+// 41.5, 6 43.6; mixed windows with k = 64: 2 1,311, 3 1,304, 4 1,391.
 template <int NL> struct TileCtas {
-    static constexpr int value = NL == 64 ? 3 : NL == 32 ? 4 : 6;
+    static constexpr int value = NL == 64 ? 3 : NL == 32 ? 4 : 5;
 };
 
 // The grid-order tile kernel for k <= NL.  A list shorter than NL keys holds

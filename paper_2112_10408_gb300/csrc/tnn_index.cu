@@ -754,13 +754,16 @@ static float host_ord2f(uint32_t u)
 // (it holds every segment midpoint up to rounding, and keys are clamped to
 // the grid), their time range and the summed segment duration.  Buckets span
 // about five mean segment durations (at most 4096 of them); cells are square,
-// about one segment per (bucket, cell) on average, at most 65,536 cells and
-// 2^22 keys.
+// 0.8 of them per segment of a bucket on average, at most 65,536 cells and
+// 2^22 keys.  (Tile + per-query kernels, us, at 1.0 / 0.8 / 0.7 cells per
+// segment: 400,000 flight samples 277 / 277 / 280, 1 M random walks 540 / 531
+// / 542, 4 M samples 3,020 / 2,878 / 2,827, a half-hour-lag nowcast of 185,376
+// 412 / 361 / 340; 2 cells defer more queries than they save: 4 M 4,300.)
 #ifndef TNN_BUCKET_SEGS
 #define TNN_BUCKET_SEGS 5.0 // bucket span in mean segment durations
 #endif
 #ifndef TNN_KEY_SEGS
-#define TNN_KEY_SEGS 1.0 // mean segments per (bucket, cell)
+#define TNN_KEY_SEGS 0.8 // cells per mean segment of a bucket
 #endif
 static GridBuild grid_geometry(double xmn, double xmx, double ymn, double ymx, double tmn,
                                double tmx, double dur, int64_t S)
