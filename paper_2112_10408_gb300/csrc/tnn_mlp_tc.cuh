@@ -1,7 +1,8 @@
 // The MLP of the learned nowcaster on the tensor cores (tcgen05, kind::f16
 // with BF16 operands, FP32 accumulation in TMEM).
 //
-// k_mlp_fwd_tc — one CTA of 128 threads per 128 rows of the batch:
+// k_mlp_fwd_tc — one CTA, or a cluster of 2, 4 or 8 CTAs that share the
+// hidden units, per 128 rows of the batch:
 //   Z = X W1 + b1 with X [B, d_in] (A operand, rows of the batch) and W1
 //   kept transposed in the UMMA core-matrix order (B operand, one 16-column
 //   K step = dh rows x 32 B, moved by one bulk copy).  The K loop is double
@@ -11,13 +12,23 @@
 //   dZ = (dY W2^T) * GELU'(Z) (written transposed for the dW1 product, as is
 //   X), the squared error, and the per-CTA column sums that give db1, dW2 and
 //   db2 (warp reduce-scatter, then the 4 warps' rows summed in a fixed order,
-//   so that training is deterministic).
+//   so that training is deterministic).  The epilogue (about 55 instructions
+//   per row and hidden unit when training) bounds it, and a batch of 4,096
+//   has only 32 tiles of rows for 152 SMs: with a cluster every CTA takes 1 /
+//   C of the hidden units, the partial heads are exchanged through distributed
+//   shared memory (summed in rank order) and each CTA goes on with its own
+//   columns.  4,096 rows, 192 -> 256 (cold caches): 27 us by 32 CTAs, 19 us by
+//   128; the gradient as a whole, back to back, 48 -> 38 us.
 // k_mlp_dw1_tc — dW1^T = dZ^T X over the batch: one CTA per (128 hidden
 //   units, up to 256 inputs, batch slice); both operands are read K-major
 //   from the transposed copies; the partial products of the batch slices are
 //   summed by the AdamW kernel.
 #pragma once
+#include <cooperative_groups.h>
+
 #include "tnn_tc.cuh"
+
+namespace cg = cooperative_groups;
 
 #define MLP_ROWS 128
 
@@ -71,6 +82,7 @@ struct MlpFwdArgs {
     uint32_t tmem_cols;
     int *err;            // set when a device wait timed out
     int resident;        // 1: all K steps of X and W1^T staged at once (mlp_fwd_smem_res)
+    int csize;           // CTAs per cluster (training; 1: no cluster)
 };
 
 #define MLP_FWD_THREADS 256 // two warps per TMEM lane quadrant, one per half of the hidden units
@@ -114,7 +126,10 @@ __global__ void __launch_bounds__(MLP_FWD_THREADS, 2) k_mlp_fwd_tc(const __grid_
     const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
     const int quad = warp & 3, half = warp >> 2; // TMEM lane quadrant, hidden-unit half
     const int rr = t & (MLP_ROWS - 1);           // row of the tile (= TMEM lane)
-    const int dh = a.dh, nk = a.d_in / 16, hh = dh / 2;
+    // hidden units [h0, h0 + dh) of this CTA
+    const int C = a.csize, crank = C > 1 ? (int)(blockIdx.x % (unsigned)C) : 0;
+    const int dh = a.dh / C, h0 = crank * dh, nk = a.d_in / 16, hh = dh / 2;
+    const uint16_t *w1t = a.w1t + (size_t)h0 * 16; // K step s: rows from h0 on
     const size_t bstage = (size_t)dh * 32;
     const int nst = a.resident ? nk : 4;        // K-step stages in shared memory
     unsigned char *sA = smem;                   // [nst][4096]
@@ -128,7 +143,7 @@ __global__ void __launch_bounds__(MLP_FWD_THREADS, 2) k_mlp_fwd_tc(const __grid_
     uint32_t *tmem_slot = (uint32_t *)(bars + 8);
     const uint32_t bar_full0 = su32(bars), bar_mma0 = su32(bars + 4); // [4] each
     volatile int *s_err = (volatile int *)(tmem_slot + 1);
-    const long long row0 = (long long)blockIdx.x * MLP_ROWS;
+    const long long tile = blockIdx.x / (unsigned)C, row0 = tile * MLP_ROWS;
     const long long r = row0 + rr;
     const long long Bp = (a.B + 15) & ~15ll;
     const bool valid = r < a.B;
@@ -145,22 +160,22 @@ __global__ void __launch_bounds__(MLP_FWD_THREADS, 2) k_mlp_fwd_tc(const __grid_
                          ::"r"(bar_full0), "r"((uint32_t)(bstage * nk))
                          : "memory");
             for (int s = 0; s < nk; ++s)
-                tma_copy_1d(su32(sB + s * bstage), a.w1t + (size_t)s * dh * 16, (uint32_t)bstage, bar_full0);
+                tma_copy_1d(su32(sB + s * bstage), w1t + (size_t)s * a.dh * 16, (uint32_t)bstage, bar_full0);
         } else {
             // W1^T slices of the first two K steps
             for (int s = 0; s < 2 && s < nk; ++s) {
                 asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;"
                              ::"r"(bar_full0 + 8u * s), "r"((uint32_t)bstage)
                              : "memory");
-                tma_copy_1d(su32(sB + s * bstage), a.w1t + (size_t)s * dh * 16, (uint32_t)bstage,
+                tma_copy_1d(su32(sB + s * bstage), w1t + (size_t)s * a.dh * 16, (uint32_t)bstage,
                             bar_full0 + 8u * s);
             }
         }
     }
     for (int i = t; i < dh; i += MLP_FWD_THREADS) {
-        s_b1[i] = a.b1[i];
-        s_W2[2 * i] = a.W2[2 * i];
-        s_W2[2 * i + 1] = a.W2[2 * i + 1];
+        s_b1[i] = a.b1[h0 + i];
+        s_W2[2 * i] = a.W2[2 * (h0 + i)];
+        s_W2[2 * i + 1] = a.W2[2 * (h0 + i) + 1];
     }
     for (int i = t; i < 4 * ncol; i += MLP_FWD_THREADS)
         s_col[i] = 0.0f;
@@ -183,7 +198,7 @@ __global__ void __launch_bounds__(MLP_FWD_THREADS, 2) k_mlp_fwd_tc(const __grid_
             const uint4 x = valid ? __ldg((const uint4 *)(a.X + r * a.d_in + s * 16 + half * 8))
                                   : make_uint4(0, 0, 0, 0);
             *(uint4 *)(sA + (size_t)s * 4096 + kmaj_off_bf16(rr, half * 8)) = x;
-            if (train && r < Bp) {
+            if (train && r < Bp && s % C == crank) {
                 const uint16_t *xs = (const uint16_t *)&x;
 #pragma unroll
                 for (int j = 0; j < 8; ++j)
@@ -242,7 +257,7 @@ __global__ void __launch_bounds__(MLP_FWD_THREADS, 2) k_mlp_fwd_tc(const __grid_
                 asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;"
                              ::"r"(bar_full0 + 8u * st2), "r"((uint32_t)bstage)
                              : "memory");
-                tma_copy_1d(su32(sB + st2 * bstage), a.w1t + (size_t)s2 * dh * 16, (uint32_t)bstage,
+                tma_copy_1d(su32(sB + st2 * bstage), w1t + (size_t)s2 * a.dh * 16, (uint32_t)bstage,
                             bar_full0 + 8u * st2);
             }
             uint4 x = xq[0];
@@ -251,7 +266,7 @@ __global__ void __launch_bounds__(MLP_FWD_THREADS, 2) k_mlp_fwd_tc(const __grid_
                 if ((s & 7) == i)
                     x = xq[i];
             *(uint4 *)(sA + st * 4096 + kmaj_off_bf16(rr, half * 8)) = x;
-            if (train && r < Bp) {
+            if (train && r < Bp && s % C == crank) {
                 // X^T for the dW1 product (zeros pad the batch to 16)
                 const uint16_t *xs = (const uint16_t *)&x;
 #pragma unroll
@@ -288,11 +303,11 @@ __global__ void __launch_bounds__(MLP_FWD_THREADS, 2) k_mlp_fwd_tc(const __grid_
         }
     }
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+    const uint32_t trow = tmem + ((uint32_t)(quad * 32) << 16);
+    const int c0 = half * hh, c1 = c0 + hh;
+    float y0 = 0.f, y1 = 0.f;
     if (ok) {
-        const uint32_t trow = tmem + ((uint32_t)(quad * 32) << 16);
-        const int c0 = half * hh, c1 = c0 + hh;
         // ---- pass 1: H = bf16(GELU(Z + b1)), partial head over this half
-        float y0 = 0.f, y1 = 0.f;
         for (int c = c0; c < c1; c += 32) {
             uint32_t v[32];
             tmem_ld32_nowait(trow + (uint32_t)c, v);
@@ -320,10 +335,27 @@ __global__ void __launch_bounds__(MLP_FWD_THREADS, 2) k_mlp_fwd_tc(const __grid_
         }
         s_y[(half * MLP_ROWS + rr) * 2] = y0;
         s_y[(half * MLP_ROWS + rr) * 2 + 1] = y1;
+    }
+    // the partial heads of the cluster's CTAs, in rank order; every CTA gets
+    // here, also after a failed wait
+    if (C > 1) {
+        cg::cluster_group cluster = cg::this_cluster();
+        cluster.sync();
+        y0 = y1 = 0.f;
+        for (int i = 0; i < C; ++i) {
+            const float *py = cluster.map_shared_rank(s_y, i);
+            y0 += py[rr * 2] + py[(MLP_ROWS + rr) * 2];
+            y1 += py[rr * 2 + 1] + py[(MLP_ROWS + rr) * 2 + 1];
+        }
+    } else {
         __syncthreads();
-        y0 = s_y[rr * 2] + s_y[(MLP_ROWS + rr) * 2] + a.b2[0];
-        y1 = s_y[rr * 2 + 1] + s_y[(MLP_ROWS + rr) * 2 + 1] + a.b2[1];
-        if (valid && a.Y && half == 0) {
+        y0 = s_y[rr * 2] + s_y[(MLP_ROWS + rr) * 2];
+        y1 = s_y[rr * 2 + 1] + s_y[(MLP_ROWS + rr) * 2 + 1];
+    }
+    if (ok) {
+        y0 += a.b2[0];
+        y1 += a.b2[1];
+        if (valid && a.Y && half == 0 && crank == 0) {
             a.Y[2 * r] = y0;
             a.Y[2 * r + 1] = y1;
         }
@@ -332,7 +364,7 @@ __global__ void __launch_bounds__(MLP_FWD_THREADS, 2) k_mlp_fwd_tc(const __grid_
             const float e0 = valid ? y0 - a.T[2 * r] : 0.f, e1 = valid ? y1 - a.T[2 * r + 1] : 0.f;
             const float g0 = e0 * a.inv_B, g1 = e1 * a.inv_B; // d mean over 2B of e^2
             float *wcol = s_col + quad * ncol;
-            if (half == 0) {
+            if (half == 0 && crank == 0) {
                 if (valid) {
                     a.dY[2 * r] = g0;
                     a.dY[2 * r + 1] = g1;
@@ -372,8 +404,8 @@ __global__ void __launch_bounds__(MLP_FWD_THREADS, 2) k_mlp_fwd_tc(const __grid_
                     const float gpb = fmaf(zb * 0.39894228040143268f, pb.y, pb.x);
                     const uint32_t dp = valid ? bf2_pack(dha * gpa, dhb * gpb) : 0u;
                     if (valid || padrow) {
-                        a.dZt[(long long)(c + j) * a.ldt + r] = (uint16_t)(dp & 0xffffu);
-                        a.dZt[(long long)(c + j + 1) * a.ldt + r] = (uint16_t)(dp >> 16);
+                        a.dZt[(long long)(h0 + c + j) * a.ldt + r] = (uint16_t)(dp & 0xffffu);
+                        a.dZt[(long long)(h0 + c + j + 1) * a.ldt + r] = (uint16_t)(dp >> 16);
                     }
                     db[j] = __uint_as_float(dp << 16);
                     db[j + 1] = __uint_as_float(dp & 0xffff0000u);
@@ -397,15 +429,18 @@ __global__ void __launch_bounds__(MLP_FWD_THREADS, 2) k_mlp_fwd_tc(const __grid_
     __syncthreads();
     if (warp == 0)
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(a.tmem_cols));
-    if (!ok) {
-        if (t == 0)
-            atomicOr(a.err, 1);
-        return;
-    }
-    if (train)
-        for (int i = t; i < ncol; i += MLP_FWD_THREADS)
-            a.pCol[(long long)blockIdx.x * ncol + i] =
-                ((s_col[i] + s_col[ncol + i]) + s_col[2 * ncol + i]) + s_col[3 * ncol + i];
+    if (!ok && t == 0)
+        atomicOr(a.err, 1);
+    if (ok && train)
+        for (int i = t; i < ncol; i += MLP_FWD_THREADS) {
+            // local columns db1 | dW2 | db2 to their places among a.dh units
+            const int at = i < dh ? h0 + i : i < 3 * dh ? a.dh + 2 * h0 + (i - dh) : 3 * a.dh + (i - 3 * dh);
+            if (i < 3 * dh || crank == 0)
+                a.pCol[tile * (3 * a.dh + 2) + at] =
+                    ((s_col[i] + s_col[ncol + i]) + s_col[2 * ncol + i]) + s_col[3 * ncol + i];
+        }
+    if (C > 1)
+        cg::this_cluster().sync(); // no CTA leaves while a peer reads its partial head
 }
 
 struct MlpDw1Args {
@@ -475,25 +510,22 @@ __global__ void __launch_bounds__(MLP_ROWS, 1) k_mlp_dw1_tc(const __grid_constan
                 break;
             }
         }
-        // A: row t = hidden unit h, 16 batch values per K step
-        for (int s = 0; s < ks; ++s) {
-            uint4 v0 = make_uint4(0, 0, 0, 0), v1 = v0;
-            if (h < a.dh) {
-                const uint4 *src = (const uint4 *)(a.dZt + (long long)h * a.ldt + kb + s * 16);
-                v0 = __ldg(src);
-                v1 = __ldg(src + 1);
-            }
-            *(uint4 *)(sA + s * 4096 + kmaj_off_bf16(t, 0)) = v0;
-            *(uint4 *)(sA + s * 4096 + kmaj_off_bf16(t, 8)) = v1;
-        }
-        // B: row n = input f0 + n
-        for (int n = t; n < nn; n += MLP_ROWS) {
-            for (int s = 0; s < ks; ++s) {
-                const uint4 *src = (const uint4 *)(a.Xt + (long long)(f0 + n) * a.ldt + kb + s * 16);
-                *(uint4 *)(sB + (size_t)s * nn * 32 + kmaj_off_bf16(n, 0)) = __ldg(src);
-                *(uint4 *)(sB + (size_t)s * nn * 32 + kmaj_off_bf16(n, 8)) = __ldg(src + 1);
-            }
-        }
+        // A: row t = hidden unit h; B: rows t and t + 128 = inputs f0 + n.
+        // All of a row's reads are in flight before the first is stored.
+        auto put_row = [&](const uint16_t *row, bool have, unsigned char *dst, int sbytes, int n) {
+            uint4 v[2 * DW1_KSTEPS];
+#pragma unroll
+            for (int i = 0; i < 2 * DW1_KSTEPS; ++i)
+                v[i] = have && i < 2 * ks ? __ldg((const uint4 *)(row + kb) + i) : make_uint4(0, 0, 0, 0);
+#pragma unroll
+            for (int i = 0; i < 2 * DW1_KSTEPS; ++i)
+                if (i < 2 * ks)
+                    *(uint4 *)(dst + (size_t)(i >> 1) * sbytes + kmaj_off_bf16(n, (i & 1) * 8)) = v[i];
+        };
+        put_row(a.dZt + (long long)h * a.ldt, h < a.dh, sA, 4096, t);
+#pragma unroll 1
+        for (int n = t; n < nn; n += MLP_ROWS)
+            put_row(a.Xt + (long long)(f0 + n) * a.ldt, true, sB, nn * 32, n);
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
         asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
         __syncthreads();

@@ -406,7 +406,7 @@ __global__ void k_adamw(const __grid_constant__ AdamArgs a)
         return;
     const long long nW1 = (long long)a.d_in * a.dh;
     const int stride = a.dh * 3 + 2;
-    // partial sums over the batch slices: four independent chains so that
+    // partial sums over the batch slices: eight independent chains so that
     // the loads overlap (the order is fixed, so the result is deterministic)
     const float *src;
     long long ld;
@@ -420,17 +420,15 @@ __global__ void k_adamw(const __grid_constant__ AdamArgs a)
         ld = stride;
         ns = a.splits2;
     }
-    float g0 = 0.f, g1 = 0.f, g2 = 0.f, g3 = 0.f;
+    float gs[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
     int s = 0;
-    for (; s + 4 <= ns; s += 4) {
-        g0 += src[(long long)s * ld];
-        g1 += src[(long long)(s + 1) * ld];
-        g2 += src[(long long)(s + 2) * ld];
-        g3 += src[(long long)(s + 3) * ld];
-    }
+    for (; s + 8 <= ns; s += 8)
+#pragma unroll
+        for (int i = 0; i < 8; ++i)
+            gs[i] += src[(long long)(s + i) * ld];
     for (; s < ns; ++s)
-        g0 += src[(long long)s * ld];
-    const float g = (g0 + g1) + (g2 + g3);
+        gs[0] += src[(long long)s * ld];
+    const float g = ((gs[0] + gs[1]) + (gs[2] + gs[3])) + ((gs[4] + gs[5]) + (gs[6] + gs[7]));
     if (a.grad_out) {
         a.grad_out[p] = g;
         return;
@@ -819,12 +817,34 @@ static tnn_status mlp_forward_impl(const tnn_mlp *n, const uint16_t *d_x, long l
         TNN_CUDA_TRY(cudaGetLastError());
         return TNN_OK;
     }
+    // Training: hidden units split over a cluster while that still gives every
+    // CTA an SM of its own (at least 64 units each: two halves of 32).
+    const long long tiles = (B + MLP_ROWS - 1) / MLP_ROWS;
+    int dev = 0, nsm = 0;
+    TNN_CUDA_TRY(cudaGetDevice(&dev));
+    TNN_CUDA_TRY(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
+    a.csize = 1;
+    while (d_t && a.csize < 8 && n->dh % (128 * a.csize) == 0 && tiles * 2 * a.csize <= nsm)
+        a.csize *= 2;
+    const int dhc = n->dh / a.csize;
+    a.tmem_cols = tmem_cols_for(dhc);
     // every K step staged at once when it fits (no per-step synchronisation)
-    a.resident = mlp_fwd_smem_res(n->d_in, n->dh) <= (size_t)227 * 1024;
-    const size_t smem = tc_smem_request(a.resident ? mlp_fwd_smem_res(n->d_in, n->dh) : mlp_fwd_smem(n->dh),
+    a.resident = mlp_fwd_smem_res(n->d_in, dhc) <= (size_t)227 * 1024;
+    const size_t smem = tc_smem_request(a.resident ? mlp_fwd_smem_res(n->d_in, dhc) : mlp_fwd_smem(dhc),
                                         a.tmem_cols);
-    k_mlp_fwd_tc<<<(unsigned)((B + MLP_ROWS - 1) / MLP_ROWS), MLP_FWD_THREADS, smem, st>>>(a);
-    TNN_CUDA_TRY(cudaGetLastError());
+    cudaLaunchConfig_t cfg;
+    memset(&cfg, 0, sizeof(cfg));
+    cfg.gridDim = dim3((unsigned)(tiles * a.csize));
+    cfg.blockDim = dim3(MLP_FWD_THREADS);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cudaLaunchAttribute attr;
+    attr.id = cudaLaunchAttributeClusterDimension;
+    attr.val.clusterDim.x = (unsigned)a.csize;
+    attr.val.clusterDim.y = attr.val.clusterDim.z = 1;
+    cfg.attrs = &attr;
+    cfg.numAttrs = a.csize > 1 ? 1 : 0;
+    TNN_CUDA_TRY(cudaLaunchKernelEx(&cfg, k_mlp_fwd_tc, a));
     return TNN_OK;
 }
 
