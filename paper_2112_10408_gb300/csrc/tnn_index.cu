@@ -56,130 +56,209 @@ __device__ __forceinline__ uint32_t f2ord(float f)
 
 enum { BAD_VALUE = 1, BAD_ORDER = 2 };
 
-// Every coordinate finite with |v| <= 1e15 (so every FP32 squared
-// difference stays finite); largest |sqrt(sigma) * x| over the spatial axes.
-__global__ void k_validate_points(const float4 *__restrict__ p, int n,
-                                  float s0, float s1, float s2,
-                                  unsigned int *flag, unsigned int *cmax_bits)
-{
-    int i = blockIdx.x * blockDim.x + threadIdx.x;
-    float m = 0.f;
-    if (i < n) {
-        float4 v = p[i];
-        bool ok = fabsf(v.x) <= 1e15f && fabsf(v.y) <= 1e15f &&
-                  fabsf(v.z) <= 1e15f && fabsf(v.w) <= 1e15f;
-        if (!ok)
-            atomicOr(flag, (unsigned)BAD_VALUE);
-        else
-            m = fmaxf(fmaxf(fabsf(s0 * v.x), fabsf(s1 * v.y)), fabsf(s2 * v.z));
-    }
-    for (int o = 16; o > 0; o >>= 1)
-        m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
-    if ((threadIdx.x & 31) == 0 && m > 0.f)
-        atomicMax(cmax_bits, __float_as_uint(m)); // m >= 0: bits are monotone
-}
+// Words of the build's device header: filled by k_validate and the segment
+// fit, read back once.
+enum {
+    META_FLAG = 0,  // BAD_* bits
+    META_CMAX = 1,  // largest |scaled spatial coordinate|, bits
+    META_BBOX = 2,  // per axis x, y, z, t: ordered minimum, maximum
+    META_DUR = 10,  // summed duration of the K-point sets (a double)
+    META_READ = 12, // words the host reads
+    META_RMAX = 12, // largest segment radius, bits
+    META_EXT = 13,  // largest key extent, bits
+    META_WORDS = 16
+};
 
-// Times non-decreasing inside each trajectory, and the summed duration
-// t_last - t_first of its K-point sets, which sizes the grid's time buckets
-// (one warp per trajectory).
-__global__ void k_validate_traj(const float4 *__restrict__ p,
-                                const int32_t *__restrict__ traj_off,
-                                int n_traj, int K, unsigned int *flag, double *dur_sum)
+#define VAL_THREADS 256
+
+// One pass over the caller's points by the first `pblocks` blocks: copied
+// into the index, every coordinate finite with |v| <= 1e15 (so every FP32
+// squared difference stays finite), the largest |sqrt(sigma) x| over the
+// spatial axes, the bounding box.  The other blocks take a trajectory per
+// warp: times non-decreasing inside it, the summed duration t_last - t_first
+// of its K-point sets, which sizes the grid's time buckets, and the sets'
+// (first point, count, trajectory) and t_A sort keys (the last of these blocks the sort's
+// padding).
+// (A copy and three kernels before; bound by the reads and the launch.)
+__global__ void __launch_bounds__(VAL_THREADS)
+    k_validate(const float4 *__restrict__ in, float4 *__restrict__ out, int n, float s0, float s1, float s2,
+               const int32_t *__restrict__ traj_off, const int32_t *__restrict__ seg_off, int n_traj, int K,
+               int pblocks, int S, int S2, int4 *__restrict__ range, unsigned long long *__restrict__ keys,
+               unsigned int *__restrict__ meta)
 {
-    const int tr = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
-    if (tr >= n_traj) // the same for the whole warp
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    if ((int)blockIdx.x >= pblocks) {
+        if (blockIdx.x == gridDim.x - 1)
+            for (int i = S + threadIdx.x; i < S2; i += VAL_THREADS)
+                keys[i] = ~0ull;
+        const int tr = ((int)blockIdx.x - pblocks) * (VAL_THREADS / 32) + w;
+        if (tr >= n_traj) // the same for the whole warp
+            return;
+        const int b = traj_off[tr], e = traj_off[tr + 1];
+        bool bad = false;
+        for (int i = b + 1 + lane; i < e; i += 32)
+            bad |= !(in[i].w >= in[i - 1].w);
+        double dur = 0.0;
+        int sg = seg_off[tr] + lane; // build id of the set
+        for (int f = b + lane * K; f < e; f += 32 * K, sg += 32) {
+            const float tA = in[f].w;
+            dur += (double)in[min(f + K - 1, e - 1)].w - (double)tA;
+            range[sg] = make_int4(f, min(K, e - f), tr, 0);
+            keys[sg] = ((unsigned long long)f2ord(tA) << 32) | (unsigned)sg;
+        }
+        for (int o = 16; o > 0; o >>= 1)
+            dur += __shfl_xor_sync(0xffffffffu, dur, o);
+        if (__any_sync(0xffffffffu, bad) && lane == 0)
+            atomicOr(meta + META_FLAG, (unsigned)BAD_ORDER);
+        if (lane == 0 && dur != 0.0)
+            atomicAdd((double *)(meta + META_DUR), dur);
         return;
-    const int b = traj_off[tr], e = traj_off[tr + 1];
+    }
+    // [0] largest |scaled coordinate|; [1 + 2 d], [2 + 2 d] axis d's minimum
+    // and maximum
+    __shared__ unsigned int s[VAL_THREADS / 32][9];
+    unsigned int m[9] = {0u, 0xffffffffu, 0u, 0xffffffffu, 0u, 0xffffffffu, 0u, 0xffffffffu, 0u};
     bool bad = false;
-    for (int i = b + 1 + lane; i < e; i += 32)
-        bad |= !(p[i].w >= p[i - 1].w);
-    double dur = 0.0;
-    for (int f = b + lane * K; f < e; f += 32 * K)
-        dur += (double)p[min(f + K - 1, e - 1)].w - (double)p[f].w;
-    for (int o = 16; o > 0; o >>= 1)
-        dur += __shfl_xor_sync(0xffffffffu, dur, o);
+    for (int i = blockIdx.x * VAL_THREADS + threadIdx.x; i < n; i += pblocks * VAL_THREADS) {
+        const float4 v = in[i];
+        out[i] = v;
+        if (fabsf(v.x) <= 1e15f && fabsf(v.y) <= 1e15f && fabsf(v.z) <= 1e15f && fabsf(v.w) <= 1e15f)
+            m[0] = max(m[0], __float_as_uint(fmaxf(fmaxf(fabsf(s0 * v.x), fabsf(s1 * v.y)), fabsf(s2 * v.z))));
+        else
+            bad = true;
+        const float c[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+        for (int d = 0; d < 4; ++d) {
+            const unsigned int u = f2ord(c[d]);
+            m[1 + 2 * d] = min(m[1 + 2 * d], u);
+            m[2 + 2 * d] = max(m[2 + 2 * d], u);
+        }
+    }
     if (__any_sync(0xffffffffu, bad) && lane == 0)
-        atomicOr(flag, (unsigned)BAD_ORDER);
-    if (lane == 0 && dur != 0.0)
-        atomicAdd(dur_sum, dur);
+        atomicOr(meta + META_FLAG, (unsigned)BAD_VALUE);
+#pragma unroll
+    for (int d = 0; d < 9; ++d) {
+        m[d] = (d & 1) ? __reduce_min_sync(0xffffffffu, m[d]) : __reduce_max_sync(0xffffffffu, m[d]);
+        if (lane == 0)
+            s[w][d] = m[d];
+    }
+    __syncthreads();
+    if (threadIdx.x < 9) {
+        const int d = threadIdx.x;
+        unsigned int r = s[0][d];
+        for (int j = 1; j < VAL_THREADS / 32; ++j)
+            r = (d & 1) ? min(r, s[j][d]) : max(r, s[j][d]);
+        if (d & 1)
+            atomicMin(meta + META_CMAX + d, r);
+        else
+            atomicMax(meta + META_CMAX + d, r);
+    }
 }
 
-// SF_LANES lanes per segment (build order).  FP64 throughout, rounded once to
-// the stored FP32 record:
+// One thread per segment (build order).  FP64, rounded once to the stored
+// FP32 record:
 //   A' = fl(sqrt(s) A),  AB' = fl(sqrt(s) B - A'),  U' = fl(AB' / |AB'|^2)
 // The stored segment is [A', A' + AB'] (both exactly representable);
 // r bounds, with upward rounding, the distance of every member's scaled
 // position sqrt(s) p_j to it (Sec. 3.4 E_app, in the cylinder reading).
-#ifndef SF_LANES
-#define SF_LANES 4 // a power of two, at most 32
-#endif
-__global__ void k_segment_fit(const float4 *__restrict__ p,
-                              const int32_t *__restrict__ traj_off,
-                              const int32_t *__restrict__ seg_off, int n_traj,
-                              int S, int K, double q0, double q1, double q2,
-                              float4 *__restrict__ rec,
-                              unsigned long long *__restrict__ keys,
-                              unsigned int *rmax_bits)
+//
+// FP64 instructions bound this kernel (one warp instruction occupies the pipe
+// of an SM for 16 cycles).  Only the largest distance is kept, so a pass in
+// FP32 first finds the members that can hold it: with offsets taken from the
+// first member (small numbers) its error is below 2^-19 (|D| + |AB|)_max, and
+// the members whose distance is within 2^-17 of that scale of the largest one
+// are measured in FP64: one, now and then two; three or more (or a segment
+// whose |AB|^2 FP32 does not hold) measure all members.  The same radius, bit
+// for bit; 20,000 segments of 20 points (cold caches): 45 us with every member
+// in FP64 by four lanes per segment, 13 us now.
+#define SF_THREADS 128
+__global__ void __launch_bounds__(SF_THREADS)
+    k_segment_fit(const float4 *__restrict__ p, const int4 *__restrict__ range, int S, double q0, double q1,
+                  double q2, float4 *__restrict__ rec, unsigned int *rmax_bits)
 {
-    // SF_LANES lanes per segment, splitting its members (FP64 is scarce:
-    // the per-segment set-up is repeated by each of them)
-    const int s_raw = (int)(((int64_t)blockIdx.x * blockDim.x + threadIdx.x) / SF_LANES);
-    const int sub = threadIdx.x % SF_LANES;
-    const bool valid = s_raw < S;
-    const int s = valid ? s_raw : S - 1;
-    // trajectory of segment s: largest tr with seg_off[tr] <= s
-    int lo = 0, hi = n_traj; // seg_off[lo] <= s < seg_off[hi]
-    while (hi - lo > 1) {
-        int mid = (lo + hi) >> 1;
-        if (seg_off[mid] <= s)
-            lo = mid;
-        else
-            hi = mid;
-    }
-    int tr = lo;
-    int first = traj_off[tr] + (s - seg_off[tr]) * K;
-    int count = min(K, traj_off[tr + 1] - first);
-    float4 pa = p[first], pb = p[first + count - 1];
-    double A[3], E[3], AB[3];
-    float Af[3], ABf[3], Uf[3];
-    const double qq[3] = {q0, q1, q2};
-    const float pav[3] = {pa.x, pa.y, pa.z}, pbv[3] = {pb.x, pb.y, pb.z};
-    for (int i = 0; i < 3; ++i) {
-        Af[i] = (float)(qq[i] * (double)pav[i]);
-        A[i] = (double)Af[i];
-        ABf[i] = (float)(qq[i] * (double)pbv[i] - A[i]);
-        AB[i] = (double)ABf[i];
-        E[i] = A[i] + AB[i];
-    }
-    const double ab2 = AB[0] * AB[0] + AB[1] * AB[1] + AB[2] * AB[2];
-    // Any lam in [0, 1] names a point of the segment, so the distance to it
-    // bounds the distance to the segment from above: lam = dot / |AB|^2 may
-    // take the reciprocal (one division per lane, not one per member).
-    const double inv_ab2 = ab2 > 0.0 ? 1.0 / ab2 : 0.0;
-    // mag only scales the rounding slack below, which is about a thousand
-    // times the FP64 error of the distances; FP32 is ample for it.
-    const float qf[3] = {(float)q0, (float)q1, (float)q2};
-    float mag = fabsf(Af[0]) + fabsf(Af[1]) + fabsf(Af[2]) + fabsf((float)E[0]) +
-                fabsf((float)E[1]) + fabsf((float)E[2]);
-    double r2 = 0.0;
-    for (int j = sub; j < (valid ? count : 0); j += SF_LANES) {
-        const float4 v = p[first + j];
-        const double D0 = qq[0] * (double)v.x - A[0], D1 = qq[1] * (double)v.y - A[1],
-                     D2 = qq[2] * (double)v.z - A[2];
-        const double lam = fmin(fmax((D0 * AB[0] + D1 * AB[1] + D2 * AB[2]) * inv_ab2, 0.0), 1.0);
-        const double e0 = D0 - lam * AB[0], e1 = D1 - lam * AB[1], e2 = D2 - lam * AB[2];
-        r2 = fmax(r2, e0 * e0 + e1 * e1 + e2 * e2);
-        mag = fmaxf(mag, fabsf(qf[0] * v.x) + fabsf(qf[1] * v.y) + fabsf(qf[2] * v.z));
-    }
-    for (int o = 1; o < SF_LANES; o <<= 1) {
-        r2 = fmax(r2, __shfl_xor_sync(0xffffffffu, r2, o));
-        mag = fmaxf(mag, __shfl_xor_sync(0xffffffffu, mag, o));
-    }
-    const bool writer = valid && sub == 0;
+    const int s = blockIdx.x * SF_THREADS + threadIdx.x;
     unsigned int rbits = 0u;
-    if (writer) {
+    if (s < S) {
+        const int4 rg = range[s];
+        const int first = rg.x, count = rg.y, tr = rg.z;
+        const float4 pa = p[first], pb = p[first + count - 1];
+        double A[3], AB[3];
+        float Af[3], ABf[3], Uf[3], res[3];
+        const double qq[3] = {q0, q1, q2};
+        const float qf[3] = {(float)q0, (float)q1, (float)q2};
+        const float pav[3] = {pa.x, pa.y, pa.z}, pbv[3] = {pb.x, pb.y, pb.z};
+        // mag only scales the rounding slack below, which is about a thousand
+        // times the FP64 error of the distances; FP32 is ample for it.
+        float mag = 0.f;
+#pragma unroll
+        for (int i = 0; i < 3; ++i) {
+            const double sa = qq[i] * (double)pav[i];
+            Af[i] = (float)sa;
+            A[i] = (double)Af[i];
+            res[i] = (float)(sa - A[i]); // sqrt(s) p - A' = sqrt(s) (p - p_a) + res
+            ABf[i] = (float)(qq[i] * (double)pbv[i] - A[i]);
+            AB[i] = (double)ABf[i];
+            mag += fabsf(Af[i]) + fabsf((float)(A[i] + AB[i]));
+        }
+        const double ab2 = AB[0] * AB[0] + AB[1] * AB[1] + AB[2] * AB[2];
+        // Any lam in [0, 1] names a point of the segment, so the distance to
+        // it bounds the distance to the segment from above: lam = dot / |AB|^2
+        // may take the reciprocal (one division, not one per member).
+        const double inv_ab2 = ab2 > 0.0 ? 1.0 / ab2 : 0.0;
+        // ---- FP32: squared distances, their maximum, the scale of the error
+        const float ab2f = (float)ab2;
+        const bool screen = ab2f > 1e-20f && ab2f < 1e35f; // else every member in FP64
+        const float inv32 = (float)inv_ab2;
+        auto dist2_32 = [&](const float4 &v, float &dm) {
+            const float D0 = fmaf(qf[0], v.x - pa.x, res[0]), D1 = fmaf(qf[1], v.y - pa.y, res[1]),
+                        D2 = fmaf(qf[2], v.z - pa.z, res[2]);
+            const float lam = __saturatef(fmaf(D2, ABf[2], fmaf(D1, ABf[1], D0 * ABf[0])) * inv32);
+            const float e0 = fmaf(-lam, ABf[0], D0), e1 = fmaf(-lam, ABf[1], D1), e2 = fmaf(-lam, ABf[2], D2);
+            dm = fmaxf(fmaxf(fabsf(D0), fabsf(D1)), fabsf(D2));
+            return fmaf(e2, e2, fmaf(e1, e1, e0 * e0));
+        };
+        // the three largest, and where the first two are
+        float m1 = -1.f, m2 = -1.f, m3 = -1.f, dmax = 0.f;
+        int j1 = 0, j2 = 0;
+#pragma unroll 4
+        for (int j = 0; j < count; ++j) {
+            const float4 v = p[first + j];
+            float dm;
+            const float e = dist2_32(v, dm);
+            m3 = e > m2 ? m2 : fmaxf(m3, e);
+            j2 = e > m1 ? j1 : e > m2 ? j : j2;
+            m2 = e > m1 ? m1 : fmaxf(m2, e);
+            j1 = e > m1 ? j : j1;
+            m1 = fmaxf(m1, e);
+            dmax = fmaxf(dmax, dm);
+            mag = fmaxf(mag, fabsf(qf[0] * v.x) + fabsf(qf[1] * v.y) + fabsf(qf[2] * v.z));
+        }
+        const float abm = fmaxf(fmaxf(fabsf(ABf[0]), fabsf(ABf[1])), fabsf(ABf[2]));
+        const float thr = fmaxf(sqrtf(fmaxf(m1, 0.0f)) - 0x1p-17f * (dmax + abm), 0.0f);
+        const float thr2 = thr * thr * (1.0f - 0x1p-20f);
+        // ---- FP64: the members that can be the farthest
+        auto dist2_64 = [&](int j) {
+            const float4 v = p[first + j];
+            const double D0 = qq[0] * (double)v.x - A[0], D1 = qq[1] * (double)v.y - A[1],
+                         D2 = qq[2] * (double)v.z - A[2];
+            const double lam = fmin(fmax((D0 * AB[0] + D1 * AB[1] + D2 * AB[2]) * inv_ab2, 0.0), 1.0);
+            const double e0 = D0 - lam * AB[0], e1 = D1 - lam * AB[1], e2 = D2 - lam * AB[2];
+            return e0 * e0 + e1 * e1 + e2 * e2;
+        };
+        double r2;
+        if (screen && m3 < thr2) {
+            r2 = dist2_64(j1);
+            if (!(m2 < thr2))
+                r2 = fmax(r2, dist2_64(j2));
+        } else {
+            r2 = 0.0;
+#pragma unroll 1
+            for (int j = 0; j < count; ++j)
+                r2 = fmax(r2, dist2_64(j));
+        }
+#pragma unroll
         for (int i = 0; i < 3; ++i)
-            Uf[i] = ab2 > 1e-30 ? (float)(AB[i] / ab2) : 0.f;
+            Uf[i] = ab2 > 1e-30 ? (float)(AB[i] * inv_ab2) : 0.f;
         // FP64 rounding of the distances above is far below 1e-12 * mag.
         const double r = sqrt(r2) + 1e-12 * (1.0 + (double)mag);
         const float rf = __double2float_ru(r);
@@ -189,7 +268,6 @@ __global__ void k_segment_fit(const float4 *__restrict__ p,
         rec[4 * s + 2] = make_float4(ABf[0], ABf[1], ABf[2], rf);
         rec[4 * s + 3] = make_float4(__int_as_float(first), __int_as_float(count),
                                      __int_as_float(tr), __int_as_float(s));
-        keys[s] = ((unsigned long long)f2ord(pa.w) << 32) | (unsigned)s;
     }
     rbits = __reduce_max_sync(0xffffffffu, rbits); // one atomic per warp
     if ((threadIdx.x & 31) == 0 && rbits != 0u)
@@ -203,13 +281,6 @@ __global__ void k_time_keys(const float4 *__restrict__ p, int n,
     if (i < n)
         keys[i] = ((unsigned long long)f2ord(p[i].w) << 32) | (unsigned)i;
     else if (i < n2)
-        keys[i] = ~0ull;
-}
-
-__global__ void k_fill(unsigned long long *keys, int from, int n2)
-{
-    int i = from + blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < n2)
         keys[i] = ~0ull;
 }
 
@@ -396,25 +467,135 @@ void tnn_bitonic_sort(unsigned long long *keys, int n2, cudaStream_t st)
     }
 }
 
-// --------------------------------------------------------- gather / scans
+// -------------------------------------------------------------- radix sort
+//
+// Stable ascending sort by the upper halves of n2 <= 32,768 keys in one
+// launch, least significant 8 bits first: a cluster of 8 CTAs, CTA c holding
+// positions c nl .. (c + 1) nl - 1 (nl = n2 / 8), IT keys per thread.  Per
+// digit: ranks inside a warp by match, per-warp counts in shared memory, their
+// prefix over the warps, the CTAs' totals exchanged through distributed shared
+// memory, and every key written straight into its place in the CTA that holds
+// it.  Keys carry their position below the sort value, so a stable sort by the
+// value is the sort of the whole key.  Latency bounds it: two cluster barriers
+// per digit (four digits for times, as many as the number of grid keys needs)
+// against two per step of the bitonic network whose partner is in another CTA;
+// 20,000 keys (cold caches): 46 us by the network, 25 us for times and 14 us
+// for grid keys.
+#define RS_CLUSTER 8
 
-__global__ void k_gather_segments(const unsigned long long *__restrict__ keys,
-                                  const float4 *__restrict__ rec, int S,
-                                  float4 *__restrict__ out,
-                                  float *__restrict__ tA, int32_t *__restrict__ pos)
+struct RadixSmem {
+    unsigned long long buf[4096];
+    unsigned short hist[32][256]; // per warp: count, then prefix over the warps
+    unsigned tot[256];            // this CTA's count per digit (read by its peers)
+    unsigned off[256];            // first position of this CTA's keys per digit
+    unsigned part[8];
+};
+
+template <int IT>
+__global__ void __cluster_dims__(RS_CLUSTER, 1, 1) __launch_bounds__(1024)
+    k_radix_cluster(unsigned long long *keys, int n2, int bits)
 {
-    int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= S)
-        return;
-    int s = (int)(keys[i] & 0xffffffffu);
-    pos[s] = i;
-    float4 a = rec[4 * s];
-    out[4 * i + 0] = a;
-    out[4 * i + 1] = rec[4 * s + 1];
-    out[4 * i + 2] = rec[4 * s + 2];
-    out[4 * i + 3] = rec[4 * s + 3];
-    tA[i] = a.w;
+    extern __shared__ __align__(16) unsigned char raw[];
+    RadixSmem &S = *(RadixSmem *)raw;
+    cg::cluster_group cluster = cg::this_cluster();
+    const int c = (int)cluster.block_rank(), nl = n2 / RS_CLUSTER, t = threadIdx.x;
+    const int lane = t & 31, w = t >> 5, nw = blockDim.x >> 5;
+    const int at = w * 32 * IT + lane; // key j of this thread: position at + 32 j of the CTA
+    unsigned long long r[IT];
+#pragma unroll
+    for (int j = 0; j < IT; ++j)
+        r[j] = keys[(size_t)c * nl + at + 32 * j];
+#pragma unroll 1
+    for (int shift = 32; shift < 32 + bits; shift += 8) {
+        for (int i = t; i < nw * 256; i += blockDim.x)
+            (&S.hist[0][0])[i] = 0;
+        __syncthreads();
+        int rank[IT];
+#pragma unroll
+        for (int j = 0; j < IT; ++j) {
+            const unsigned d = (unsigned)(r[j] >> shift) & 255u;
+            const unsigned same = __match_any_sync(0xffffffffu, d);
+            const unsigned before = same & ((1u << lane) - 1u);
+            rank[j] = S.hist[w][d] + __popc(before);
+            __syncwarp();
+            if (before == 0)
+                S.hist[w][d] = (unsigned short)(S.hist[w][d] + __popc(same));
+            __syncwarp();
+        }
+        __syncthreads();
+        if (t < 256) {
+            unsigned sum = 0;
+#pragma unroll 8
+            for (int i = 0; i < nw; ++i) {
+                const unsigned h = S.hist[i][t];
+                S.hist[i][t] = (unsigned short)sum;
+                sum += h;
+            }
+            S.tot[t] = sum;
+        }
+        // every key of this digit is in registers, every total is visible
+        cluster.sync();
+        unsigned all = 0, mine = 0;
+        if (t < 256) {
+#pragma unroll
+            for (int i = 0; i < RS_CLUSTER; ++i) {
+                const unsigned v = *cluster.map_shared_rank(&S.tot[t], i);
+                all += v;
+                mine += i < c ? v : 0u;
+            }
+            unsigned inc = all;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const unsigned v = __shfl_up_sync(0xffffffffu, inc, o);
+                if (lane >= o)
+                    inc += v;
+            }
+            if (lane == 31)
+                S.part[w] = inc;
+            mine += inc - all;
+        }
+        __syncthreads();
+        if (t < 256) {
+            for (int i = 0; i < w; ++i)
+                mine += S.part[i];
+            S.off[t] = mine;
+        }
+        __syncthreads();
+#pragma unroll
+        for (int j = 0; j < IT; ++j) {
+            const unsigned d = (unsigned)(r[j] >> shift) & 255u;
+            const unsigned pos = S.off[d] + S.hist[w][d] + (unsigned)rank[j];
+            const unsigned dst = pos / (unsigned)nl;
+            *cluster.map_shared_rank(&S.buf[pos - dst * (unsigned)nl], dst) = r[j];
+        }
+        cluster.sync(); // every key is in place
+#pragma unroll
+        for (int j = 0; j < IT; ++j)
+            r[j] = S.buf[at + 32 * j];
+    }
+#pragma unroll
+    for (int j = 0; j < IT; ++j)
+        keys[(size_t)c * nl + at + 32 * j] = r[j];
 }
+
+// Ascending sort of n2 keys (sort value << 32 | position, in the order of
+// their positions, padding ~0 behind them); the values fit in `bits` bits and
+// are not all ones there.
+static tnn_status sort_by_value(unsigned long long *keys, int n2, int bits, cudaStream_t st)
+{
+    if (n2 > RS_CLUSTER * 4096) {
+        tnn_bitonic_sort(keys, n2, st);
+        return TNN_OK;
+    }
+    const int nl = n2 / RS_CLUSTER, threads = std::min(nl, 1024), it = nl / threads;
+    const auto kern = it == 1 ? k_radix_cluster<1> : it == 2 ? k_radix_cluster<2> : k_radix_cluster<4>;
+    TNN_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(RadixSmem)));
+    kern<<<RS_CLUSTER, threads, sizeof(RadixSmem), st>>>(keys, n2, bits);
+    TNN_CUDA_TRY(cudaGetLastError());
+    return TNN_OK;
+}
+
+// --------------------------------------------------------- gather / scans
 
 // Running maximum of t_B over the t_A order, in two passes over blocks of
 // 1024 segments: the maximum of every block, then per block the maxima of
@@ -434,12 +615,28 @@ __device__ __forceinline__ float block_max_1024(float v, float *sh)
     return v;
 }
 
-__global__ void __launch_bounds__(1024) k_pm_block_max(const float4 *__restrict__ seg, int S,
-                                                       float *__restrict__ bmax)
+// The records in t_A order (keys hold build ids), their start times, the
+// position of every build id, and the block maxima.
+__global__ void __launch_bounds__(1024)
+    k_gather_segments(const unsigned long long *__restrict__ keys, const float4 *__restrict__ rec, int S,
+                      float4 *__restrict__ out, float *__restrict__ tA, int32_t *__restrict__ pos,
+                      float *__restrict__ bmax)
 {
     __shared__ float sh[32];
     const int i = blockIdx.x * 1024 + threadIdx.x;
-    const float v = block_max_1024(i < S ? seg[4 * i + 1].w : -INFINITY, sh);
+    float tB = -INFINITY;
+    if (i < S) {
+        const int s = (int)(keys[i] & 0xffffffffu);
+        pos[s] = i;
+        const float4 a = rec[4 * s], u = rec[4 * s + 1];
+        out[4 * i + 0] = a;
+        out[4 * i + 1] = u;
+        out[4 * i + 2] = rec[4 * s + 2];
+        out[4 * i + 3] = rec[4 * s + 3];
+        tA[i] = a.w;
+        tB = u.w;
+    }
+    const float v = block_max_1024(tB, sh);
     if (threadIdx.x == 0)
         bmax[blockIdx.x] = v;
 }
@@ -500,71 +697,57 @@ __device__ __forceinline__ float ord2f(uint32_t u)
     return __uint_as_float((u & 0x80000000u) ? (u & 0x7fffffffu) : ~u);
 }
 
-// Bounding box of the raw points (x, y, z, t): ordered min/max per axis,
-// reduced over the block (grid-stride) before one atomic per value.
-__global__ void k_point_bbox(const float4 *__restrict__ p, int n, unsigned int *ord)
-{
-    __shared__ unsigned int s[32][8];
-    unsigned int m[8] = {0xffffffffu, 0u, 0xffffffffu, 0u, 0xffffffffu, 0u, 0xffffffffu, 0u};
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
-        const float4 v = p[i];
-        const float c[4] = {v.x, v.y, v.z, v.w};
-#pragma unroll
-        for (int d = 0; d < 4; ++d) {
-            const unsigned int u = f2ord(c[d]);
-            m[2 * d] = min(m[2 * d], u);
-            m[2 * d + 1] = max(m[2 * d + 1], u);
-        }
-    }
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = blockDim.x >> 5;
-#pragma unroll
-    for (int d = 0; d < 8; ++d)
-        for (int o = 16; o > 0; o >>= 1) {
-            const unsigned int x = __shfl_xor_sync(0xffffffffu, m[d], o);
-            m[d] = (d & 1) ? max(m[d], x) : min(m[d], x);
-        }
-    if (lane == 0)
-        for (int d = 0; d < 8; ++d)
-            s[w][d] = m[d];
-    __syncthreads();
-    if (threadIdx.x < 8) {
-        const int d = threadIdx.x;
-        unsigned int r = s[0][d];
-        for (int j = 1; j < nw; ++j)
-            r = (d & 1) ? max(r, s[j][d]) : min(r, s[j][d]);
-        if (d & 1)
-            atomicMax(ord + d, r);
-        else
-            atomicMin(ord + d, r);
-    }
-}
-
 struct GridBuild {
     float x0, y0, cell, inv_cell, t0, dt, inv_dt;
     int nx, ny, ncell, nb;
 };
 
-// Key of every segment (records in build order; the key's low half is the
-// build id, so the keys sort without the t_A order and the two sorts run
-// side by side) and the per-key aggregates: the extent (FP64, rounded up) of
-// the member cylinders around the key's cell rectangle and the largest t_B;
-// the per-bucket largest t_B.
-__global__ void k_grid_keys(const float4 *__restrict__ seg, int S, GridBuild g,
-                            unsigned long long *__restrict__ keys,
-                            unsigned int *__restrict__ ext_bits,
-                            unsigned int *__restrict__ tB_ord,
-                            unsigned int *__restrict__ bmax_ord)
+// Grid key of a segment: bucket of t_A, cell of the midpoint of [A', A' + AB'].
+__device__ __forceinline__ int grid_key(const GridBuild &g, float tA, float ax, float ay, float bx, float by,
+                                        int &bk, int &cx, int &cy)
+{
+    const float mx = fmaf(0.5f, bx, ax), my = fmaf(0.5f, by, ay);
+    bk = min(max((int)floorf((tA - g.t0) * g.inv_dt), 0), g.nb - 1);
+    cx = min(max((int)floorf((mx - g.x0) * g.inv_cell), 0), g.nx - 1);
+    cy = min(max((int)floorf((my - g.y0) * g.inv_cell), 0), g.ny - 1);
+    return bk * g.ncell + cy * g.nx + cx;
+}
+
+// Sort keys (grid key << 32 | build id) straight from the end points, with
+// the segment fit's rounding: they need none of its radii, so their sort runs
+// beside the fit.
+__global__ void k_grid_sort_keys(const float4 *__restrict__ p, const int4 *__restrict__ range, int S, int S2,
+                                 double q0, double q1, const __grid_constant__ GridBuild g,
+                                 unsigned long long *__restrict__ keys)
+{
+    const int s = blockIdx.x * blockDim.x + threadIdx.x; // build id
+    if (s >= S) {
+        if (s < S2)
+            keys[s] = ~0ull; // the sort's padding
+        return;
+    }
+    const int4 r = range[s];
+    const float4 pa = p[r.x], pb = p[r.x + r.y - 1];
+    const float ax = (float)(q0 * (double)pa.x), ay = (float)(q1 * (double)pa.y);
+    const float bx = (float)(q0 * (double)pb.x - (double)ax), by = (float)(q1 * (double)pb.y - (double)ay);
+    int bk, cx, cy;
+    const int key = grid_key(g, pa.w, ax, ay, bx, by, bk, cx, cy);
+    keys[s] = ((unsigned long long)(unsigned)key << 32) | (unsigned)s;
+}
+
+// The per-key aggregates of the records: the extent (FP64, rounded up) of the
+// member cylinders around the key's cell rectangle and the largest t_B; the
+// per-bucket largest t_B.
+__global__ void k_grid_extents(const float4 *__restrict__ seg, int S, const __grid_constant__ GridBuild g,
+                               unsigned int *__restrict__ ext_bits, unsigned int *__restrict__ tB_ord,
+                               unsigned int *__restrict__ bmax_ord)
 {
     const int p = blockIdx.x * blockDim.x + threadIdx.x; // build id
     if (p >= S)
         return;
     const float4 a = seg[4 * p], u = seg[4 * p + 1], b = seg[4 * p + 2];
-    const float mx = fmaf(0.5f, b.x, a.x), my = fmaf(0.5f, b.y, a.y);
-    const int bk = min(max((int)floorf((a.w - g.t0) * g.inv_dt), 0), g.nb - 1);
-    const int cx = min(max((int)floorf((mx - g.x0) * g.inv_cell), 0), g.nx - 1);
-    const int cy = min(max((int)floorf((my - g.y0) * g.inv_cell), 0), g.ny - 1);
-    const int key = bk * g.ncell + cy * g.nx + cx;
-    keys[p] = ((unsigned long long)(unsigned)key << 32) | (unsigned)p;
+    int bk, cx, cy;
+    const int key = grid_key(g, a.w, a.x, a.y, b.x, b.y, bk, cx, cy);
     // every cylinder point is within |AB|/2 + r of the midpoint
     const double ax = a.x, ay = a.y, bx = b.x, by = b.y, bz = b.z;
     const double half = 0.5 * sqrt(bx * bx + by * by + bz * bz) + (double)b.w;
@@ -582,91 +765,136 @@ __global__ void k_grid_keys(const float4 *__restrict__ seg, int S, GridBuild g,
     atomicMax(bmax_ord + bk, f2ord(u.w));
 }
 
-// off[k] = number of sorted keys below k.
-__global__ void k_grid_offsets(const unsigned long long *__restrict__ keys, int S,
-                               int nkeys, int32_t *__restrict__ off)
-{
-    const int k = blockIdx.x * blockDim.x + threadIdx.x;
-    if (k > nkeys)
-        return;
-    const unsigned long long t = (unsigned long long)(unsigned)k << 32;
-    int lo = 0, hi = S;
-    while (lo < hi) {
-        const int mid = (lo + hi) >> 1;
-        if (keys[mid] < t)
-            lo = mid + 1;
-        else
-            hi = mid;
-    }
-    off[k] = lo;
-}
+struct GridTail {
+    const unsigned long long *keys; // sorted (grid key << 32 | build id)
+    const float4 *rec;              // build order
+    const int32_t *pos;             // t_A position of every build id
+    int S, nkeys, nb, kblocks, rblocks;
+    int32_t *off, *ids;
+    float4 *gseg;
+    float *ext, *tB, *bpm;
+    int4 *krec;
+    unsigned int *ext_max;
+};
 
-// t_A position of the segment of every sorted grid key (keys hold build ids).
-__global__ void k_grid_ids(const unsigned long long *__restrict__ keys, int S,
-                           const int32_t *__restrict__ pos, int32_t *__restrict__ ids)
-{
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < S)
-        ids[i] = pos[(int)(keys[i] & 0xffffffffu)];
-}
+#define GT_THREADS 256
+#define GT_STAGE 2048
 
-// Segment records in grid-key order (record 3's trajectory field replaced by
-// the t_A position), so that the search reads a key's segments without an
-// indirection.
-__global__ void k_grid_records(const float4 *__restrict__ seg, const int32_t *__restrict__ ids, int S,
-                               float4 *__restrict__ gseg)
+// Everything the grid needs from its sorted keys, by block:
+//   the first kblocks   256 keys each: CSR offsets (the block's slice of the
+//                       sorted keys is found once and searched in shared
+//                       memory), largest t_B decoded, the 16-byte key record,
+//                       the largest extent;
+//   the next rblocks    segment records in key order (record 3's trajectory
+//                       field replaced by the t_A position), so that the
+//                       search reads a key's segments without an indirection;
+//   the last one        running maximum of t_B over the buckets.
+// (Eight kernels before, four of them a search of all keys or less than one
+// wave of work each, 33 us one after the other at 20,000 segments; 5 us.)
+__global__ void __launch_bounds__(GT_THREADS) k_grid_tail(const __grid_constant__ GridTail g)
 {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= S)
-        return;
-    const int p = ids[i];
-    gseg[4 * (size_t)i] = seg[4 * (size_t)p];
-    gseg[4 * (size_t)i + 1] = seg[4 * (size_t)p + 1];
-    gseg[4 * (size_t)i + 2] = seg[4 * (size_t)p + 2];
-    float4 r3 = seg[4 * (size_t)p + 3];
-    r3.z = __int_as_float(p);
-    gseg[4 * (size_t)i + 3] = r3;
-}
-
-__global__ void k_decode_ord(unsigned int *__restrict__ v, int n)
-{
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < n) {
-        const unsigned int u = v[i];
-        v[i] = u ? __float_as_uint(ord2f(u)) : __float_as_uint(-INFINITY);
-    }
-}
-
-// Per key, its CSR range, extent and largest t_B packed in one record.
-__global__ void k_key_records(const int32_t *__restrict__ off, const float *__restrict__ ext,
-                              const float *__restrict__ tB, int nkeys, int4 *__restrict__ kr)
-{
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < nkeys)
-        kr[i] = make_int4(off[i], off[i + 1], __float_as_int(ext[i]), __float_as_int(tB[i]));
-}
-
-// Maximum of non-negative floats given as their bits (the bits order them).
-__global__ void k_max_bits(const unsigned int *__restrict__ v, int n, unsigned int *out)
-{
-    unsigned int m = 0;
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x)
-        m = max(m, v[i]);
-    for (int o = 16; o > 0; o >>= 1)
-        m = max(m, __shfl_xor_sync(0xffffffffu, m, o));
-    if ((threadIdx.x & 31) == 0 && m)
-        atomicMax(out, m);
-}
-
-// Running maximum over buckets (one block).
-__global__ void k_prefix_max(float *__restrict__ v, int n)
-{
-    if (threadIdx.x == 0 && blockIdx.x == 0) {
-        float m = -INFINITY;
-        for (int i = 0; i < n; ++i) {
-            m = fmaxf(m, v[i]);
-            v[i] = m;
+    const int t = threadIdx.x, lane = t & 31, w = t >> 5;
+    int b = blockIdx.x;
+    if (b < g.kblocks) {
+        __shared__ int s_lo[2], s_off[GT_THREADS + 1];
+        __shared__ unsigned s_key[GT_STAGE];
+        const int k0 = b * GT_THREADS;
+        // segments of keys [k0, k0 + 256): a 32-way search of one warp each
+        if (w < 2) {
+            const unsigned kt = (unsigned)(k0 + w * GT_THREADS);
+            int lo = 0, hi = g.S; // every index < lo is below, every index >= hi is not
+            while (hi > lo) {
+                const int step = (hi - lo + 31) >> 5, at = lo + (lane + 1) * step - 1;
+                const bool lt = at < hi && (unsigned)(g.keys[at] >> 32) < kt;
+                const int n = __popc(__ballot_sync(0xffffffffu, lt));
+                const int nlo = min(lo + n * step, hi);
+                hi = min(hi, lo + (n + 1) * step - 1);
+                lo = nlo;
+            }
+            if (lane == 0)
+                s_lo[w] = lo;
         }
+        __syncthreads();
+        const int lo = s_lo[0], m = s_lo[1] - lo;
+        const bool staged = m <= GT_STAGE;
+        if (staged)
+            for (int i = t; i < m; i += GT_THREADS)
+                s_key[i] = (unsigned)(g.keys[lo + i] >> 32);
+        __syncthreads();
+        const int k = k0 + t;
+        {
+            int l = 0, h = m; // first of the slice not below k
+            while (l < h) {
+                const int mid = (l + h) >> 1;
+                const unsigned v = staged ? s_key[mid] : (unsigned)(g.keys[lo + mid] >> 32);
+                if (v < (unsigned)k)
+                    l = mid + 1;
+                else
+                    h = mid;
+            }
+            s_off[t] = lo + l;
+        }
+        if (t == 0)
+            s_off[GT_THREADS] = lo + m;
+        __syncthreads();
+        unsigned int e = 0;
+        if (k < g.nkeys) {
+            const int o0 = s_off[t], o1 = s_off[t + 1];
+            e = __float_as_uint(g.ext[k]); // extents are non-negative: the bits order them
+            const unsigned int u = __float_as_uint(g.tB[k]);
+            const float tB = u ? ord2f(u) : -INFINITY;
+            g.tB[k] = tB;
+            g.off[k] = o0;
+            g.krec[k] = make_int4(o0, o1, (int)e, __float_as_int(tB));
+            if (k == g.nkeys - 1)
+                g.off[g.nkeys] = o1;
+        }
+        e = __reduce_max_sync(0xffffffffu, e);
+        if (lane == 0 && e)
+            atomicMax(g.ext_max, e);
+        return;
+    }
+    b -= g.kblocks;
+    if (b < g.rblocks) {
+        const int i = b * GT_THREADS + t;
+        if (i >= g.S)
+            return;
+        const int s = (int)(g.keys[i] & 0xffffffffu), p = g.pos[s];
+        g.ids[i] = p;
+        g.gseg[4 * (size_t)i] = g.rec[4 * (size_t)s];
+        g.gseg[4 * (size_t)i + 1] = g.rec[4 * (size_t)s + 1];
+        g.gseg[4 * (size_t)i + 2] = g.rec[4 * (size_t)s + 2];
+        float4 r3 = g.rec[4 * (size_t)s + 3];
+        r3.z = __int_as_float(p);
+        g.gseg[4 * (size_t)i + 3] = r3;
+        return;
+    }
+    // buckets: 256 per step, the running maximum carried over
+    __shared__ float s_w[GT_THREADS / 32];
+    float carry = -INFINITY;
+    for (int i0 = 0; i0 < g.nb; i0 += GT_THREADS) {
+        const int i = i0 + t;
+        const unsigned int u = i < g.nb ? __float_as_uint(g.bpm[i]) : 0u;
+        float v = u ? ord2f(u) : -INFINITY;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const float x = __shfl_up_sync(0xffffffffu, v, o);
+            if (lane >= o)
+                v = fmaxf(v, x);
+        }
+        if (lane == 31)
+            s_w[w] = v;
+        __syncthreads();
+        float all = carry;
+        for (int j = 0; j < GT_THREADS / 32; ++j) {
+            if (j == w)
+                v = fmaxf(v, all); // the warps and steps before
+            all = fmaxf(all, s_w[j]);
+        }
+        if (i < g.nb)
+            g.bpm[i] = v;
+        carry = all;
+        __syncthreads();
     }
 }
 
@@ -677,15 +905,10 @@ __global__ void k_prefix_max(float *__restrict__ v, int n)
 // Arrays back to the pool in the order of `st`, host parts freed.
 static void release_index(tnn_index *ix, cudaStream_t st)
 {
-    void *arrays[] = {ix->pts,   ix->seg,   ix->segTA, ix->segPM, ix->pts_t,
-                      ix->idx_t, ix->g_off, ix->g_ids, ix->g_seg, ix->g_ext,
-                      ix->g_tB,  ix->g_krec, ix->g_bpm, ix->g_ext_max,
-                      ix->pts_k, ix->idx_k, ix->kp_start, ix->pts_m,
-                      ix->idx_m, ix->code_m};
+    void *arrays[] = {ix->mem_seg, ix->mem_grid, ix->pts_t, ix->idx_t, ix->pts_k,
+                      ix->idx_k,   ix->kp_start, ix->pts_m, ix->idx_m, ix->code_m};
     for (void *p : arrays)
         tnn_free(p, st);
-    tnn_free(ix->d_rmax, st);
-    tnn_free(ix->d_tiles, st);
     free(ix->h_tiles);
     if (ix->built)
         cudaEventDestroy(ix->built);
@@ -706,29 +929,51 @@ void tnn_index_release(tnn_index *ix, cudaStream_t st)
         release_index(ix, st);
 }
 
-// The build's second stream per device (non-blocking, created on first
-// use): the grid keys and their sort run there beside the t_A sort.
+// The build's two further streams per device (non-blocking, created on first
+// use): the t_A sort and the grid-key sort run there beside the segment fit.
 #define TNN_BUILD_MAX_DEVICES 64
 static std::mutex g_side_mu;
-static cudaStream_t g_side_stream[TNN_BUILD_MAX_DEVICES];
+static cudaStream_t g_side_stream[TNN_BUILD_MAX_DEVICES][2];
 
-static cudaError_t side_stream(cudaStream_t *out)
+static cudaError_t side_streams(int dev, cudaStream_t out[2])
 {
-    int dev = 0;
-    cudaError_t e = cudaGetDevice(&dev);
-    if (e != cudaSuccess)
-        return e;
     if (dev < 0 || dev >= TNN_BUILD_MAX_DEVICES)
         return cudaErrorInvalidDevice;
     std::lock_guard<std::mutex> lk(g_side_mu);
-    if (!g_side_stream[dev]) {
-        e = cudaStreamCreateWithFlags(&g_side_stream[dev], cudaStreamNonBlocking);
-        if (e != cudaSuccess)
-            return e;
+    for (int i = 0; i < 2; ++i) {
+        if (!g_side_stream[dev][i]) {
+            cudaError_t e = cudaStreamCreateWithFlags(&g_side_stream[dev][i], cudaStreamNonBlocking);
+            if (e != cudaSuccess)
+                return e;
+        }
+        out[i] = g_side_stream[dev][i];
     }
-    *out = g_side_stream[dev];
     return cudaSuccess;
 }
+
+// Events of this host thread on one device, kept between builds: after the
+// validation, its read-back, the t_A sort, the grid keys, the segment fit.
+struct BuildEvents {
+    cudaEvent_t e[5] = {nullptr, nullptr, nullptr, nullptr, nullptr};
+    ~BuildEvents()
+    {
+        for (cudaEvent_t x : e)
+            if (x)
+                cudaEventDestroy(x);
+    }
+    cudaError_t get()
+    {
+        for (cudaEvent_t &x : e)
+            if (!x) {
+                const cudaError_t r = cudaEventCreateWithFlags(&x, cudaEventDisableTiming);
+                if (r != cudaSuccess) {
+                    x = nullptr;
+                    return r;
+                }
+            }
+        return cudaSuccess;
+    }
+};
 
 // Build-time scratch, returned to the pool in stream order.
 struct DevBuf {
@@ -740,6 +985,44 @@ struct DevBuf {
         return tnn_alloc(&p, bytes, s);
     }
     ~DevBuf() { tnn_free(p, st); }
+};
+
+// Consecutive arrays of one allocation, each on a 256-byte boundary: sized
+// first (base NULL), then placed.
+struct Carve {
+    char *base;
+    size_t used = 0;
+    explicit Carve(void *b) : base((char *)b) {}
+    template <typename T> void take(T *&p, size_t count)
+    {
+        if (base)
+            p = (T *)(base + used);
+        used += (count * sizeof(T) + 255) & ~(size_t)255;
+    }
+};
+
+// Page-locked staging of this host thread for the build's uploads and the
+// values it reads back (larger uploads go through pageable memory).
+struct Staging {
+    static constexpr size_t bytes = 1 << 20;
+    unsigned char *p = nullptr;
+    ~Staging()
+    {
+        if (p)
+            cudaFreeHost(p);
+    }
+    cudaError_t get(unsigned char **out)
+    {
+        if (!p) {
+            cudaError_t e = cudaHostAlloc((void **)&p, bytes, cudaHostAllocPortable);
+            if (e != cudaSuccess) {
+                p = nullptr;
+                return e;
+            }
+        }
+        *out = p;
+        return cudaSuccess;
+    }
 };
 
 static float host_ord2f(uint32_t u)
@@ -805,40 +1088,47 @@ static GridBuild grid_geometry(double xmn, double xmx, double ymn, double ymx, d
 // The grid's arrays, zeroed where the key kernel takes maxima.
 static tnn_status grid_alloc(tnn_index *ix, const GridBuild &g, cudaStream_t st)
 {
-    const int S = (int)ix->S, nb = g.nb, nkeys = nb * g.ncell;
-    TNN_CUDA_TRY(tnn_alloc((void **)&ix->g_off, sizeof(int32_t) * (nkeys + 1), st));
-    TNN_CUDA_TRY(tnn_alloc((void **)&ix->g_ids, sizeof(int32_t) * S, st));
-    TNN_CUDA_TRY(tnn_alloc((void **)&ix->g_seg, sizeof(float4) * 4 * (size_t)S, st));
-    TNN_CUDA_TRY(tnn_alloc((void **)&ix->g_ext, sizeof(float) * nkeys, st));
-    TNN_CUDA_TRY(tnn_alloc((void **)&ix->g_tB, sizeof(float) * nkeys, st));
-    TNN_CUDA_TRY(tnn_alloc((void **)&ix->g_bpm, sizeof(float) * nb, st));
-    TNN_CUDA_TRY(tnn_alloc((void **)&ix->g_krec, sizeof(int4) * (size_t)nkeys, st));
-    TNN_CUDA_TRY(tnn_alloc((void **)&ix->g_ext_max, sizeof(float), st));
-    TNN_CUDA_TRY(cudaMemsetAsync(ix->g_ext_max, 0, sizeof(float), st));
-    TNN_CUDA_TRY(cudaMemsetAsync(ix->g_ext, 0, sizeof(float) * nkeys, st));
-    TNN_CUDA_TRY(cudaMemsetAsync(ix->g_tB, 0, sizeof(float) * nkeys, st));
-    TNN_CUDA_TRY(cudaMemsetAsync(ix->g_bpm, 0, sizeof(float) * nb, st));
+    const size_t S = (size_t)ix->S, nb = (size_t)g.nb, nkeys = nb * g.ncell;
+    size_t zeroed = 0;
+    for (int pass = 0; pass < 2; ++pass) {
+        Carve c(ix->mem_grid);
+        c.take(ix->g_ext, nkeys);
+        c.take(ix->g_tB, nkeys);
+        c.take(ix->g_bpm, nb);
+        zeroed = c.used;
+        c.take(ix->g_off, nkeys + 1);
+        c.take(ix->g_ids, S);
+        c.take(ix->g_seg, 4 * S);
+        c.take(ix->g_krec, nkeys);
+        if (pass == 0)
+            TNN_CUDA_TRY(tnn_alloc(&ix->mem_grid, c.used, st));
+    }
+    TNN_CUDA_TRY(cudaMemsetAsync(ix->mem_grid, 0, zeroed, st));
     return TNN_OK;
 }
 
 // The grid from its sorted keys (build ids; pos = t_A position of each).
-static tnn_status build_grid(tnn_index *ix, const unsigned long long *keys, const int32_t *pos,
-                             const GridBuild &g, cudaStream_t st)
+static tnn_status build_grid(tnn_index *ix, const unsigned long long *keys, const float4 *rec,
+                             const int32_t *pos, const GridBuild &g, cudaStream_t st)
 {
-    const int S = (int)ix->S, tb = 256;
-    const int nx = g.nx, ny = g.ny, nb = g.nb;
-    const int nkeys = nb * g.ncell;
-    k_grid_offsets<<<(nkeys + 1 + tb - 1) / tb, tb, 0, st>>>(keys, S, nkeys, ix->g_off);
-    k_grid_ids<<<(S + tb - 1) / tb, tb, 0, st>>>(keys, S, pos, ix->g_ids);
-    k_grid_records<<<(S + tb - 1) / tb, tb, 0, st>>>(ix->seg, ix->g_ids, S, ix->g_seg);
-    k_decode_ord<<<(nkeys + tb - 1) / tb, tb, 0, st>>>((unsigned int *)ix->g_tB, nkeys);
-    k_decode_ord<<<(nb + tb - 1) / tb, tb, 0, st>>>((unsigned int *)ix->g_bpm, nb);
-    k_prefix_max<<<1, 32, 0, st>>>(ix->g_bpm, nb);
-    k_key_records<<<(nkeys + tb - 1) / tb, tb, 0, st>>>(ix->g_off, ix->g_ext, ix->g_tB, nkeys,
-                                                       ix->g_krec);
-    // largest extent (for the search region)
-    k_max_bits<<<std::min((nkeys + tb - 1) / tb, 1024), tb, 0, st>>>(
-        (const unsigned int *)ix->g_ext, nkeys, (unsigned int *)ix->g_ext_max);
+    GridTail a;
+    a.keys = keys;
+    a.rec = rec;
+    a.pos = pos;
+    a.S = (int)ix->S;
+    a.nb = g.nb;
+    a.nkeys = g.nb * g.ncell;
+    a.kblocks = (a.nkeys + GT_THREADS - 1) / GT_THREADS;
+    a.rblocks = (a.S + GT_THREADS - 1) / GT_THREADS;
+    a.off = ix->g_off;
+    a.ids = ix->g_ids;
+    a.gseg = ix->g_seg;
+    a.ext = ix->g_ext;
+    a.tB = ix->g_tB;
+    a.bpm = ix->g_bpm;
+    a.krec = ix->g_krec;
+    a.ext_max = (unsigned int *)ix->g_ext_max;
+    k_grid_tail<<<a.kblocks + a.rblocks + 1, GT_THREADS, 0, st>>>(a);
     TNN_CUDA_TRY(cudaGetLastError());
     GridDesc &G = ix->grid;
     G.x0 = g.x0;
@@ -849,10 +1139,10 @@ static tnn_status build_grid(tnn_index *ix, const unsigned long long *keys, cons
     G.dt = g.dt;
     G.inv_dt = g.inv_dt;
     G.ext_max = ix->g_ext_max;
-    G.nx = nx;
-    G.ny = ny;
+    G.nx = g.nx;
+    G.ny = g.ny;
     G.ncell = g.ncell;
-    G.nb = nb;
+    G.nb = g.nb;
     G.off = ix->g_off;
     G.ids = ix->g_ids;
     G.gseg = ix->g_seg;
@@ -887,17 +1177,13 @@ extern "C" tnn_status tnn_build_segments(const float *d_xyzt, int64_t n,
     }
     TNN_ARG_CHECK(h_traj_off[0] == 0 && h_traj_off[n_traj] == n,
                   "traj_off must start at 0 and end at n");
-    std::vector<int32_t> toff(n_traj + 1), soff(n_traj + 1);
-    int64_t S = 0;
+    int64_t S = 0, nt = 0; // segments; query tiles of up to 32 points of one trajectory
     for (int64_t t = 0; t < n_traj; ++t) {
-        int64_t len = h_traj_off[t + 1] - h_traj_off[t];
+        const int64_t len = h_traj_off[t + 1] - h_traj_off[t];
         TNN_ARG_CHECK(len >= 0, "traj_off must be non-decreasing");
-        toff[t] = (int32_t)h_traj_off[t];
-        soff[t] = (int32_t)S;
-        S += (len + K - 1) / K;
+        S += (uint32_t)(len + K - 1) / (uint32_t)K; // len < 2^31
+        nt += (len + 31) >> 5;
     }
-    toff[n_traj] = (int32_t)n;
-    soff[n_traj] = (int32_t)S;
     cudaStream_t st = (cudaStream_t)stream;
 
     tnn_index *ix = new tnn_index();
@@ -907,6 +1193,7 @@ extern "C" tnn_status tnn_build_segments(const float *d_xyzt, int64_t n,
     ix->n_traj = n_traj;
     ix->S = S;
     ix->K = K;
+    ix->n_tiles = nt;
     for (int i = 0; i < 4; ++i) {
         ix->sigma[i] = params->sigma[i];
         ix->sig_f[i] = (float)params->sigma[i];
@@ -914,132 +1201,146 @@ extern "C" tnn_status tnn_build_segments(const float *d_xyzt, int64_t n,
     for (int i = 0; i < 3; ++i)
         ix->ssq_f[i] = (float)sqrt(params->sigma[i]);
 
-    const int s2 = tnn_next_pow2_sort(S);
-    DevBuf toff_d, soff_d, rec_d, keys_d, flags_d;
-    cudaError_t e = cudaSuccess;
-#define ALLOC(ptr, bytes)                                                     \
-    if (e == cudaSuccess)                                                     \
-        e = tnn_alloc((void **)&(ptr), (bytes), st);
-    ALLOC(ix->pts, sizeof(float4) * n);
-    ALLOC(ix->seg, sizeof(float4) * 4 * S);
-    ALLOC(ix->segTA, sizeof(float) * S);
-    ALLOC(ix->segPM, sizeof(float) * S);
-#undef ALLOC
-    if (e == cudaSuccess)
-        e = toff_d.alloc(sizeof(int32_t) * (n_traj + 1), st);
-    if (e == cudaSuccess)
-        e = soff_d.alloc(sizeof(int32_t) * (n_traj + 1), st);
-    if (e == cudaSuccess)
-        e = rec_d.alloc(sizeof(float4) * 4 * S, st);
-    if (e == cudaSuccess)
-        e = keys_d.alloc(sizeof(unsigned long long) * s2, st);
-    if (e == cudaSuccess)
-        e = flags_d.alloc(sizeof(unsigned int) * 12, st);
+    // What goes up in one copy: the header, trajectory and segment offsets
+    // per trajectory, tile starts.
+    const size_t up_words = META_WORDS + 2 * (size_t)(n_traj + 1) + (size_t)(nt + 1);
+    static thread_local Staging t_stage;
+    unsigned char *stage = nullptr;
+    std::vector<unsigned int> big;
+    cudaError_t e = t_stage.get(&stage);
+    unsigned int *up = (unsigned int *)stage;
+    if (e == cudaSuccess && up_words * 4 > Staging::bytes - 64) {
+        big.resize(up_words);
+        up = big.data();
+    }
+    ix->h_tiles = (int32_t *)malloc(sizeof(int32_t) * (size_t)(nt + 1));
+    if (e != cudaSuccess || !ix->h_tiles) {
+        free_index(ix);
+        tnn_set_error("index allocation failed (host tables)");
+        return TNN_ERR_OOM;
+    }
+    int32_t *toff_h = (int32_t *)(up + META_WORDS), *soff_h = toff_h + n_traj + 1;
+    {
+        static const unsigned int meta_init[META_WORDS] = {0u, 0u, 0xffffffffu, 0u, 0xffffffffu, 0u,
+                                                           0xffffffffu, 0u, 0xffffffffu, 0u};
+        memcpy(up, meta_init, sizeof(meta_init));
+        int64_t j = 0, sj = 0;
+        for (int64_t t = 0; t < n_traj; ++t) {
+            const int64_t a = h_traj_off[t], b = h_traj_off[t + 1];
+            toff_h[t] = (int32_t)a;
+            soff_h[t] = (int32_t)sj;
+            sj += (uint32_t)(b - a + K - 1) / (uint32_t)K;
+            for (int64_t r = a; r < b; r += 32)
+                ix->h_tiles[j++] = (int32_t)r;
+        }
+        toff_h[n_traj] = (int32_t)n;
+        soff_h[n_traj] = (int32_t)S;
+        ix->h_tiles[nt] = (int32_t)n;
+        memcpy(soff_h + n_traj + 1, ix->h_tiles, sizeof(int32_t) * (size_t)(nt + 1));
+    }
+
+    // One allocation for what stays before the grid's geometry is known, one
+    // for the build's scratch.
+    const int s2 = tnn_next_pow2_sort(S), nblk = (int)((S + 1023) / 1024);
+    DevBuf scratch;
+    unsigned int *d_up = nullptr;
+    float4 *rec = nullptr;
+    unsigned long long *keys = nullptr, *keys2 = nullptr;
+    int32_t *pos = nullptr;
+    float *bmax = nullptr;
+    int4 *range = nullptr;
+    for (int pass = 0; pass < 2 && e == cudaSuccess; ++pass) {
+        Carve c(ix->mem_seg), x(scratch.p);
+        c.take(ix->pts, (size_t)n);
+        c.take(ix->seg, 4 * (size_t)S);
+        c.take(ix->segTA, (size_t)S);
+        c.take(ix->segPM, (size_t)S);
+        c.take(d_up, up_words);
+        x.take(rec, 4 * (size_t)S);
+        x.take(keys, (size_t)s2);
+        x.take(keys2, (size_t)s2);
+        x.take(pos, (size_t)S);
+        x.take(bmax, (size_t)nblk);
+        x.take(range, (size_t)S);
+        if (pass == 0) {
+            e = tnn_alloc(&ix->mem_seg, c.used, st);
+            if (e == cudaSuccess)
+                e = scratch.alloc(x.used, st);
+        }
+    }
     if (e != cudaSuccess) {
         free_index(ix);
         tnn_set_error("index allocation failed: %s", cudaGetErrorString(e));
         return e == cudaErrorMemoryAllocation ? TNN_ERR_OOM : TNN_ERR_CUDA;
     }
-    // flags_d: [0] validation flags, [1] largest |scaled coordinate| bits,
-    // [2..9] point bounding box (ordered min, max per axis), [10..11] summed
-    // segment duration (double)
-    static const unsigned int meta_init[12] = {0u, 0u, 0xffffffffu, 0u, 0xffffffffu, 0u,
-                                               0xffffffffu, 0u, 0xffffffffu, 0u, 0u, 0u};
-    unsigned int *flag = (unsigned int *)flags_d.p;
-    unsigned long long *keys = (unsigned long long *)keys_d.p;
+    unsigned int *meta = d_up;
+    const int32_t *toff = (const int32_t *)(d_up + META_WORDS), *soff = toff + n_traj + 1;
+    ix->d_tiles = (int32_t *)(soff + n_traj + 1);
+    ix->d_rmax = meta + META_RMAX;
+    ix->g_ext_max = (float *)(meta + META_EXT);
     const int tb = 256;
-    e = cudaMemcpyAsync(ix->pts, d_xyzt, sizeof(float4) * n, cudaMemcpyDeviceToDevice, st);
+    static thread_local BuildEvents t_events[TNN_BUILD_MAX_DEVICES];
+    cudaStream_t side[2] = {nullptr, nullptr};
+    e = side_streams(ix->device, side);
+    BuildEvents &ev = t_events[e == cudaSuccess ? ix->device : 0];
     if (e == cudaSuccess)
-        e = cudaMemcpyAsync(toff_d.p, toff.data(), sizeof(int32_t) * (n_traj + 1),
-                            cudaMemcpyHostToDevice, st);
-    if (e == cudaSuccess)
-        e = cudaMemcpyAsync(soff_d.p, soff.data(), sizeof(int32_t) * (n_traj + 1),
-                            cudaMemcpyHostToDevice, st);
-    if (e == cudaSuccess)
-        e = cudaMemcpyAsync(flag, meta_init, sizeof(meta_init), cudaMemcpyHostToDevice, st);
-    // query tiles of the self-queries: runs of up to 32 points of one trajectory
-    {
-        int64_t nt = 0;
-        for (int64_t t = 0; t < n_traj; ++t)
-            nt += (h_traj_off[t + 1] - h_traj_off[t] + 31) / 32;
-        ix->n_tiles = nt;
-        ix->h_tiles = (int32_t *)malloc(sizeof(int32_t) * (size_t)(nt + 1));
-        if (!ix->h_tiles) {
-            free_index(ix);
-            tnn_set_error("index allocation failed (host tile table)");
-            return TNN_ERR_OOM;
-        }
-        int64_t j = 0;
-        for (int64_t t = 0; t < n_traj; ++t)
-            for (int64_t r = h_traj_off[t]; r < h_traj_off[t + 1]; r += 32)
-                ix->h_tiles[j++] = (int32_t)r;
-        ix->h_tiles[nt] = (int32_t)n;
-    }
-    if (e == cudaSuccess)
-        e = tnn_alloc((void **)&ix->d_tiles, sizeof(int32_t) * (size_t)(ix->n_tiles + 1), st);
-    if (e == cudaSuccess)
-        e = cudaMemcpyAsync(ix->d_tiles, ix->h_tiles, sizeof(int32_t) * (size_t)(ix->n_tiles + 1),
-                            cudaMemcpyHostToDevice, st);
-    if (e == cudaSuccess)
-        e = tnn_alloc((void **)&ix->d_rmax, sizeof(unsigned int), st);
-    if (e == cudaSuccess)
-        e = cudaMemsetAsync(ix->d_rmax, 0, sizeof(unsigned int), st);
+        e = ev.get();
     if (e == cudaSuccess)
         e = cudaEventCreateWithFlags(&ix->built, cudaEventDisableTiming);
+    if (e == cudaSuccess)
+        e = cudaMemcpyAsync(d_up, up, up_words * 4, cudaMemcpyHostToDevice, st);
     if (e != cudaSuccess) {
         free_index(ix);
         tnn_set_error("index upload failed: %s", cudaGetErrorString(e));
         return TNN_ERR_CUDA;
     }
     const int ni = (int)n, Si = (int)S, Ti = (int)n_traj;
-    // ---- validation, and what the grid geometry needs: the build's only
-    // host synchronisation; everything after it is enqueued at once
-    k_validate_points<<<(ni + tb - 1) / tb, tb, 0, st>>>(
-        ix->pts, ni, ix->ssq_f[0], ix->ssq_f[1], ix->ssq_f[2], flag, flag + 1);
-    k_validate_traj<<<(int)(((int64_t)Ti * 32 + tb - 1) / tb), tb, 0, st>>>(
-        ix->pts, (const int32_t *)toff_d.p, Ti, K, flag, (double *)(flag + 10));
-    k_point_bbox<<<(int)std::min<int64_t>((ix->n + tb - 1) / tb, 608), tb, 0, st>>>(
-        ix->pts, (int)ix->n, flag + 2);
-    // The values come back through a page-locked buffer of this host thread
-    // and an event: the segment fit (which needs neither the geometry nor
-    // the validation result) is enqueued before the host waits, so it runs while the
-    // host chooses the geometry and enqueues the rest.  Invalid input is
-    // still reported here; the fit's output is then dropped.
-    static thread_local unsigned int *t_meta = nullptr;
-    unsigned int hm[12];
-    cudaEvent_t ev_meta = nullptr;
+    // ---- validation, and what the grid geometry needs.  The values come
+    // back through page-locked memory and an event, the build's only host
+    // synchronisation; the t_A sort (on the first side stream) and the
+    // segment fit need neither the geometry nor the validation result and run
+    // while the host waits, chooses the geometry and enqueues the rest.
+    // Invalid input is still reported here; their output is then dropped.
+    const int pblocks = (int)std::min<int64_t>((n + 4 * VAL_THREADS - 1) / (4 * VAL_THREADS), 608);
+    k_validate<<<pblocks + (Ti + VAL_THREADS / 32 - 1) / (VAL_THREADS / 32), VAL_THREADS, 0, st>>>(
+        (const float4 *)d_xyzt, ix->pts, ni, ix->ssq_f[0], ix->ssq_f[1], ix->ssq_f[2], toff, soff, Ti, K, pblocks,
+        Si, s2, range, keys, meta);
+    unsigned int hm[META_READ], *back = (unsigned int *)(stage + Staging::bytes - 64);
     e = cudaGetLastError();
-    if (e == cudaSuccess && !t_meta)
-        e = cudaHostAlloc((void **)&t_meta, sizeof(hm), cudaHostAllocPortable);
     if (e == cudaSuccess)
-        e = cudaEventCreateWithFlags(&ev_meta, cudaEventDisableTiming);
+        e = cudaEventRecord(ev.e[0], st);
     if (e == cudaSuccess)
-        e = cudaMemcpyAsync(t_meta, flag, sizeof(hm), cudaMemcpyDeviceToHost, st);
+        e = cudaMemcpyAsync(back, meta, sizeof(hm), cudaMemcpyDeviceToHost, st);
     if (e == cudaSuccess)
-        e = cudaEventRecord(ev_meta, st);
+        e = cudaEventRecord(ev.e[1], st);
+    if (e == cudaSuccess)
+        e = cudaStreamWaitEvent(side[0], ev.e[0], 0);
     const double q0 = sqrt(params->sigma[0]), q1 = sqrt(params->sigma[1]);
     if (e == cudaSuccess) {
-        k_segment_fit<<<(int)(((int64_t)Si * SF_LANES + tb - 1) / tb), tb, 0, st>>>(
-            ix->pts, (const int32_t *)toff_d.p, (const int32_t *)soff_d.p, Ti, Si, K,
-            q0, q1, sqrt(params->sigma[2]), (float4 *)rec_d.p, keys, ix->d_rmax);
+        if (sort_by_value(keys, s2, 32, side[0]) != TNN_OK)
+            e = cudaErrorUnknown;
+        else
+            e = cudaEventRecord(ev.e[2], side[0]);
+    }
+    if (e == cudaSuccess) {
+        k_segment_fit<<<(Si + SF_THREADS - 1) / SF_THREADS, SF_THREADS, 0, st>>>(
+            ix->pts, range, Si, q0, q1, sqrt(params->sigma[2]), rec, ix->d_rmax);
         e = cudaGetLastError();
     }
     if (e == cudaSuccess)
-        e = cudaEventSynchronize(ev_meta);
-    if (ev_meta)
-        cudaEventDestroy(ev_meta);
+        e = cudaEventSynchronize(ev.e[1]);
     if (e != cudaSuccess) {
         free_index(ix);
         tnn_set_error("index validation failed: %s", cudaGetErrorString(e));
         return TNN_ERR_CUDA;
     }
-    memcpy(hm, t_meta, sizeof(hm));
-    if (hm[0] & BAD_VALUE) {
+    memcpy(hm, back, sizeof(hm));
+    if (hm[META_FLAG] & BAD_VALUE) {
         free_index(ix);
         tnn_set_error("non-finite or too large (|v| > 1e15) coordinate in input");
         return TNN_ERR_INVALID_ARG;
     }
-    if (hm[0] & BAD_ORDER) {
+    if (hm[META_FLAG] & BAD_ORDER) {
         free_index(ix);
         tnn_set_error("times are not sorted inside a trajectory");
         return TNN_ERR_INVALID_ARG;
@@ -1054,66 +1355,42 @@ extern "C" tnn_status tnn_build_segments(const float *d_xyzt, int64_t n,
     const GridBuild geo = grid_geometry(q0 * ix->bb_lo[0], q0 * ix->bb_hi[0], q1 * ix->bb_lo[1],
                                         q1 * ix->bb_hi[1], ix->bb_lo[3], ix->bb_hi[3], dur, S);
 
-    // ---- segments, their t_A order, the running maximum of t_B, the grid.
-    // The grid keys come from the build-order records, so their sort runs on
-    // a second stream beside the t_A sort; the two join before the grid's
-    // offsets and records.
-    {
-        DevBuf keys2_d, pos_d, bmax_d;
-        cudaStream_t st2 = nullptr;
-        cudaEvent_t ev_fit = nullptr, ev_keys = nullptr;
-        const int nblk = (Si + 1023) / 1024;
-        e = side_stream(&st2);
+    // ---- the grid-key sort and, after the fit, the grid's per-key aggregates
+    // on the second side stream; the t_A order and the running maximum of t_B
+    // on `st`; all join before the grid's offsets and records
+    e = cudaStreamWaitEvent(side[1], ev.e[0], 0);
+    if (e == cudaSuccess) {
+        k_grid_sort_keys<<<(s2 + tb - 1) / tb, tb, 0, side[1]>>>(ix->pts, range, Si, s2, q0, q1, geo, keys2);
+        int bits = 1;
+        while ((1ll << bits) - 1 < (long long)geo.nb * geo.ncell) // all ones stays free for the padding
+            ++bits;
+        if (sort_by_value(keys2, s2, bits, side[1]) != TNN_OK)
+            e = cudaErrorUnknown;
+    }
+    tnn_status gs = e == cudaSuccess ? grid_alloc(ix, geo, st) : TNN_ERR_CUDA;
+    if (gs == TNN_OK) {
+        e = cudaEventRecord(ev.e[4], st); // the fit and the grid's zeroed arrays
         if (e == cudaSuccess)
-            e = keys2_d.alloc(sizeof(unsigned long long) * s2, st);
-        if (e == cudaSuccess)
-            e = pos_d.alloc(sizeof(int32_t) * (size_t)Si, st);
-        if (e == cudaSuccess)
-            e = bmax_d.alloc(sizeof(float) * (size_t)nblk, st);
-        if (e == cudaSuccess)
-            e = cudaEventCreateWithFlags(&ev_fit, cudaEventDisableTiming);
-        if (e == cudaSuccess)
-            e = cudaEventCreateWithFlags(&ev_keys, cudaEventDisableTiming);
-        tnn_status gs = e == cudaSuccess ? grid_alloc(ix, geo, st) : TNN_ERR_CUDA;
-        if (gs == TNN_OK) {
-            unsigned long long *keys2 = (unsigned long long *)keys2_d.p;
-            e = cudaEventRecord(ev_fit, st); // the fit (enqueued above) and the grid's zeroing
-            if (e == cudaSuccess)
-                e = cudaStreamWaitEvent(st2, ev_fit, 0);
-            if (e == cudaSuccess) {
-                // second stream: grid keys of the build-order records, sorted
-                k_fill<<<(s2 - Si + tb - 1) / tb + 1, tb, 0, st2>>>(keys2, Si, s2);
-                k_grid_keys<<<(Si + tb - 1) / tb, tb, 0, st2>>>(
-                    (const float4 *)rec_d.p, Si, geo, keys2, (unsigned int *)ix->g_ext,
-                    (unsigned int *)ix->g_tB, (unsigned int *)ix->g_bpm);
-                tnn_bitonic_sort(keys2, s2, st2);
-                e = cudaEventRecord(ev_keys, st2);
-            }
-            // this stream: the t_A order and the running maximum of t_B
-            k_fill<<<(s2 - Si + tb - 1) / tb + 1, tb, 0, st>>>(keys, Si, s2);
-            tnn_bitonic_sort(keys, s2, st);
-            k_gather_segments<<<(Si + tb - 1) / tb, tb, 0, st>>>(keys, (const float4 *)rec_d.p, Si,
-                                                                 ix->seg, ix->segTA, (int32_t *)pos_d.p);
-            k_pm_block_max<<<nblk, 1024, 0, st>>>(ix->seg, Si, (float *)bmax_d.p);
-            k_pm_apply<<<nblk, 1024, 0, st>>>(ix->seg, Si, (const float *)bmax_d.p, ix->segPM);
-            if (e == cudaSuccess)
-                e = cudaStreamWaitEvent(st, ev_keys, 0);
-            if (e == cudaSuccess)
-                gs = build_grid(ix, keys2, (const int32_t *)pos_d.p, geo, st);
-            else
-                gs = TNN_ERR_CUDA;
+            e = cudaStreamWaitEvent(side[1], ev.e[4], 0);
+        if (e == cudaSuccess) {
+            k_grid_extents<<<(Si + 127) / 128, 128, 0, side[1]>>>(
+                rec, Si, geo, (unsigned int *)ix->g_ext, (unsigned int *)ix->g_tB, (unsigned int *)ix->g_bpm);
+            e = cudaEventRecord(ev.e[3], side[1]);
         }
-        if (ev_fit)
-            cudaEventDestroy(ev_fit);
-        if (ev_keys)
-            cudaEventDestroy(ev_keys);
-        if (gs != TNN_OK) {
-            if (e != cudaSuccess)
-                tnn_set_error("index build failed: %s", cudaGetErrorString(e));
-            cudaStreamSynchronize(st2);
-            free_index(ix);
-            return gs;
+        if (e == cudaSuccess)
+            e = cudaStreamWaitEvent(st, ev.e[2], 0);
+        if (e == cudaSuccess) {
+            k_gather_segments<<<nblk, 1024, 0, st>>>(keys, rec, Si, ix->seg, ix->segTA, pos, bmax);
+            k_pm_apply<<<nblk, 1024, 0, st>>>(ix->seg, Si, bmax, ix->segPM);
+            e = cudaStreamWaitEvent(st, ev.e[3], 0);
         }
+        gs = e == cudaSuccess ? build_grid(ix, keys2, rec, pos, geo, st) : TNN_ERR_CUDA;
+    }
+    if (gs != TNN_OK) {
+        if (e != cudaSuccess)
+            tnn_set_error("index build failed: %s", cudaGetErrorString(e));
+        free_index(ix); // waits for the device, the side streams included
+        return gs;
     }
     // The build runs on after this call returns (stream order); a failure
     // there surfaces at the next synchronising call.

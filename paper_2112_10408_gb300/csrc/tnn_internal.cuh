@@ -59,6 +59,7 @@ struct GridDesc {
 
 struct tnn_index {
     int device;
+    void *mem_seg, *mem_grid; // the allocations that hold the arrays below
     int64_t n;      // points
     int64_t n_traj; // trajectories
     int64_t S;      // segments
