@@ -143,6 +143,8 @@ __global__ void __launch_bounds__(TNN_WARPS_PER_CTA * 32, TNN_WARP_MINB)
     __shared__ __align__(16) WarpSmem smem[TNN_WARPS_PER_CTA];
     const int lane = threadIdx.x & 31;
     WarpSmem &S = smem[threadIdx.x >> 5];
+    pdl_trigger();
+    pdl_wait();
 
     unsigned nfb = *(volatile unsigned *)&L.scr->n_fallback;
     if ((long long)nfb > L.fb_cap)
@@ -598,8 +600,9 @@ static __device__ unsigned int g_search_fault;
 __global__ void __launch_bounds__(TNN_WARPS_PER_CTA * 32)
     k_fallback_exact(const __grid_constant__ KnnLaunch L)
 {
-    // The kernels before this one on the stream have completed: their flags
-    // are final.  Nothing below sets a flag.
+    // After the wait the kernels before this one on the stream have completed:
+    // their flags are final.  Nothing below sets a flag.
+    pdl_wait();
     if (blockIdx.x == 0 && threadIdx.x == 0) {
         const unsigned f = *(volatile unsigned *)&L.scr->status;
         if (f)

@@ -571,6 +571,7 @@ __global__ void __launch_bounds__(GKA_WARPS * 32) k_gkamlp(const __grid_constant
     float *s_part = s_w + P;
     __syncthreads();
     const float *W1 = s_w, *b1 = s_w + 3 * H, *W2 = s_w + 4 * H, *b2 = s_w + 7 * H;
+    pdl_trigger();
     // the update kernel that follows on the stream reads the new count
     if (a.step_inc && blockIdx.x == 0 && threadIdx.x == 0)
         *a.step_inc += 1;
@@ -714,6 +715,7 @@ __global__ void __launch_bounds__(GKAMLP_SUM * 32) k_gkamlp_adam(const __grid_co
     __shared__ float s_sum[GKAMLP_SUM][32];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int i = blockIdx.x * 32 + lane;
+    pdl_wait();
     float g = 0.f;
     if (i <= a.P) {
 #pragma unroll 8
@@ -944,7 +946,7 @@ extern "C" tnn_status tnn_gkamlp_train_step(tnn_gkamlp *g, const tnn_index *ix, 
         d.eps = opt->eps;
         d.wd = opt->weight_decay;
     }
-    k_gkamlp_adam<<<(g->P + 1 + 31) / 32, GKAMLP_SUM * 32, 0, st>>>(d);
-    TNN_CUDA_TRY(cudaGetLastError());
+    TNN_CUDA_TRY(launch_dependent<GkaMlpAdamArgs>(k_gkamlp_adam, (unsigned)((g->P + 1 + 31) / 32),
+                                                  GKAMLP_SUM * 32, 0, st, d));
     return TNN_OK;
 }

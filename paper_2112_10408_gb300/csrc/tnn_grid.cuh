@@ -368,6 +368,7 @@ __global__ void __launch_bounds__(TNN_WARPS_PER_CTA * 32, TileCtas<NL>::value)
     TileSmem<NL> &S = *(TileSmem<NL> *)ws;
     unsigned long long *Kw = (unsigned long long *)ws;
     const int seed_cell = tg_seed_cell[lane];
+    pdl_trigger();
 
     unsigned n_q = 0, n_lb = 0, n_pairs = 0, n_segs = 0, n_fp = 0;
     for (;;) {

@@ -199,6 +199,37 @@ struct KnnLaunch {
     int32_t pad2_;
 };
 
+// Programmatic dependent launch.  A kernel that calls pdl_trigger lets the
+// next kernel of its stream, if that was launched with launch_dependent, take
+// SMs as they fall free and set itself up; pdl_wait holds such a kernel until
+// every kernel before it has completed and its writes are visible (a no-op in
+// a kernel launched plainly).  Every kernel launched with launch_dependent
+// calls pdl_wait in all of its threads before it touches what an earlier
+// kernel writes.
+__device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
+// Launch `kern` behind the stream's previous kernel without waiting for its
+// end (see above); plainly while the stream is being captured.
+template <typename Arg>
+inline cudaError_t launch_dependent(void (*kern)(const Arg), unsigned grid, unsigned block, size_t smem,
+                                    cudaStream_t st, const Arg &arg, dim3 grid3 = dim3(0))
+{
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    cudaStreamIsCapturing(st, &cap);
+    cudaLaunchAttribute at;
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t c = {};
+    c.gridDim = grid3.x ? grid3 : dim3(grid);
+    c.blockDim = dim3(block);
+    c.dynamicSmemBytes = smem;
+    c.stream = st;
+    c.attrs = &at;
+    c.numAttrs = cap == cudaStreamCaptureStatusNone ? 1 : 0;
+    return cudaLaunchKernelEx(&c, kern, arg);
+}
+
 // Ascending sort of n2 (a power of two, >= 2048) 64-bit keys in place
 // (tnn_index.cu); tnn_next_pow2_sort gives the n2 for n keys.
 int tnn_next_pow2_sort(int64_t n);

@@ -280,14 +280,13 @@ static tnn_status finish_search(const KnnLaunch &L, cudaStream_t st, bool prof, 
         const TileKernel kern = L.k_max <= 16 ? k_tnn_warp<1> : L.k_max <= 32 ? k_tnn_warp<2> : k_tnn_warp<4>;
         int nbw = 0;
         TNN_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nbw, kern, TNN_WARPS_PER_CTA * 32, 0));
-        kern<<<(unsigned)(std::max(nbw, 1) * g_num_sms), TNN_WARPS_PER_CTA * 32, 0, st>>>(L);
+        TNN_CUDA_TRY(launch_dependent<KnnLaunch>(kern, (unsigned)(std::max(nbw, 1) * g_num_sms),
+                                                 TNN_WARPS_PER_CTA * 32, 0, st, L));
     }
-    TNN_CUDA_TRY(cudaGetLastError());
     if (prof)
         TNN_CUDA_TRY(cudaEventRecord(pr.e[2], st));
-    k_fallback_exact<<<(unsigned)g_num_sms, TNN_WARPS_PER_CTA * 32,
-                       fb_exact_smem_per_warp(L.L_max) * TNN_WARPS_PER_CTA, st>>>(L);
-    TNN_CUDA_TRY(cudaGetLastError());
+    TNN_CUDA_TRY(launch_dependent<KnnLaunch>(k_fallback_exact, (unsigned)g_num_sms, TNN_WARPS_PER_CTA * 32,
+                                             fb_exact_smem_per_warp(L.L_max) * TNN_WARPS_PER_CTA, st, L));
     if (prof) {
         TNN_CUDA_TRY(cudaEventRecord(pr.e[3], st));
         g_prof_ev.push_back(pr);

@@ -148,6 +148,7 @@ __global__ void __launch_bounds__(MLP_FWD_THREADS, 2) k_mlp_fwd_tc(const __grid_
     const long long Bp = (a.B + 15) & ~15ll;
     const bool valid = r < a.B;
     const bool train = a.T != nullptr;
+    pdl_trigger();
 
     if (t == 0) {
         for (int i = 0; i < 8; ++i)
@@ -482,10 +483,14 @@ __global__ void __launch_bounds__(MLP_ROWS, 1) k_mlp_dw1_tc(const __grid_constan
         asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(su32(bar)));
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         *s_err = 0;
-        // the AdamW kernel that follows on the stream reads the new count
-        if (a.step_inc && blockIdx.x == 0 && blockIdx.y == 0 && blockIdx.z == 0)
-            *a.step_inc += 1;
     }
+    pdl_trigger();
+    // Before the TMEM allocation: a CTA that held columns here while it waits
+    // could keep a forward CTA on its SM from getting its own.
+    pdl_wait();
+    // the AdamW kernel that follows on the stream reads the new count
+    if (t == 0 && a.step_inc && blockIdx.x == 0 && blockIdx.y == 0 && blockIdx.z == 0)
+        *a.step_inc += 1;
     if (warp == 0) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;"
                      ::"r"(su32(tmem_slot)), "r"(a.tmem_cols));
@@ -660,6 +665,9 @@ __global__ void __launch_bounds__(MLP_INF_THREADS, 1) k_mlp_infer_tc(const __gri
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     const uint32_t tmem = *tmem_slot;
     bool w_seen = false;
+    // The weights above come from no kernel right before this one when it is
+    // launched dependently (tnn_nowcast: behind the context features); X does.
+    pdl_wait();
 
     if (t < MLP_INF_LOADERS) {
         // ---- loaders: rows t and t + 64 of each tile

@@ -123,6 +123,7 @@ __global__ void __launch_bounds__(CF_WARPS * 32, CF_CTAS)
     constexpr int Q = 4 / R;
     __shared__ __align__(16) uint32_t s_feat[CF_WARPS][128 * 3];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    pdl_trigger();
     // A CTA answers one run of consecutive queries, whose neighbours overlap.
     constexpr int step = CF_WARPS * Q;
     const int64_t per = (m + (int64_t)gridDim.x * step - 1) / ((int64_t)gridDim.x * step) * step;
@@ -213,6 +214,7 @@ __global__ void __launch_bounds__(CF_WARPS * 32, 5)
     // (32 >> lg) queries x k neighbours x 3 words, at most 128 neighbours
     __shared__ __align__(16) uint32_t s_feat[CF_WARPS][128 * 3];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    pdl_trigger();
     const int G = 1 << lg, nq = 32 >> lg, ql = lane >> lg, r0 = lane & (G - 1);
     const int64_t q0 = ((int64_t)blockIdx.x * CF_WARPS + warp) * nq;
     if (q0 >= m) // the same for the whole warp
@@ -391,6 +393,7 @@ struct AdamArgs {
 __global__ void k_adamw(const __grid_constant__ AdamArgs a)
 {
     __shared__ float s_bc[2];
+    pdl_wait();
     if (threadIdx.x == 0 && !a.grad_out) {
         // 1 - beta^t = -expm1(t log1p(beta - 1)): beta - 1 is exact in FP32
         // and neither step cancels, so no FP64 is needed
@@ -773,8 +776,10 @@ static tnn_status mlp_setup()
     return TNN_OK;
 }
 
+// after_features: the stream's last kernel is the one that wrote d_x, and
+// the weights were complete before that one began.
 static tnn_status mlp_forward_impl(const tnn_mlp *n, const uint16_t *d_x, long long B,
-                                   float *d_y, const float *d_t, cudaStream_t st)
+                                   float *d_y, const float *d_t, cudaStream_t st, bool after_features = false)
 {
     TNN_ARG_CHECK(((uintptr_t)d_x & 15) == 0, "X must be 16-byte aligned");
     tnn_status s = mlp_setup();
@@ -812,9 +817,14 @@ static tnn_status mlp_forward_impl(const tnn_mlp *n, const uint16_t *d_x, long l
         TNN_CUDA_TRY(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
         a.tmem_cols = tmem_cols_for(2 * n->dh);
         const long long tiles = (B + MLP_ROWS - 1) / MLP_ROWS;
-        k_mlp_infer_tc<<<(unsigned)std::min<long long>(tiles, nsm), MLP_INF_THREADS,
-                         mlp_infer_smem(n->d_in, n->dh), st>>>(a);
-        TNN_CUDA_TRY(cudaGetLastError());
+        const unsigned grid = (unsigned)std::min<long long>(tiles, nsm);
+        if (after_features) {
+            TNN_CUDA_TRY(launch_dependent<MlpFwdArgs>(k_mlp_infer_tc, grid, MLP_INF_THREADS,
+                                                      mlp_infer_smem(n->d_in, n->dh), st, a));
+        } else {
+            k_mlp_infer_tc<<<grid, MLP_INF_THREADS, mlp_infer_smem(n->d_in, n->dh), st>>>(a);
+            TNN_CUDA_TRY(cudaGetLastError());
+        }
         return TNN_OK;
     }
     // Training: hidden units split over a cluster while that still gives every
@@ -882,8 +892,8 @@ static tnn_status mlp_backward_impl(tnn_mlp *n, const uint16_t *d_x, long long B
     d.err = n->err;
     d.step_inc = opt ? n->step : nullptr;
     dim3 grid((unsigned)((n->dh + 127) / 128), (unsigned)((n->d_in + 255) / 256), (unsigned)splits1);
-    k_mlp_dw1_tc<<<grid, MLP_ROWS, tc_smem_request(mlp_dw1_smem(), d.tmem_cols), st>>>(d);
-    TNN_CUDA_TRY(cudaGetLastError());
+    TNN_CUDA_TRY(launch_dependent<MlpDw1Args>(k_mlp_dw1_tc, 0, MLP_ROWS,
+                                              tc_smem_request(mlp_dw1_smem(), d.tmem_cols), st, d, grid));
     AdamArgs a;
     memset(&a, 0, sizeof(a));
     a.w = n->w;
@@ -909,8 +919,7 @@ static tnn_status mlp_backward_impl(tnn_mlp *n, const uint16_t *d_x, long long B
         a.wd = opt->weight_decay;
         a.step = n->step;
     }
-    k_adamw<<<(unsigned)((n->P + 255) / 256), 256, 0, st>>>(a);
-    TNN_CUDA_TRY(cudaGetLastError());
+    TNN_CUDA_TRY(launch_dependent<AdamArgs>(k_adamw, (unsigned)((n->P + 255) / 256), 256, 0, st, a));
     return TNN_OK;
 }
 
@@ -982,7 +991,8 @@ extern "C" tnn_status tnn_nowcast(const tnn_index *ix, const float *d_wind,
         s = tnn_context_features(ix, d_wind, d_q, m, idx, d2, k, h_mean, h_std, idw_eps,
                                  feat, mlp ? nullptr : d_uv, stream);
     if (s == TNN_OK && mlp)
-        s = tnn_mlp_forward(mlp, feat, m, d_uv, stream);
+        s = m < (1ll << 31) / 512 ? mlp_forward_impl(mlp, feat, m, d_uv, nullptr, st, true)
+                                  : tnn_mlp_forward(mlp, feat, m, d_uv, stream); // refused there
     tnn_free(idx, st);
     if (d2)
         tnn_free(d2, st);
