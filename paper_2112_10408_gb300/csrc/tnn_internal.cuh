@@ -290,6 +290,8 @@ tnn_status tnn_launch_search(const KnnLaunch &L, bool brute,
 // and the warp-per-query and exact kernels over what it handed over.
 tnn_status tnn_launch_tiles(const KnnLaunch &L, cudaStream_t stream);
 tnn_status tnn_launch_finish(const KnnLaunch &L, cudaStream_t stream);
+// SMs of a device (0: unknown device), asked once (tnn_knn.cu).
+int tnn_num_sms(int dev);
 size_t tnn_search_smem_per_warp(int L_max, int kseg_max, int mode);
 
 // Search faults flagged on the device since the last report: synchronise

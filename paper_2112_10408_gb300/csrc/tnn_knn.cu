@@ -51,6 +51,7 @@
 #include <string.h>
 
 #include <algorithm>
+#include <atomic>
 #include <mutex>
 #include <vector>
 
@@ -81,8 +82,10 @@ __global__ void k_segment_lb(const __grid_constant__ KnnWin W, float *out)
 
 // -------------------------------------------------------------- host side
 
-static int g_num_sms = 0;
-static int g_smem_per_sm = 0; // shared memory of one SM (bytes)
+// of the current device, set by device_setup for the calling thread
+static thread_local int g_dev = -1;
+static thread_local int g_num_sms = 0;
+static thread_local int g_smem_per_sm = 0; // shared memory of one SM (bytes)
 
 // ---- kernel timing for measurement tools (tnn_profile_*): four events per
 // search launch, on its stream -- before the main kernel (tile kernel, or
@@ -124,29 +127,60 @@ static size_t grid_smem(int cls) // per CTA
     return t[cls] * TNN_WARPS_PER_CTA;
 }
 
+// What a launch needs to know of a device, asked once (the driver's answers
+// cost more than the launch): zero until known.
+struct DeviceFacts {
+    std::atomic<int> sms, smem_per_sm, ready;
+    std::atomic<int> ctas[TNN_CLASSES + 3]; // CTAs per SM of the tile and warp kernels
+};
+static DeviceFacts g_facts[TNN_MAX_DEVICES];
+
+int tnn_num_sms(int dev)
+{
+    if (dev < 0 || dev >= TNN_MAX_DEVICES)
+        return 0;
+    int n = g_facts[dev].sms.load(std::memory_order_relaxed);
+    if (n == 0 && cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess)
+        g_facts[dev].sms.store(n, std::memory_order_relaxed);
+    return n;
+}
+
+static cudaError_t ctas_per_sm(int slot, TileKernel kern, size_t smem, int *out)
+{
+    int n = g_facts[g_dev].ctas[slot].load(std::memory_order_relaxed);
+    if (n == 0) {
+        const cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, kern, TNN_WARPS_PER_CTA * 32, smem);
+        if (e != cudaSuccess)
+            return e;
+        g_facts[g_dev].ctas[slot].store(n, std::memory_order_relaxed);
+    }
+    *out = n;
+    return cudaSuccess;
+}
+
 static tnn_status device_setup()
 {
     int dev = 0;
     TNN_CUDA_TRY(cudaGetDevice(&dev));
-    cudaDeviceProp prop;
-    TNN_CUDA_TRY(cudaGetDeviceProperties(&prop, dev));
-    if (prop.major != 10 || prop.minor != 3) {
-        tnn_set_error("libtnn is built for sm_103 (GB300); device %d is sm_%d%d",
-                      dev, prop.major, prop.minor);
-        return TNN_ERR_UNSUPPORTED;
-    }
-    g_num_sms = prop.multiProcessorCount;
-    g_smem_per_sm = (int)prop.sharedMemPerMultiprocessor;
-    // The shared-memory limit of a kernel is a per-device attribute: raised
-    // once on every device that runs a search.
-    static std::mutex mu;
-    static bool attrs[TNN_MAX_DEVICES];
     if (dev < 0 || dev >= TNN_MAX_DEVICES) {
         tnn_set_error("device ids must be below %d, got %d", TNN_MAX_DEVICES, dev);
         return TNN_ERR_UNSUPPORTED;
     }
-    std::lock_guard<std::mutex> lk(mu);
-    if (!attrs[dev]) {
+    DeviceFacts &f = g_facts[dev];
+    // The shared-memory limit of a kernel is a per-device attribute: raised
+    // once on every device that runs a search.
+    if (!f.ready.load(std::memory_order_acquire)) {
+        static std::mutex mu;
+        std::lock_guard<std::mutex> lk(mu);
+        cudaDeviceProp prop;
+        TNN_CUDA_TRY(cudaGetDeviceProperties(&prop, dev));
+        if (prop.major != 10 || prop.minor != 3) {
+            tnn_set_error("libtnn is built for sm_103 (GB300); device %d is sm_%d%d",
+                          dev, prop.major, prop.minor);
+            return TNN_ERR_UNSUPPORTED;
+        }
+        f.sms.store(prop.multiProcessorCount);
+        f.smem_per_sm.store((int)prop.sharedMemPerMultiprocessor);
         const int maxs = 227 * 1024;
         TNN_CUDA_TRY(cudaFuncSetAttribute(k_tnn_search<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, maxs));
         TNN_CUDA_TRY(cudaFuncSetAttribute(k_tnn_search<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, maxs));
@@ -156,8 +190,11 @@ static tnn_status device_setup()
         TNN_CUDA_TRY(cudaFuncSetAttribute(k_linear_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, maxs));
         TNN_CUDA_TRY(cudaFuncSetAttribute(k_fallback_exact, cudaFuncAttributeMaxDynamicSharedMemorySize, maxs));
         TNN_CUDA_TRY(cudaFuncSetAttribute(k_tnn_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, maxs));
-        attrs[dev] = true;
+        f.ready.store(1, std::memory_order_release);
     }
+    g_dev = dev;
+    g_num_sms = f.sms.load(std::memory_order_relaxed);
+    g_smem_per_sm = f.smem_per_sm.load(std::memory_order_relaxed);
     return TNN_OK;
 }
 
@@ -277,9 +314,10 @@ static tnn_status finish_search(const KnnLaunch &L, cudaStream_t st, bool prof, 
         TNN_CUDA_TRY(cudaEventRecord(pr.e[1], st));
     {
         // list registers by the largest k of the launch
-        const TileKernel kern = L.k_max <= 16 ? k_tnn_warp<1> : L.k_max <= 32 ? k_tnn_warp<2> : k_tnn_warp<4>;
+        const int v = L.k_max <= 16 ? 0 : L.k_max <= 32 ? 1 : 2;
+        const TileKernel kern = v == 0 ? k_tnn_warp<1> : v == 1 ? k_tnn_warp<2> : k_tnn_warp<4>;
         int nbw = 0;
-        TNN_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nbw, kern, TNN_WARPS_PER_CTA * 32, 0));
+        TNN_CUDA_TRY(ctas_per_sm(TNN_CLASSES + v, kern, 0, &nbw));
         TNN_CUDA_TRY(launch_dependent<KnnLaunch>(kern, (unsigned)(std::max(nbw, 1) * g_num_sms),
                                                  TNN_WARPS_PER_CTA * 32, 0, st, L));
     }
@@ -301,7 +339,7 @@ static tnn_status launch_grid_tiles(const KnnLaunch &L, int cls, cudaStream_t st
     const TileKernel kern = grid_kernel(cls);
     const size_t smem = grid_smem(cls);
     int nb = 0;
-    TNN_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, kern, TNN_WARPS_PER_CTA * 32, smem));
+    TNN_CUDA_TRY(ctas_per_sm(cls, kern, smem, &nb));
     if (nb < 1) {
         tnn_set_error("search kernel does not fit on an SM (%zu B shared memory)", smem);
         return TNN_ERR_UNSUPPORTED;

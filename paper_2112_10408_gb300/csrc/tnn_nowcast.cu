@@ -298,9 +298,7 @@ extern "C" tnn_status tnn_context_features(const tnn_index *ix, const float *d_w
     const int64_t per_cta = (int64_t)CF_WARPS * (k > 32 ? 2 : k > 16 ? 4 : 32 >> lg);
     int64_t grid = (m + per_cta - 1) / per_cta;
     if (k > 16) { // persistent: CF_CTAS CTAs per SM
-        int nsm = 0;
-        TNN_CUDA_TRY(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, ix->device));
-        grid = std::min<int64_t>(grid, (int64_t)CF_CTAS * nsm);
+        grid = std::min<int64_t>(grid, (int64_t)CF_CTAS * std::max(tnn_num_sms(ix->device), 1));
     }
     const float2 *wind = (const float2 *)d_wind;
     cudaStream_t st = (cudaStream_t)stream;
@@ -812,9 +810,7 @@ static tnn_status mlp_forward_impl(const tnn_mlp *n, const uint16_t *d_x, long l
     if (!d_t && n->dh % 128 == 0 && n->dh <= 256 &&
         mlp_infer_smem(n->d_in, n->dh) <= (size_t)227 * 1024) {
         // inference: persistent warp-specialised kernel, one CTA per SM
-        int dev = 0, nsm = 0;
-        TNN_CUDA_TRY(cudaGetDevice(&dev));
-        TNN_CUDA_TRY(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
+        const int nsm = std::max(tnn_num_sms(n->device), 1);
         a.tmem_cols = tmem_cols_for(2 * n->dh);
         const long long tiles = (B + MLP_ROWS - 1) / MLP_ROWS;
         const unsigned grid = (unsigned)std::min<long long>(tiles, nsm);
@@ -830,9 +826,7 @@ static tnn_status mlp_forward_impl(const tnn_mlp *n, const uint16_t *d_x, long l
     // Training: hidden units split over a cluster while that still gives every
     // CTA an SM of its own (at least 64 units each: two halves of 32).
     const long long tiles = (B + MLP_ROWS - 1) / MLP_ROWS;
-    int dev = 0, nsm = 0;
-    TNN_CUDA_TRY(cudaGetDevice(&dev));
-    TNN_CUDA_TRY(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
+    const int nsm = tnn_num_sms(n->device);
     a.csize = 1;
     while (d_t && a.csize < 8 && n->dh % (128 * a.csize) == 0 && tiles * 2 * a.csize <= nsm)
         a.csize *= 2;

@@ -243,9 +243,9 @@ def tnn_build_segments(xyzt: torch.Tensor, traj_off, sigma, seg_len: int) -> Ind
         p.sigma[i] = float(sigma[i])
     p.seg_len = int(seg_len)
     h = c_p()
-    _check(_L().tnn_build_segments(_ptr(xyzt), xyzt.shape[0], off.ctypes.data_as(c_p),
+    _check(_L().tnn_build_segments(_ptr(xyzt), xyzt.shape[0], c_p(off.ctypes.data),
                                    off.shape[0] - 1, ctypes.byref(p), _stream(), ctypes.byref(h)))
-    n_segments = int(((np.diff(off) + seg_len - 1) // seg_len).sum())
+    n_segments = int(np.add.reduce((off[1:] - off[:-1] + (seg_len - 1)) // seg_len))
     return Index(h, sigma, seg_len, xyzt.shape[0], off.shape[0] - 1, n_segments)
 
 
