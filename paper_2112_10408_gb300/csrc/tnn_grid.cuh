@@ -116,6 +116,20 @@ __device__ __forceinline__ float box_lb(const GroupBox &g, float st, float4 a, f
     return (a.w < g.T32) ? lb : INFINITY;
 }
 
+// The same for every segment of one grid key (cell rectangle, extent, largest
+// t_B).
+__device__ __forceinline__ float box_key_lb(const GroupBox &g, float st, float rx0, float rx1, float ry0,
+                                            float ry1, float ext, float tBk)
+{
+    const float dx = fmaxf(fmaxf(rx0 - g.bx1, g.bx0 - rx1), 0.0f);
+    const float dy = fmaxf(fmaxf(ry0 - g.by1, g.by0 - ry1), 0.0f);
+    const float a2 = fmaf(dy, dy, dx * dx);
+    const float dist = a2 * rsqrtf(fmaxf(a2, 1e-37f));
+    const float sp = fmaxf(fmaf(dist, 1.0f - 0x1p-20f, -(ext + g.delta)), 0.0f);
+    const float et = fmaxf(fmaxf(__fsub_rd(g.qt, tBk), g.gap), 0.0f);
+    return fmaf(sp, sp, (st * et) * et) * (1.0f - 0x1p-18f);
+}
+
 // ------------------------------------------------- candidate keys, networks
 
 #define TG_EMPTY 0xffffffffu // sorts after every key
@@ -124,6 +138,9 @@ __device__ __forceinline__ float box_lb(const GroupBox &g, float st, float4 a, f
 #define TG_NB 8        // points sorted at a time
 #define TG_INSERT 1    // batches with at most this many candidates are inserted one by one
                        // (400,000 points: 1 279.8 us, 2 280.0, 3 281.3, 5 285.2)
+#ifndef TG_KEYS
+#define TG_KEYS 2         // grid keys per lane and round of reads
+#endif
 #define TG_MIN_GROUP 3       // smaller groups of a tile go to the warp-per-query kernel
 
 // Key of a distance (>= 0) in a slot: its bits, the lowest SB replaced by the
@@ -243,8 +260,8 @@ template <int NL> struct TileSmem {
             float4 seg[32][3];
             unsigned used[32]; // one word per 32 slots
             int pre[32];
-            int kend[32];
-            int krel[32];
+            int kend[32 * TG_KEYS];
+            int krel[32 * TG_KEYS];
         };
         unsigned raw[NL + TG_EXTRA][32];
     };
@@ -456,19 +473,28 @@ __global__ void __launch_bounds__(TNN_WARPS_PER_CTA * 32, TileCtas<NL>::value)
         bool near_phase = true;
         int total = 0, pos = 0; // segments of the present key group, handled so far
 
-        // The segments of up to 32 keys (lane: [klo, klo + kn) in key order)
-        // become the present group.
-        auto take_keys = [&](int klo, int kn) {
-            int inc = kn;
+        // The segments of up to 32 TG_KEYS keys (lane: [klo, klo + kn) in key
+        // order) become the present group.
+        auto take_keys = [&](const int (&klo)[TG_KEYS], const int (&kn)[TG_KEYS]) {
+            int inc = 0;
+#pragma unroll
+            for (int u = 0; u < TG_KEYS; ++u)
+                inc += kn[u];
+            int at = -inc;
 #pragma unroll
             for (int s = 1; s < 32; s <<= 1) {
                 const int v = __shfl_up_sync(FULLMASK, inc, s);
                 if (lane >= s)
                     inc += v;
             }
+            at += inc;
             __syncwarp();
-            S.kend[lane] = inc;
-            S.krel[lane] = klo - (inc - kn); // record = krel[j] + position in the group
+#pragma unroll
+            for (int u = 0; u < TG_KEYS; ++u) {
+                S.krel[lane * TG_KEYS + u] = klo[u] - at; // record = krel[j] + position in the group
+                at += kn[u];
+                S.kend[lane * TG_KEYS + u] = at;
+            }
             total = __shfl_sync(FULLMASK, inc, 31);
             pos = 0;
             __syncwarp();
@@ -476,11 +502,11 @@ __global__ void __launch_bounds__(TNN_WARPS_PER_CTA * 32, TileCtas<NL>::value)
         {
             const int bq = bhi - (seed_cell >> 4);
             const int cx = hx + (seed_cell & 3) - 1, cy = hy + ((seed_cell >> 2) & 3) - 1;
-            int klo = 0, kn = 0;
+            int klo[TG_KEYS] = {0}, kn[TG_KEYS] = {0};
             if (lane < 9 * TNN_SEED_BUCKETS && bq >= 0 && cx >= 0 && cx < G.nx && cy >= 0 && cy < G.ny) {
                 const int key = bq * G.ncell + cy * G.nx + cx;
-                klo = __ldg(G.off + key);
-                kn = __ldg(G.off + key + 1) - klo;
+                klo[0] = __ldg(G.off + key);
+                kn[0] = __ldg(G.off + key + 1) - klo[0];
             }
             take_keys(klo, kn);
         }
@@ -505,8 +531,8 @@ __global__ void __launch_bounds__(TNN_WARPS_PER_CTA * 32, TileCtas<NL>::value)
                     if (fill > 0) {
                         flush = true;
                     } else {
-                        // the next buckets, as many as give 32 cells: their
-                        // records are one round of reads
+                        // the next buckets, as many as give 32 TG_KEYS cells:
+                        // their records are one round of reads
                         b -= gb;
                         if (b < 0)
                             break;
@@ -530,7 +556,7 @@ __global__ void __launch_bounds__(TNN_WARPS_PER_CTA * 32, TileCtas<NL>::value)
                         nc = max(wx, 0) * max(cy1 - cy0 + 1, 0);
                         if (nc == 0)
                             break; // no cell within reach
-                        const int most = min(b + 1, 32 / nc);
+                        const int most = min(min(b + 1, 32), 32 * TG_KEYS / nc);
 #pragma unroll 1
                         for (gb = 1; gb < most; ++gb) {
                             const float tg = time_lb(c, s3, __shfl_sync(FULLMASK, bp, gb));
@@ -542,39 +568,37 @@ __global__ void __launch_bounds__(TNN_WARPS_PER_CTA * 32, TileCtas<NL>::value)
                         continue;
                     }
                 } else {
-                    // up to 32 cells of the group: the keys some lane needs
-                    const int t = t0 + lane;
-                    t0 += 32;
-                    int klo = 0, kn = 0, cx = 0, cy = 0;
-                    float ex = 0.f, tk = 0.f;
-                    if (t < ncells) {
+                    // up to 32 TG_KEYS cells of the group: the keys the
+                    // query group as a whole may need
+                    const float inv_nc = 1.0f / (float)nc, inv_wx = 1.0f / (float)wx, reach = warp_maxf(lim);
+                    int klo[TG_KEYS], kn[TG_KEYS], any = 0;
+                    int4 kr[TG_KEYS];
+                    int kx[TG_KEYS], ky[TG_KEYS];
+#pragma unroll
+                    for (int u = 0; u < TG_KEYS; ++u) {
+                        const int t = t0 + u * 32 + lane;
                         // quotients of integers below 2^21: exact
-                        const int db = (int)(((float)t + 0.5f) * (1.0f / (float)nc)), rem = t - db * nc;
-                        const int dy = (int)(((float)rem + 0.5f) * (1.0f / (float)wx));
-                        cx = cx0 + rem - dy * wx;
-                        cy = cy0 + dy;
-                        const bool staged = b - db > bhi - TNN_SEED_BUCKETS && abs(cx - hx) <= 1 && abs(cy - hy) <= 1;
-                        if (!staged) {
-                            const int4 kr = __ldg(G.krec + ((b - db) * G.ncell + cy * G.nx + cx));
-                            klo = kr.x;
-                            kn = kr.y - kr.x;
-                            ex = __int_as_float(kr.z);
-                            tk = __int_as_float(kr.w);
-                        }
+                        const int db = (int)(((float)t + 0.5f) * inv_nc), rem = t - db * nc;
+                        const int dy = (int)(((float)rem + 0.5f) * inv_wx);
+                        kx[u] = cx0 + rem - dy * wx;
+                        ky[u] = cy0 + dy;
+                        const bool staged = b - db > bhi - TNN_SEED_BUCKETS && abs(kx[u] - hx) <= 1 &&
+                                            abs(ky[u] - hy) <= 1;
+                        kr[u] = t < ncells && !staged ? __ldg(G.krec + ((b - db) * G.ncell + ky[u] * G.nx + kx[u]))
+                                                      : make_int4(0, 0, 0, 0);
                     }
-                    unsigned m = __ballot_sync(FULLMASK, kn > 0), want = 0;
-                    while (m) {
-                        const int j = __ffs(m) - 1;
-                        m &= m - 1;
-                        const int jx = __shfl_sync(FULLMASK, cx, j), jy = __shfl_sync(FULLMASK, cy, j);
-                        const float jex = __shfl_sync(FULLMASK, ex, j), jtk = __shfl_sync(FULLMASK, tk, j);
-                        const float rx0 = G.x0 + (float)jx * G.cell, ry0 = G.y0 + (float)jy * G.cell;
-                        if (__any_sync(FULLMASK, cell_lb(c, s3, rx0, rx0 + G.cell, ry0, ry0 + G.cell, jex,
-                                                         jtk) <= lim))
-                            want |= 1u << j;
+#pragma unroll
+                    for (int u = 0; u < TG_KEYS; ++u) {
+                        const float rx0 = G.x0 + (float)kx[u] * G.cell, ry0 = G.y0 + (float)ky[u] * G.cell;
+                        const bool want = box_key_lb(box, s3, rx0, rx0 + G.cell, ry0, ry0 + G.cell,
+                                                     __int_as_float(kr[u].z), __int_as_float(kr[u].w)) <= reach;
+                        klo[u] = kr[u].x;
+                        kn[u] = want ? kr[u].y - kr[u].x : 0;
+                        any |= kn[u];
                     }
-                    if (want)
-                        take_keys(klo, (want >> lane) & 1u ? kn : 0);
+                    t0 += 32 * TG_KEYS;
+                    if (__any_sync(FULLMASK, any != 0))
+                        take_keys(klo, kn);
                     continue;
                 }
             }
@@ -587,9 +611,9 @@ __global__ void __launch_bounds__(TNN_WARPS_PER_CTA * 32, TileCtas<NL>::value)
                 __syncwarp();
                 if (lane < cnt) {
                     const int g = pos + lane;
-                    int lo = 0, hi = 31; // smallest key with kend > g
-#pragma unroll
-                    for (int s = 0; s < 5; ++s) {
+                    int lo = 0, hi = 32 * TG_KEYS - 1; // smallest key with kend > g
+#pragma unroll 1
+                    while (lo < hi) {
                         const int mid = (lo + hi) >> 1;
                         if (S.kend[mid] > g)
                             hi = mid;
