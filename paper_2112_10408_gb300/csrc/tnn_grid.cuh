@@ -42,7 +42,12 @@
 // when its turn comes (every lane's bound of every staged segment before: 47
 // of them per query at 400,000 points), and reading the key records of as many
 // buckets as fill a warp took these three figures from 280, 3,016 and 79 us to
-// 232, 2,669 and 44 us.  (Dropping single points by their distance to the
+// 232, 2,669 and 44 us; bounding the keys the same way, two per lane and round
+// of reads, 4,000,000 to 2,497 us; settling only the runs of rows that are not
+// certainly in order and keeping the warp's counters and rectangle in shared
+// memory (fewer spills, 60 instead of 69 KB of code) to 217, 2,318 and 40 us.
+// (More rows per step of the settlement, 4, 6 or 9 instead of 2, are slower:
+// 234, 247, 257 against 229 us.  Dropping single points by their distance to the
 // tile's rectangle before the lanes score them costs more than it saves: 251
 // against 234 us.)
 #pragma once
@@ -134,13 +139,12 @@ __device__ __forceinline__ float box_key_lb(const GroupBox &g, float st, float r
 
 #define TG_EMPTY 0xffffffffu // sorts after every key
 #define TG_INF 0x7f800000u   // keys of infinite distances
+#define TG_ROWS 2            // list rows settled per step
 #define TG_EXTRA 4           // candidates kept beyond the k-th
 #define TG_NB 8        // points sorted at a time
 #define TG_INSERT 1    // batches with at most this many candidates are inserted one by one
                        // (400,000 points: 1 279.8 us, 2 280.0, 3 281.3, 5 285.2)
-#ifndef TG_KEYS
-#define TG_KEYS 2         // grid keys per lane and round of reads
-#endif
+#define TG_KEYS 2         // grid keys per lane and round of reads (4: 227 us against 217)
 #define TG_MIN_GROUP 3       // smaller groups of a tile go to the warp-per-query kernel
 
 // Key of a distance (>= 0) in a slot: its bits, the lowest SB replaced by the
@@ -252,7 +256,7 @@ __device__ __forceinline__ void tg_insert(unsigned (&a)[NL], unsigned (&o)[TG_EX
 // the slots in use and their prefix, the key ranges' ends and offsets; the
 // slot table behind them.  To
 // settle, the lists' 32-bit keys take the first part's place, and then the
-// 64-bit lists [NL + TG_EXTRA + 1][32] everything's.
+// 64-bit lists [NL + TG_EXTRA][32] everything's.
 template <int NL> struct TileSmem {
     union {
         struct {
@@ -268,10 +272,18 @@ template <int NL> struct TileSmem {
     int slot[TileSlots<NL>::n];
 };
 
+// Kept through all of it: the group's rectangle and the warp's counters
+// (queries, bounds, distances, segments, FP64 distances), which would take
+// registers from the lists.
+struct TileKeep {
+    GroupBox box;
+    unsigned count[8];
+};
+
 template <int NL> __host__ __device__ constexpr size_t tg_smem_per_warp()
 {
-    const size_t lists = (size_t)(NL + TG_EXTRA + 1) * 256;
-    return lists > sizeof(TileSmem<NL>) ? lists : sizeof(TileSmem<NL>);
+    const size_t lists = (size_t)(NL + TG_EXTRA) * 256;
+    return (lists > sizeof(TileSmem<NL>) ? lists : sizeof(TileSmem<NL>)) + sizeof(TileKeep);
 }
 
 // Entry e of a lane's settled list: the lane's column is rotated by the entry
@@ -282,46 +294,38 @@ __device__ __forceinline__ unsigned long long *tg_entry(unsigned long long *Kw, 
     return Kw + e * 32 + (lane ^ (e & 31));
 }
 
-// Settle one query whose n exact keys (list rows z ...) are not yet in certain order: sort
-// them, drop those at or above `bound` (every point outside the list lies at
-// or above it), then rank chains of close keys in FP64, in place.  Bit 0 of
-// the result: settled; the rest counts the FP64 distances.  Out of line: a
-// few per cent of the queries come here.
+// Settle rows r0 .. r1 of one query's list, whose order is not certain: sort
+// them by their exact keys, then rank chains of close ones in FP64, in place.
+// The rows before and after are certain.  Bit 0 of the result: settled; the
+// rest counts the FP64 distances.  Out of line: a few per cent of the queries
+// come here, mostly with two rows.
 static __device__ __noinline__ unsigned tg_settle(const KnnWin *W, float4 q, unsigned long long *Kw,
-                                                  int lane, int z, int n, float bound)
+                                                  int lane, int r0, int r1)
 {
-    for (int i = 1; i < n; ++i) {
-        const unsigned long long v = *tg_entry(Kw, z + i, lane);
+    for (int i = r0 + 1; i <= r1; ++i) {
+        const unsigned long long v = *tg_entry(Kw, i, lane);
         int j = i;
-        while (j > 0) {
-            const unsigned long long u = *tg_entry(Kw, z + j - 1, lane);
+        while (j > r0) {
+            const unsigned long long u = *tg_entry(Kw, j - 1, lane);
             if (u <= v)
                 break;
-            *tg_entry(Kw, z + j, lane) = u;
+            *tg_entry(Kw, j, lane) = u;
             --j;
         }
         if (j < i)
-            *tg_entry(Kw, z + j, lane) = v;
+            *tg_entry(Kw, j, lane) = v;
     }
-    const bool full = bound < INFINITY;
-    if (full) {
-        while (n > 0 && key_d(*tg_entry(Kw, z + n - 1, lane)) >= bound)
-            --n;
-        *tg_entry(Kw, z + n, lane) = pack_key(bound, 0x7fffffff); // end marker
-        ++n;
-    }
-    const int k = W->k;
     const bool exact_all = (W->flags & TNN_FLAG_EXACT_D2) != 0;
     unsigned nfp = 0;
-    int i = 0;
-    while (i < k && i < n) {
-        const unsigned long long ki = *tg_entry(Kw, z + i, lane);
+    int i = r0;
+    while (i <= r1) {
+        const unsigned long long ki = *tg_entry(Kw, i, lane);
         if (ki == SENT)
             break;
         int e = i;
         float de = key_d(ki);
-        while (e + 1 < n) {
-            const unsigned long long kn = *tg_entry(Kw, z + e + 1, lane);
+        while (e < r1) {
+            const unsigned long long kn = *tg_entry(Kw, e + 1, lane);
             const float dn = key_d(kn);
             if (kn == SENT || !(dn <= fmaf(de, 0x1p-17f, de) + 0x1p-100f))
                 break;
@@ -329,13 +333,13 @@ static __device__ __noinline__ unsigned tg_settle(const KnnWin *W, float4 q, uns
             de = dn;
         }
         const int c = e - i + 1;
-        if ((full && e == n - 1) || c > CMAX)
+        if (c > CMAX)
             return nfp << 1;
         if (c > 1 || exact_all) {
             double dd[CMAX];
             int id[CMAX];
             for (int t = 0; t < c; ++t) {
-                const int j = key_i(*tg_entry(Kw, z + i + t, lane));
+                const int j = key_i(*tg_entry(Kw, i + t, lane));
                 const double d = dist64(W->sigd, q, W->pts[j]);
                 ++nfp;
                 int pos = t;
@@ -348,12 +352,10 @@ static __device__ __noinline__ unsigned tg_settle(const KnnWin *W, float4 q, uns
                 id[pos] = j;
             }
             for (int t = 0; t < c; ++t)
-                *tg_entry(Kw, z + i + t, lane) = pack_key((float)dd[t], id[t]);
+                *tg_entry(Kw, i + t, lane) = pack_key((float)dd[t], id[t]);
         }
         i = e + 1;
     }
-    if (full && i < k)
-        return nfp << 1;
     return (nfp << 1) | 1u;
 }
 
@@ -384,15 +386,16 @@ __global__ void __launch_bounds__(TNN_WARPS_PER_CTA * 32, TileCtas<NL>::value)
     unsigned char *ws = smem + (threadIdx.x >> 5) * tg_smem_per_warp<NL>();
     TileSmem<NL> &S = *(TileSmem<NL> *)ws;
     unsigned long long *Kw = (unsigned long long *)ws;
-    const int seed_cell = tg_seed_cell[lane];
+    TileKeep &KP = *(TileKeep *)(ws + tg_smem_per_warp<NL>() - sizeof(TileKeep));
+    if (lane < 8)
+        KP.count[lane] = 0;
+    __syncwarp();
     pdl_trigger();
 
-    unsigned n_q = 0, n_lb = 0, n_pairs = 0, n_segs = 0, n_fp = 0;
+    // First tile by the warp's number, then the queue.
+    long long claim = (long long)blockIdx.x * TNN_WARPS_PER_CTA + (threadIdx.x >> 5);
     for (;;) {
-        long long tile = 0;
-        if (lane == 0)
-            tile = L.tile_lo + (long long)atomicAdd(&L.scr->tile_counter[L.queue], 1ull);
-        tile = __shfl_sync(FULLMASK, tile, 0);
+        const long long tile = L.tile_lo + __shfl_sync(FULLMASK, claim, 0);
         if (tile >= L.total_tiles)
             break;
         const KnnWin *W = find_window(L, tile);
@@ -404,9 +407,6 @@ __global__ void __launch_bounds__(TNN_WARPS_PER_CTA * 32, TileCtas<NL>::value)
         const GridDesc &G = W->grid;
         const float tau_defer = W->tau_defer;
         const int k = W->k;
-        const float ext_max = __ldg(G.ext_max);
-        if (active)
-            n_q++;
 
         // A tile whose queries lie far apart (the caller's own order, two
         // flights in one tile) is answered in groups around its first query
@@ -440,9 +440,17 @@ __global__ void __launch_bounds__(TNN_WARPS_PER_CTA * 32, TileCtas<NL>::value)
         const float bx1 = warp_maxf(act ? c.sx : -INFINITY);
         const float by0 = warp_minf(act ? c.sy : INFINITY);
         const float by1 = warp_maxf(act ? c.sy : -INFINITY);
-        const GroupBox box = {bx0, bx1, by0, by1, warp_minf(act ? c.qt : INFINITY), tmax,
-                              warp_minf(act ? __fsub_rd(c.qt, c.T32) : INFINITY),
-                              warp_maxf(act ? c.delta : 0.0f)};
+        {
+            const GroupBox box = {bx0, bx1, by0, by1, warp_minf(act ? c.qt : INFINITY), tmax,
+                                  warp_minf(act ? __fsub_rd(c.qt, c.T32) : INFINITY),
+                                  warp_maxf(act ? c.delta : 0.0f)};
+            __syncwarp();
+            if (lane == 0) {
+                KP.box = box;
+                KP.count[0] += __popc(grp);
+            }
+            __syncwarp();
+        }
         int bhi = -1;
         {
             const float fb = (tmax - G.t0) * G.inv_dt;
@@ -500,6 +508,7 @@ __global__ void __launch_bounds__(TNN_WARPS_PER_CTA * 32, TileCtas<NL>::value)
             __syncwarp();
         };
         {
+            const int seed_cell = tg_seed_cell[lane];
             const int bq = bhi - (seed_cell >> 4);
             const int cx = hx + (seed_cell & 3) - 1, cy = hy + ((seed_cell >> 2) & 3) - 1;
             int klo[TG_KEYS] = {0}, kn[TG_KEYS] = {0};
@@ -548,9 +557,9 @@ __global__ void __launch_bounds__(TNN_WARPS_PER_CTA * 32, TileCtas<NL>::value)
                         cy0 = 0;
                         if (tmx < INFINITY) {
                             // any key outside this reach has a bound above every key
-                            const float R = sqrtf(tmx) * (1.0f + 0x1p-18f) + ext_max + box.delta;
-                            reach_cells(bx0, bx1, R, G.x0, G.inv_cell, G.nx, cx0, cx1);
-                            reach_cells(by0, by1, R, G.y0, G.inv_cell, G.ny, cy0, cy1);
+                            const float R = sqrtf(tmx) * (1.0f + 0x1p-18f) + __ldg(G.ext_max) + KP.box.delta;
+                            reach_cells(KP.box.bx0, KP.box.bx1, R, G.x0, G.inv_cell, G.nx, cx0, cx1);
+                            reach_cells(KP.box.by0, KP.box.by1, R, G.y0, G.inv_cell, G.ny, cy0, cy1);
                         }
                         wx = cx1 - cx0 + 1;
                         nc = max(wx, 0) * max(cy1 - cy0 + 1, 0);
@@ -590,7 +599,7 @@ __global__ void __launch_bounds__(TNN_WARPS_PER_CTA * 32, TileCtas<NL>::value)
 #pragma unroll
                     for (int u = 0; u < TG_KEYS; ++u) {
                         const float rx0 = G.x0 + (float)kx[u] * G.cell, ry0 = G.y0 + (float)ky[u] * G.cell;
-                        const bool want = box_key_lb(box, s3, rx0, rx0 + G.cell, ry0, ry0 + G.cell,
+                        const bool want = box_key_lb(KP.box, s3, rx0, rx0 + G.cell, ry0, ry0 + G.cell,
                                                      __int_as_float(kr[u].z), __int_as_float(kr[u].w)) <= reach;
                         klo[u] = kr[u].x;
                         kn[u] = want ? kr[u].y - kr[u].x : 0;
@@ -627,7 +636,7 @@ __global__ void __launch_bounds__(TNN_WARPS_PER_CTA * 32, TileCtas<NL>::value)
                     S.seg[lane][2] = rb;
                     sfirst = __float_as_int(r3.x);
                     scnt = __float_as_int(r3.y);
-                    const float lb = box_lb(box, s3, ra, ru, rb);
+                    const float lb = box_lb(KP.box, s3, ra, ru, rb);
                     if (lb < INFINITY) // truncated towards zero: still a bound
                         score = (__float_as_uint(lb) & ~31u) | (unsigned)lane;
                 }
@@ -649,12 +658,14 @@ __global__ void __launch_bounds__(TNN_WARPS_PER_CTA * 32, TileCtas<NL>::value)
                         if (lane == j)
                             score = TG_EMPTY;
                         const float lb = seg_lb(c, s3, S.seg[j][0], S.seg[j][1], S.seg[j][2]);
-                        n_lb += act;
+                        if (lane == 0)
+                            KP.count[1] += __popc(grp);
                         if (!__any_sync(FULLMASK, lb <= lim))
                             continue;
                         lf = __shfl_sync(FULLMASK, sfirst, j);
                         lc = __shfl_sync(FULLMASK, scnt, j);
-                        n_segs += act;
+                        if (lane == 0)
+                            KP.count[3] += __popc(grp);
                     }
                     const int take = min(lc, 32 - fill);
                     if (lane >= fill && lane < fill + take)
@@ -730,13 +741,12 @@ __global__ void __launch_bounds__(TNN_WARPS_PER_CTA * 32, TileCtas<NL>::value)
                     S.pts[lane] = p;
                 }
                 __syncwarp();
-                if (act) {
-                    n_pairs += fill;
-                    if (L.dbg_seen)
+                if (lane == 0)
+                    KP.count[2] += __popc(grp) * fill;
+                if (L.dbg_seen && act)
 #pragma unroll 1
-                        for (int i = 0; i < fill; ++i)
-                            dbg_mark_seen(L, qrow, S.slot[base + i], 1);
-                }
+                    for (int i = 0; i < fill; ++i)
+                        dbg_mark_seen(L, qrow, S.slot[base + i], 1);
                 unsigned kept = 0;
 #pragma unroll 1
                 for (int s = 0; s < fill; s += NB) {
@@ -817,34 +827,49 @@ __global__ void __launch_bounds__(TNN_WARPS_PER_CTA * 32, TileCtas<NL>::value)
             S.raw[e][lane] = settle && v != TG_EMPTY ? (unsigned)S.slot[v & SL::mask] : TG_EMPTY;
         }
         {
-            // Exact keys, from the last row down: 64-bit row e covers 32-bit
-            // rows 2 e and 2 e + 1, which every lane has read by then.
-            // `slow`: some entry is not certainly below its successor (a little
-            // more than the margin of the settlement, so that a plain
-            // comparison will do: missing entries are infinite).
-            bool slow = (W->flags & TNN_FLAG_EXACT_D2) != 0;
+            // Exact keys, TG_ROWS rows per step (their gathers in flight
+            // together) from the last one down: 64-bit row e covers 32-bit
+            // rows 2 e and 2 e + 1, which every lane has read by then.  Rows r0 .. r1 hold every row that is not certainly
+            // below its successor: not in another bucket of the truncated
+            // keys, or within the margin of the settlement.
+            constexpr float link = 0x1.02p-23f * (float)SL::n;
+            int r0 = NL + TG_EXTRA, r1 = -1;
             float dn = INFINITY;
 #pragma unroll 1
-            for (int e = NL + TG_EXTRA - 1; e >= z; e -= 2) {
-                const int e1 = max(e - 1, z); // two rows per step, the last may be one
-                const unsigned i0 = S.raw[e][lane], i1 = S.raw[e1][lane];
+            for (int e = NL + TG_EXTRA - 1; e >= z; e -= TG_ROWS) {
+                unsigned id[TG_ROWS];
+                float4 p[TG_ROWS];
+#pragma unroll
+                for (int u = 0; u < TG_ROWS; ++u)
+                    id[u] = S.raw[max(e - u, z)][lane];
                 __syncwarp();
-                const float4 p0 = __ldg(pts + (i0 != TG_EMPTY ? i0 : 0u));
-                const float4 p1 = __ldg(pts + (i1 != TG_EMPTY ? i1 : 0u));
-                const float d0 = i0 != TG_EMPTY ? dist32(c, s0, s1, s2, s3, p0) : INFINITY;
-                const float d1 = i1 != TG_EMPTY ? dist32(c, s0, s1, s2, s3, p1) : INFINITY;
-                *tg_entry(Kw, e, lane) = pack_key(d0, (int)i0); // (infinity, -1) is SENT
-                *tg_entry(Kw, e1, lane) = pack_key(d1, (int)i1);
-                slow |= dn < fmaf(d0, 0x1.1p-17f, d0) + 0x1p-99f;
-                slow |= e1 < e && d0 < fmaf(d1, 0x1.1p-17f, d1) + 0x1p-99f;
-                dn = d1;
+#pragma unroll
+                for (int u = 0; u < TG_ROWS; ++u)
+                    p[u] = __ldg(pts + (id[u] != TG_EMPTY ? id[u] : 0u));
+#pragma unroll
+                for (int u = 0; u < TG_ROWS; ++u) {
+                    const float d = id[u] != TG_EMPTY ? dist32(c, s0, s1, s2, s3, p[u]) : INFINITY;
+                    if (e - u >= z) {
+                        *tg_entry(Kw, e - u, lane) = pack_key(d, (int)id[u]); // (infinity, -1) is SENT
+                        if (dn < fmaf(d, link, d) + 0x1p-99f) {
+                            r0 = e - u;
+                            r1 = max(r1, e - u + 1);
+                        }
+                        dn = d;
+                    }
+                }
             }
+            // every point outside the list lies at or above `bound`
             const float dk = key_d(*tg_entry(Kw, NL - 1, lane));
-            slow |= bound < fmaf(dk, 0x1.1p-17f, dk) + 0x1p-99f;
-            if (settle && ok && slow) {
-                const unsigned r = tg_settle(W, q, Kw, lane, z, k + TG_EXTRA, bound);
+            ok = ok && !(bound < fmaf(dk, 0x1.1p-17f, dk) + 0x1p-99f);
+            if (W->flags & TNN_FLAG_EXACT_D2) {
+                r0 = z;
+                r1 = NL + TG_EXTRA - 1;
+            }
+            if (settle && ok && r0 < r1) {
+                const unsigned r = tg_settle(W, q, Kw, lane, r0, r1);
                 ok = r & 1u;
-                n_fp += r >> 1;
+                atomicAdd(&KP.count[4], r >> 1);
             }
         }
         if (settle && !ok) {
@@ -907,6 +932,11 @@ __global__ void __launch_bounds__(TNN_WARPS_PER_CTA * 32, TileCtas<NL>::value)
         }
         __syncwarp();
         }
+        if (lane == 0 && lone)
+            KP.count[0] += __popc(lone);
+        if (lane == 0)
+            claim = (long long)gridDim.x * TNN_WARPS_PER_CTA +
+                    (long long)atomicAdd(&L.scr->tile_counter[L.queue], 1ull);
         if ((lone >> lane) & 1u) {
             const unsigned slot = atomicAdd(&L.scr->n_fallback, 1u);
             if (slot < (unsigned long long)L.fb_cap) {
@@ -917,6 +947,7 @@ __global__ void __launch_bounds__(TNN_WARPS_PER_CTA * 32, TileCtas<NL>::value)
         }
         __syncwarp();
     }
-    LaneStats st = {n_q, n_lb, n_pairs, n_segs, n_fp};
-    flush_stats(L.scr, st);
+    __syncwarp();
+    if (lane < 5 && KP.count[lane])
+        atomicAdd(&L.scr->stats[lane], (unsigned long long)KP.count[lane]);
 }
