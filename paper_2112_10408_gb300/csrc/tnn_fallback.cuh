@@ -135,8 +135,11 @@ template <int NR> __device__ __forceinline__ void wq_insert(unsigned (&a)[NR], u
 #ifndef TNN_WARP_MINB
 #define TNN_WARP_MINB 6 // CTAs per SM (4 M points: 5 368 us, 6 350, 7 353; fewer spill less when few queries come)
 #endif
-// NR list registers per lane: 32 NR candidates, for k <= 32 NR - 16.
-template <int NR>
+// NR list registers per lane: 32 NR candidates, for k <= 32 NR - 16.  A single
+// window (MANY false) is read from the kernel's parameters, so that its fields
+// are constant operands and take no registers (handed-over queries of 4 M
+// points 239 -> 221 us; the tile kernel gains nothing from it).
+template <int NR, bool MANY>
 __global__ void __launch_bounds__(TNN_WARPS_PER_CTA * 32, TNN_WARP_MINB)
     k_tnn_warp(const __grid_constant__ KnnLaunch L)
 {
@@ -172,7 +175,7 @@ __global__ void __launch_bounds__(TNN_WARPS_PER_CTA * 32, TNN_WARP_MINB)
         }
         const bool unsettled = retry || ent.x < 0;
         const int wid = ent.x < 0 ? -1 - ent.x : ent.x;
-        const KnnWin *W = L.nwin <= 1 ? &L.w0 : L.wins + wid;
+        const KnnWin *W = MANY ? L.wins + wid : &L.w0;
         const float4 q = W->q[ent.y];
         const QCtx c = make_qctx(W, q, true);
         const float s0 = W->sig[0], s1 = W->sig[1], s2 = W->sig[2], s3 = W->sig[3];

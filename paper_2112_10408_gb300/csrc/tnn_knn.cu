@@ -120,6 +120,14 @@ static TileKernel grid_kernel(int cls)
                                               k_tnn_grid_search<32>, k_tnn_grid_search<64>};
     return t[cls];
 }
+// The warp-per-query kernel: list registers by the largest k of the launch.
+static int warp_class(int k_max) { return k_max <= 16 ? 0 : k_max <= 32 ? 1 : 2; }
+static TileKernel warp_kernel(int v, bool many)
+{
+    static const TileKernel t[2][3] = {{k_tnn_warp<1, false>, k_tnn_warp<2, false>, k_tnn_warp<4, false>},
+                                       {k_tnn_warp<1, true>, k_tnn_warp<2, true>, k_tnn_warp<4, true>}};
+    return t[many][v];
+}
 static size_t grid_smem(int cls) // per CTA
 {
     static const size_t t[TNN_CLASSES] = {tg_smem_per_warp<8>(), tg_smem_per_warp<16>(),
@@ -131,7 +139,7 @@ static size_t grid_smem(int cls) // per CTA
 // cost more than the launch): zero until known.
 struct DeviceFacts {
     std::atomic<int> sms, smem_per_sm, ready;
-    std::atomic<int> ctas[TNN_CLASSES + 3]; // CTAs per SM of the tile and warp kernels
+    std::atomic<int> ctas[TNN_CLASSES + 6]; // CTAs per SM of the tile and warp kernels
 };
 static DeviceFacts g_facts[TNN_MAX_DEVICES];
 
@@ -313,11 +321,11 @@ static tnn_status finish_search(const KnnLaunch &L, cudaStream_t st, bool prof, 
     if (prof)
         TNN_CUDA_TRY(cudaEventRecord(pr.e[1], st));
     {
-        // list registers by the largest k of the launch
-        const int v = L.k_max <= 16 ? 0 : L.k_max <= 32 ? 1 : 2;
-        const TileKernel kern = v == 0 ? k_tnn_warp<1> : v == 1 ? k_tnn_warp<2> : k_tnn_warp<4>;
+        const bool many = L.nwin > 1;
+        const int v = warp_class(L.k_max);
+        const TileKernel kern = warp_kernel(v, many);
         int nbw = 0;
-        TNN_CUDA_TRY(ctas_per_sm(TNN_CLASSES + v, kern, 0, &nbw));
+        TNN_CUDA_TRY(ctas_per_sm(TNN_CLASSES + 2 * v + many, kern, 0, &nbw));
         TNN_CUDA_TRY(launch_dependent<KnnLaunch>(kern, (unsigned)(std::max(nbw, 1) * g_num_sms),
                                                  TNN_WARPS_PER_CTA * 32, 0, st, L));
     }
