@@ -77,8 +77,7 @@ enum {
 // spatial axes, the bounding box.  The other blocks take a trajectory per
 // warp: times non-decreasing inside it, the summed duration t_last - t_first
 // of its K-point sets, which sizes the grid's time buckets, and the sets'
-// (first point, count, trajectory) and t_A sort keys (the last of these blocks the sort's
-// padding).
+// (first point, count, trajectory) and t_A sort keys.
 // (A copy and three kernels before; bound by the reads and the launch.)
 __global__ void __launch_bounds__(VAL_THREADS)
     k_validate(const float4 *__restrict__ in, float4 *__restrict__ out, int n, float s0, float s1, float s2,
@@ -88,9 +87,9 @@ __global__ void __launch_bounds__(VAL_THREADS)
 {
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     if ((int)blockIdx.x >= pblocks) {
-        if (blockIdx.x == gridDim.x - 1)
-            for (int i = S + threadIdx.x; i < S2; i += VAL_THREADS)
-                keys[i] = ~0ull;
+        for (int i = S + ((int)blockIdx.x - pblocks) * VAL_THREADS + threadIdx.x; i < S2;
+             i += ((int)gridDim.x - pblocks) * VAL_THREADS)
+            keys[i] = ~0ull; // the sort's padding
         const int tr = ((int)blockIdx.x - pblocks) * (VAL_THREADS / 32) + w;
         if (tr >= n_traj) // the same for the whole warp
             return;
