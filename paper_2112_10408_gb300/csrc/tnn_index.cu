@@ -154,6 +154,11 @@ __global__ void __launch_bounds__(VAL_THREADS)
     }
 }
 
+// AB' of one axis, sqrt(s) b - A', with its roundings spelled out: the grid
+// key is taken from it twice (sort keys, extents) and both must agree, whatever
+// the compiler would contract around them.
+__device__ __forceinline__ float scaled_step(double q, float b, float a) { return (float)fma(q, (double)b, -(double)a); }
+
 // One thread per segment (build order).  FP64, rounded once to the stored
 // FP32 record:
 //   A' = fl(sqrt(s) A),  AB' = fl(sqrt(s) B - A'),  U' = fl(AB' / |AB'|^2)
@@ -195,7 +200,7 @@ __global__ void __launch_bounds__(SF_THREADS)
             Af[i] = (float)sa;
             A[i] = (double)Af[i];
             res[i] = (float)(sa - A[i]); // sqrt(s) p - A' = sqrt(s) (p - p_a) + res
-            ABf[i] = (float)(qq[i] * (double)pbv[i] - A[i]);
+            ABf[i] = scaled_step(qq[i], pbv[i], Af[i]);
             AB[i] = (double)ABf[i];
             mag += fabsf(Af[i]) + fabsf((float)(A[i] + AB[i]));
         }
@@ -728,7 +733,7 @@ __global__ void k_grid_sort_keys(const float4 *__restrict__ p, const int4 *__res
     const int4 r = range[s];
     const float4 pa = p[r.x], pb = p[r.x + r.y - 1];
     const float ax = (float)(q0 * (double)pa.x), ay = (float)(q1 * (double)pa.y);
-    const float bx = (float)(q0 * (double)pb.x - (double)ax), by = (float)(q1 * (double)pb.y - (double)ay);
+    const float bx = scaled_step(q0, pb.x, ax), by = scaled_step(q1, pb.y, ay);
     int bk, cx, cy;
     const int key = grid_key(g, pa.w, ax, ay, bx, by, bk, cx, cy);
     keys[s] = ((unsigned long long)(unsigned)key << 32) | (unsigned)s;
