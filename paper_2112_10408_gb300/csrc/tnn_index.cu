@@ -174,7 +174,7 @@ __device__ __forceinline__ float scaled_step(double q, float b, float a) { retur
 // are measured in FP64: one, now and then two; three or more (or a segment
 // whose |AB|^2 FP32 does not hold) measure all members.  The same radius, bit
 // for bit; 20,000 segments of 20 points (cold caches): 45 us with every member
-// in FP64 by four lanes per segment, 13 us now.
+// in FP64 by four lanes per segment, 23 us now.
 #define SF_THREADS 128
 __global__ void __launch_bounds__(SF_THREADS)
     k_segment_fit(const float4 *__restrict__ p, const int4 *__restrict__ range, int S, double q0, double q1,

@@ -41,7 +41,7 @@ struct FeatNorm {
     float ssq[4];
 };
 
-// A warp takes 128 neighbours' worth of queries.  What must be moved is 44 k +
+// A warp takes 128 neighbours' worth of queries.  What must be moved is 20 k +
 // 32 B per query of HBM traffic; what kept the kernel from that rate were
 // the passes through the load/store data path: with one query per warp, 15
 // shuffles per query and three 4-byte stores with a 12-byte stride (each
