@@ -19,6 +19,9 @@
 //   shared memory (summed in rank order) and each CTA goes on with its own
 //   columns.  4,096 rows, 192 -> 256 (cold caches): 27 us by 32 CTAs, 19 us by
 //   128; the gradient as a whole, back to back, 48 -> 38 us.
+//   (C is a power of two, used as a mask: a quotient per K step took a batch
+//   of 34,672 rows, 384 -> 128, where C is 1, from 107 to 115 us; the mask takes
+//   99.5.  An instantiation of its own for C = 1: 107.)
 // k_mlp_dw1_tc — dW1^T = dZ^T X over the batch: one CTA per (128 hidden
 //   units, up to 256 inputs, batch slice); both operands are read K-major
 //   from the transposed copies; the partial products of the batch slices are
@@ -199,7 +202,7 @@ __global__ void __launch_bounds__(MLP_FWD_THREADS, 2) k_mlp_fwd_tc(const __grid_
             const uint4 x = valid ? __ldg((const uint4 *)(a.X + r * a.d_in + s * 16 + half * 8))
                                   : make_uint4(0, 0, 0, 0);
             *(uint4 *)(sA + (size_t)s * 4096 + kmaj_off_bf16(rr, half * 8)) = x;
-            if (train && r < Bp && s % C == crank) {
+            if (train && r < Bp && (s & (C - 1)) == crank) {
                 const uint16_t *xs = (const uint16_t *)&x;
 #pragma unroll
                 for (int j = 0; j < 8; ++j)
@@ -267,7 +270,7 @@ __global__ void __launch_bounds__(MLP_FWD_THREADS, 2) k_mlp_fwd_tc(const __grid_
                 if ((s & 7) == i)
                     x = xq[i];
             *(uint4 *)(sA + st * 4096 + kmaj_off_bf16(rr, half * 8)) = x;
-            if (train && r < Bp && s % C == crank) {
+            if (train && r < Bp && (s & (C - 1)) == crank) {
                 // X^T for the dW1 product (zeros pad the batch to 16)
                 const uint16_t *xs = (const uint16_t *)&x;
 #pragma unroll
