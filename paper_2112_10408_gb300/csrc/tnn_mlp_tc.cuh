@@ -10,9 +10,9 @@
 //   runs.  Epilogue, thread = row = TMEM lane: H = bf16(GELU(Z)), the
 //   256 -> 2 head Y = H W2 + b2; with targets also the MSE gradient dY,
 //   dZ = (dY W2^T) * GELU'(Z) (written transposed for the dW1 product, as is
-//   X), the squared error, and the per-CTA column sums that give db1, dW2 and
-//   db2 (warp reduce-scatter, then the 4 warps' rows summed in a fixed order,
-//   so that training is deterministic).  The epilogue (about 55 instructions
+//   X), and the per-CTA column sums that give db1, dW2, db2 and the squared
+//   error (warp reduce-scatter, then the 4 warps' rows summed in a fixed order,
+//   so that training is deterministic, its loss included).  The epilogue (about 55 instructions
 //   per row and hidden unit when training) bounds it, and a batch of 4,096
 //   has only 32 tiles of rows for 152 SMs: with a cluster every CTA takes 1 /
 //   C of the hidden units, the partial heads are exchanged through distributed
@@ -79,8 +79,7 @@ struct MlpFwdArgs {
     uint16_t *dZt;       // [dh][ldt]
     uint16_t *Xt;        // [d_in][ldt]
     long long ldt;       // >= B rounded up to 16
-    float *pCol;         // [gridDim.x][3 dh + 2]: db1 | dW2 | db2 per CTA
-    float *sse;          // squared error, summed
+    float *pCol;         // [row tiles][3 dh + 3]: db1 | dW2 | db2 | squared error
     float inv_B;
     uint32_t tmem_cols;
     int *err;            // set when a device wait timed out
@@ -95,15 +94,15 @@ struct MlpFwdArgs {
 __host__ __device__ inline size_t mlp_fwd_smem_res(int d_in, int dh)
 {
     const size_t nk = (size_t)d_in / 16;
-    return nk * (4096 + (size_t)dh * 32) + (size_t)dh * 12 + 4 * ((size_t)dh * 3 + 2) * 4 + 2048 + 128;
+    return nk * (4096 + (size_t)dh * 32) + (size_t)dh * 12 + 4 * ((size_t)dh * 3 + 3) * 4 + 2048 + 128;
 }
 
 __host__ __device__ inline size_t mlp_fwd_smem(int dh)
 {
     // 4 stages x (A 4 KB + B dh x 32 B) + b1, W2 (3 dh floats) + column sums
-    // of the 4 lane quadrants (4 x (3 dh + 2) floats) + head partials
+    // of the 4 lane quadrants (4 x (3 dh + 3) floats) + head partials
     // (2 x 128 x 2 floats) + barriers
-    return 4 * (4096 + (size_t)dh * 32) + (size_t)dh * 12 + 4 * ((size_t)dh * 3 + 2) * 4 + 2048 + 128;
+    return 4 * (4096 + (size_t)dh * 32) + (size_t)dh * 12 + 4 * ((size_t)dh * 3 + 3) * 4 + 2048 + 128;
 }
 
 // Sum over the 32 lanes of v[i] for 16 columns i: on return lanes l and
@@ -139,8 +138,8 @@ __global__ void __launch_bounds__(MLP_FWD_THREADS, 2) k_mlp_fwd_tc(const __grid_
     unsigned char *sB = smem + (size_t)nst * 4096; // [nst][bstage]
     float *s_b1 = (float *)(sB + nst * bstage); // [dh]
     float *s_W2 = s_b1 + dh;                  // [dh][2]
-    const int ncol = 3 * dh + 2;
-    float *s_col = s_W2 + 2 * dh;             // [4 quadrants][3 dh + 2]
+    const int ncol = 3 * dh + 3;
+    float *s_col = s_W2 + 2 * dh;             // [4 quadrants][3 dh + 3]
     float *s_y = s_col + 4 * ncol;            // [2 halves][128][2]
     unsigned long long *bars = (unsigned long long *)(s_y + 2 * MLP_ROWS * 2);
     uint32_t *tmem_slot = (uint32_t *)(bars + 8);
@@ -380,9 +379,9 @@ __global__ void __launch_bounds__(MLP_FWD_THREADS, 2) k_mlp_fwd_tc(const __grid_
                     gs1 += __shfl_xor_sync(FULLMASK, gs1, o);
                 }
                 if (lane == 0) {
-                    atomicAdd(a.sse, se);
                     wcol[3 * dh] = gs0;
                     wcol[3 * dh + 1] = gs1;
+                    wcol[3 * dh + 2] = se;
                 }
             }
             const bool padrow = !valid && r < Bp;
@@ -437,10 +436,10 @@ __global__ void __launch_bounds__(MLP_FWD_THREADS, 2) k_mlp_fwd_tc(const __grid_
         atomicOr(a.err, 1);
     if (ok && train)
         for (int i = t; i < ncol; i += MLP_FWD_THREADS) {
-            // local columns db1 | dW2 | db2 to their places among a.dh units
+            // local columns db1 | dW2 | db2, error to their places among a.dh units
             const int at = i < dh ? h0 + i : i < 3 * dh ? a.dh + 2 * h0 + (i - dh) : 3 * a.dh + (i - 3 * dh);
             if (i < 3 * dh || crank == 0)
-                a.pCol[tile * (3 * a.dh + 2) + at] =
+                a.pCol[tile * (3 * a.dh + 3) + at] =
                     ((s_col[i] + s_col[ncol + i]) + s_col[2 * ncol + i]) + s_col[3 * ncol + i];
         }
     if (C > 1)

@@ -375,13 +375,12 @@ struct AdamArgs {
     float *grad_out; // if non-null: write the reduced gradient, no update
     const float *pW1; // [splits1][d_in*dh]
     int splits1;
-    const float *pCol; // [splits2][dh*3+2]
+    const float *pCol; // [splits2][dh*3+3]: the partials of b1 | W2 | b2, of the squared error
     int splits2;
     int d_in, dh;
     long long P;
     float lr, b1, b2, eps, wd;
     const long long *step; // already advanced for this update
-    const float *sse;
     float *loss_out;
     float inv_count;
 };
@@ -401,12 +400,10 @@ __global__ void k_adamw(const __grid_constant__ AdamArgs a)
     }
     __syncthreads();
     const long long p = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (p == 0 && a.loss_out)
-        *a.loss_out = *a.sse * a.inv_count;
-    if (p >= a.P)
+    if (p > a.P || (p == a.P && !a.loss_out)) // p == P: the loss
         return;
     const long long nW1 = (long long)a.d_in * a.dh;
-    const int stride = a.dh * 3 + 2;
+    const int stride = a.dh * 3 + 3;
     // partial sums over the batch slices: eight independent chains, 32 loads in
     // flight (the order is fixed, so the result is deterministic).  The latency
     // of the column sums, one partial per 128 rows of the batch, bounds the
@@ -420,7 +417,7 @@ __global__ void k_adamw(const __grid_constant__ AdamArgs a)
         ld = nW1;
         ns = a.splits1;
     } else {
-        src = a.pCol + (p - nW1); // b1 | W2 | b2 in the same order as pCol
+        src = a.pCol + (p - nW1); // b1 | W2 | b2 | error in the order of pCol
         ld = stride;
         ns = a.splits2;
     }
@@ -442,6 +439,10 @@ __global__ void k_adamw(const __grid_constant__ AdamArgs a)
     for (; s < ns; ++s)
         gs[0] += src[(long long)s * ld];
     const float g = ((gs[0] + gs[1]) + (gs[2] + gs[3])) + ((gs[4] + gs[5]) + (gs[6] + gs[7]));
+    if (p == a.P) {
+        *a.loss_out = g * a.inv_count;
+        return;
+    }
     if (a.grad_out) {
         a.grad_out[p] = g;
         return;
@@ -473,7 +474,6 @@ struct tnn_mlp {
     long long P;
     float *w, *m, *v;
     uint16_t *w1t; // BF16 W1^T in the tensor-core operand order
-    float *acc;    // [0] squared error, [1] loss
     int *err;      // set by a kernel whose device wait timed out
     long long *step; // AdamW step count, on the device (CUDA-graph replays advance it)
     // training workspace, grown on demand
@@ -505,7 +505,6 @@ extern "C" void tnn_mlp_destroy(tnn_mlp *n)
     cudaFree(n->m);
     cudaFree(n->v);
     cudaFree(n->w1t);
-    cudaFree(n->acc);
     cudaFree(n->err);
     cudaFree(n->step);
     delete n;
@@ -539,7 +538,7 @@ static tnn_status mlp_reserve(tnn_mlp *n, long long B)
     A_(n->dY, sizeof(float) * cap * 2);
     A_(n->Y, sizeof(float) * cap * 2);
     A_(n->pW1, sizeof(float) * MLP_MAX_SPLITS * nW1);
-    A_(n->pCol, sizeof(float) * ((cap + MLP_ROWS - 1) / MLP_ROWS) * (3LL * n->dh + 2));
+    A_(n->pCol, sizeof(float) * ((cap + MLP_ROWS - 1) / MLP_ROWS) * (3LL * n->dh + 3));
     A_(n->grad, sizeof(float) * n->P);
     A_(n->Xt, sizeof(uint16_t) * n->d_in * ldt);
     A_(n->dZt, sizeof(uint16_t) * n->dh * ldt);
@@ -595,8 +594,6 @@ extern "C" tnn_status tnn_mlp_create(int32_t d_in, int32_t d_hidden, uint64_t se
         e = cudaMalloc(&n->v, sizeof(float) * n->P);
     if (e == cudaSuccess)
         e = cudaMalloc(&n->w1t, sizeof(uint16_t) * nW1);
-    if (e == cudaSuccess)
-        e = cudaMalloc(&n->acc, sizeof(float) * 4);
     if (e == cudaSuccess)
         e = cudaMalloc(&n->err, sizeof(int));
     if (e == cudaSuccess)
@@ -813,12 +810,9 @@ static tnn_status mlp_forward_impl(const tnn_mlp *n, const uint16_t *d_x, long l
     a.Xt = n->Xt;
     a.ldt = n->ldt;
     a.pCol = n->pCol;
-    a.sse = n->acc;
     a.inv_B = 1.0f / (float)B;
     a.tmem_cols = tmem_cols_for(n->dh);
     a.err = n->err;
-    if (d_t)
-        TNN_CUDA_TRY(cudaMemsetAsync(n->acc, 0, sizeof(float) * 4, st));
     if (!d_t && n->dh % 128 == 0 && n->dh <= 256 &&
         mlp_infer_smem(n->d_in, n->dh) <= (size_t)227 * 1024) {
         // inference: persistent warp-specialised kernel, one CTA per SM
@@ -914,7 +908,6 @@ static tnn_status mlp_backward_impl(tnn_mlp *n, const uint16_t *d_x, long long B
     a.d_in = n->d_in;
     a.dh = n->dh;
     a.P = n->P;
-    a.sse = n->acc;
     a.loss_out = d_loss;
     a.inv_count = 1.0f / (2.0f * (float)B);
     if (opt) {
@@ -925,7 +918,7 @@ static tnn_status mlp_backward_impl(tnn_mlp *n, const uint16_t *d_x, long long B
         a.wd = opt->weight_decay;
         a.step = n->step;
     }
-    TNN_CUDA_TRY(launch_dependent<AdamArgs>(k_adamw, (unsigned)((n->P + 255) / 256), 256, 0, st, a));
+    TNN_CUDA_TRY(launch_dependent<AdamArgs>(k_adamw, (unsigned)((n->P + 256) / 256), 256, 0, st, a));
     return TNN_OK;
 }
 
