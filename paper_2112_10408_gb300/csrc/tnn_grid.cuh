@@ -834,7 +834,7 @@ __global__ void __launch_bounds__(TNN_WARPS_PER_CTA * 32, TileCtas<NL>::value)
             // keys, or within the margin of the settlement.
             constexpr float link = 0x1.02p-23f * (float)SL::n;
             int r0 = NL + TG_EXTRA, r1 = -1;
-            float dn = INFINITY;
+            float dn = INFINITY, dk = 0.0f; // dk: the largest of the first k rows
 #pragma unroll 1
             for (int e = NL + TG_EXTRA - 1; e >= z; e -= TG_ROWS) {
                 unsigned id[TG_ROWS];
@@ -856,11 +856,14 @@ __global__ void __launch_bounds__(TNN_WARPS_PER_CTA * 32, TileCtas<NL>::value)
                             r1 = max(r1, e - u + 1);
                         }
                         dn = d;
+                        if (e - u < NL)
+                            dk = fmaxf(dk, d);
                     }
                 }
             }
-            // every point outside the list lies at or above `bound`
-            const float dk = key_d(*tg_entry(Kw, NL - 1, lane));
+            // every point outside the list lies at or above `bound`: certainly
+            // beyond k listed ones when it is beyond the first k rows, whichever
+            // of them is the farthest (a bucket's rows stand in any order)
             ok = ok && !(bound < fmaf(dk, 0x1.1p-17f, dk) + 0x1p-99f);
             if (W->flags & TNN_FLAG_EXACT_D2) {
                 r0 = z;
