@@ -829,10 +829,14 @@ __global__ void __launch_bounds__(TNN_WARPS_PER_CTA * 32, TileCtas<NL>::value)
         {
             // Exact keys, TG_ROWS rows per step (their gathers in flight
             // together) from the last one down: 64-bit row e covers 32-bit
-            // rows 2 e and 2 e + 1, which every lane has read by then.  Rows r0 .. r1 hold every row that is not certainly
-            // below its successor: not in another bucket of the truncated
-            // keys, or within the margin of the settlement.
-            constexpr float link = 0x1.02p-23f * (float)SL::n;
+            // rows 2 e and 2 e + 1, which every lane has read by then.  Rows
+            // r0 .. r1 hold every row that is not certainly below its
+            // successor: nearer to it than the width of a bucket of truncated
+            // keys (at most 2^-23 n of the distance) plus the settlement's
+            // margin of 2^-17.  The width, because rows behind the successor
+            // may lie lower in its bucket, and rows of r0 .. r1 higher in that
+            // of r1; 2^-21 more covers the products of these factors.
+            constexpr float link = 0x1p-23f * (float)SL::n + 0x1.1p-17f;
             int r0 = NL + TG_EXTRA, r1 = -1;
             float dn = INFINITY, dk = 0.0f; // dk: the largest of the first k rows
 #pragma unroll 1

@@ -77,3 +77,34 @@ def _clusters(k, n, seed):
 def test_distances_on_both_sides_of_a_bucket_boundary(k):
     xyzt, off, q = _clusters(k, 2500, 40 + k)
     _run(xyzt, off, q, k, SIG, K=64, what=f"bucket boundary k={k}", defer_cells=-1.0)
+
+
+def _point(target):
+    """(x, y) whose FP32 distance from the origin, at scales 1, is `target`."""
+    target = np.float32(target)
+    x = np.nextafter(np.float32(np.sqrt(float(target))), np.float32(0.0))
+    while np.float32(float(x) * float(x)) > target:
+        x = np.nextafter(x, np.float32(0.0))
+    base = np.float32(float(x) * float(x))
+    y = np.float32(np.sqrt(max(float(target) - float(base), 0.0)))
+    assert np.float32(float(y) * float(y) + float(base)) == target
+    return float(x), float(y)
+
+
+@pytest.mark.parametrize("slots,k", [(512, 5), (1024, 33)])
+def test_close_distances_two_rows_apart_are_ranked_in_fp64(slots, k):
+    # A: 6 units below a bucket's start (10 of the wider ones), C: 1 above it,
+    # E: at that bucket's end and listed before C.  A and C are within the
+    # settlement's margin of 2^-17 (64 units), so both are ranked in FP64.
+    edge = 64.0 * (1.0 + 4 * slots * 2.0 ** -23)
+    u = 2.0 ** -17
+    below = 6 if slots == 512 else 10
+    near = [(0.125 * (i + 1), 0.0) for i in range(k - 3)]
+    far = [(9.0 + i, 0.0) for i in range(6)]
+    pts = near + [_point(edge - below * u), _point(edge + u), _point(edge + (slots - 1) * u)] + far
+    xyzt = np.array([(x, y, 0.0, float(i)) for i, (x, y) in enumerate(pts)], np.float32)
+    q = np.tile(np.array([[0.0, 0.0, 0.0, 100.0]], np.float32), (3, 1))
+    st = _run(xyzt, np.array([0, len(pts)], np.int64), q, k, (1.0, 1.0, 1.0, 0.0), K=64, what="two rows apart",
+              defer_cells=-1.0)
+    assert st["warp_queries"] == 0
+    assert st["fp64_rechecks"] == 2 * 3
