@@ -790,11 +790,12 @@ __global__ void __launch_bounds__(TNN_WARPS_PER_CTA * 32, TileCtas<NL>::value)
         }
 
         // ---- hand-over of deferred lanes, with a pruning key when the list
-        // is as long as the warp-per-query kernel's
+        // is as long as the warp-per-query kernel's (and the key is a
+        // distance: what lies above that of an overflowed one is no number)
         if (given_up)
             deferred = act;
         if (deferred) {
-            const float hand = !given_up && W->L <= k + TG_EXTRA && o[TG_EXTRA - 1] != TG_EMPTY
+            const float hand = !given_up && W->L <= k + TG_EXTRA && o[TG_EXTRA - 1] < TG_INF
                                    ? SL::upper(o[TG_EXTRA - 1])
                                    : INFINITY;
             const unsigned slot = atomicAdd(&L.scr->n_fallback, 1u);

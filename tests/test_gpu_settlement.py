@@ -108,3 +108,21 @@ def test_close_distances_two_rows_apart_are_ranked_in_fp64(slots, k):
               defer_cells=-1.0)
     assert st["warp_queries"] == 0
     assert st["fp64_rechecks"] == 2 * 3
+
+
+def _overflow(n, seed):
+    """Points and four copies of a query whose squared distances pass FP32's
+    range (they are finite in FP64), scattered so that neither slot nor index
+    order is the distance order."""
+    rng = np.random.default_rng(seed)
+    xyzt = np.zeros((n, 4), np.float32)
+    xyzt[:, :2] = rng.uniform(-1e15, 1e15, (n, 2))
+    xyzt[:, 3] = np.arange(n)
+    return xyzt, np.tile(np.array([[3e16, -1e16, 0.0, 1e4]], np.float32), (4, 1))
+
+
+@pytest.mark.parametrize("k,n", [(8, 13), (20, 40), (32, 36), (64, 90)])
+def test_handed_over_queries_with_overflowed_distances(k, n):
+    xyzt, q = _overflow(n, k + n)
+    st = _run(xyzt, np.array([0, n], np.int64), q, k, (1e6, 1e6, 1.0, 1.0), K=10, what=f"overflow k={k} n={n}")
+    assert st["warp_queries"] == 4
