@@ -870,7 +870,9 @@ __global__ void __launch_bounds__(TNN_WARPS_PER_CTA * 32, TileCtas<NL>::value)
             // beyond k listed ones when it is beyond the first k rows, whichever
             // of them is the farthest (a bucket's rows stand in any order)
             ok = ok && !(bound < fmaf(dk, 0x1.1p-17f, dk) + 0x1p-99f);
-            if (W->flags & TNN_FLAG_EXACT_D2) {
+            // Fewer than k points, perhaps of overflowed distances: these are
+            // equal in FP32 and ranked in FP64.
+            if ((W->flags & TNN_FLAG_EXACT_D2) || !(dk < INFINITY)) {
                 r0 = z;
                 r1 = NL + TG_EXTRA - 1;
             }

@@ -126,3 +126,12 @@ def test_handed_over_queries_with_overflowed_distances(k, n):
     xyzt, q = _overflow(n, k + n)
     st = _run(xyzt, np.array([0, n], np.int64), q, k, (1e6, 1e6, 1.0, 1.0), K=10, what=f"overflow k={k} n={n}")
     assert st["warp_queries"] == 4
+
+
+@pytest.mark.parametrize("k,n", [(8, 5), (20, 19), (20, 40), (64, 40)])
+def test_overflowed_distances_of_a_tile(k, n):
+    # ranked in FP64 also where fewer than k points exist
+    xyzt, q = _overflow(n, k + n)
+    for defer in (0.0, -1.0):
+        _run(xyzt, np.array([0, n], np.int64), q, k, (1e6, 1e6, 1.0, 1.0), K=10, what=f"overflow k={k} n={n}",
+             defer_cells=defer)
