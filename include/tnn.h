@@ -163,7 +163,7 @@ typedef struct {
                               segments are searched for those F
                               (0 = no limit, the default)                     */
     int32_t extra;         /* candidate slots kept beyond k, 2..32 (0 = 4);
-                              the grid order's shared tiles always keep 4     */
+                              the grid order ignores it: its tiles keep 4     */
     int32_t flags;         /* TNN_FLAG_*                                      */
     float defer_cells;     /* grid order: a query whose k-th candidate after
                               seeding is farther than defer_cells grid cells
@@ -440,8 +440,8 @@ void tnn_batch_destroy(tnn_batch *batch);
 /* -------------------------------------------------------------- autotune */
 
 /*
- * Choose the segment order (TNN_FLAG_SWEEP), seed_segments, extra and
- * defer_cells for one index and k by timing
+ * Choose the segment order (TNN_FLAG_SWEEP), seed_segments and defer_cells
+ * (extra is set to 4) for one index and k by timing
  * the search on a sample of self-queries (CUDA events): one run of
  * max(m_sample, 262,144) consecutive indexed points (at most all n) from
  * the middle of the index, so that the sample fills the GPU and takes the

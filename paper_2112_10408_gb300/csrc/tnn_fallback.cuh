@@ -3,7 +3,7 @@
 //     was too large for a shared tile (e.g. a flight's first samples, whose
 //     neighbours are far away); Algorithm 2 puts such unfinished lines
 //     aside and carries on with the others -- they are finished here, where
-//     the whole warp works on one query (list of k + extra candidates);
+//     the whole warp works on one query (32, 64 or 128 candidates by k);
 //   - unsettled (window id stored as -1 - w): the chain of FP32 keys that FP32
 //     cannot order reached the last candidate; here the pruning key is that
 //     of a later rank (a deferred query that ends the same way is run again

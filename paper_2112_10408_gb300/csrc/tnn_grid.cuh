@@ -789,13 +789,13 @@ __global__ void __launch_bounds__(TNN_WARPS_PER_CTA * 32, TileCtas<NL>::value)
                 break;
         }
 
-        // ---- hand-over of deferred lanes, with a pruning key when the list
-        // is as long as the warp-per-query kernel's (and the key is a
-        // distance: what lies above that of an overflowed one is no number)
+        // ---- hand-over of deferred lanes, with a pruning key when k +
+        // TG_EXTRA points lie at or below it (and it is a distance: what lies
+        // above the key of an overflowed one is no number)
         if (given_up)
             deferred = act;
         if (deferred) {
-            const float hand = !given_up && W->L <= k + TG_EXTRA && o[TG_EXTRA - 1] < TG_INF
+            const float hand = !given_up && o[TG_EXTRA - 1] < TG_INF
                                    ? SL::upper(o[TG_EXTRA - 1])
                                    : INFINITY;
             const unsigned slot = atomicAdd(&L.scr->n_fallback, 1u);

@@ -974,25 +974,25 @@ extern "C" tnn_status tnn_autotune(const tnn_index *ix, tnn_knn_params *params,
         tnn_set_error("autotune setup failed: %s", cudaGetErrorString(e));
         s = TNN_ERR_CUDA;
     }
-    // Candidates: the grid order over spare slots and the deferral threshold
-    // (it has no seed count), plus the sweep order with two seed counts.
+    // Candidates: the grid order over the deferral threshold (neither the
+    // seed count nor the spare slots change what it does), plus the sweep
+    // order with two seed counts.
     struct Cand {
-        int F, E, flags;
+        int F, flags;
         float defer;
     };
     std::vector<Cand> cands;
-    for (int E : {4, 8})
-        for (float dfr : {0.6f, 0.75f, 1.0f, 1.5f, 2.0f, 3.0f, 6.0f})
-            cands.push_back({4, E, 0, dfr});
+    for (float dfr : {0.6f, 0.75f, 1.0f, 1.5f, 2.0f, 3.0f, 6.0f})
+        cands.push_back({4, 0, dfr});
     for (int F : {3, 4})
-        cands.push_back({F, 4, TNN_FLAG_SWEEP, 0.0f});
+        cands.push_back({F, TNN_FLAG_SWEEP, 0.0f});
     float best = 1e30f;
     tnn_knn_params bestp = *params;
     for (size_t ci = 0; ci < cands.size() && s == TNN_OK; ++ci) {
         tnn_knn_params p = *params;
         p.seed_segments = cands[ci].F;
         p.seed_window = 0;
-        p.extra = cands[ci].E;
+        p.extra = 4;
         p.flags = (params->flags & ~TNN_FLAG_SWEEP) | cands[ci].flags;
         p.defer_cells = cands[ci].defer;
         s = tnn_knn(ix, (const float *)dq, m, &p, di, dd, nullptr, stream);

@@ -135,3 +135,19 @@ def test_overflowed_distances_of_a_tile(k, n):
     for defer in (0.0, -1.0):
         _run(xyzt, np.array([0, n], np.int64), q, k, (1e6, 1e6, 1.0, 1.0), K=10, what=f"overflow k={k} n={n}",
              defer_cells=defer)
+
+
+def test_spare_slots_make_no_difference_to_the_grid_order():
+    # the grid order keeps lists of its own length: `extra` changes neither the
+    # lists nor the work, nor what a handed-over query takes along
+    wl = synth.flights(60, 80, seed=12, n_routes=5)
+    ix = tnn.tnn_build_segments(torch.from_numpy(wl.xyzt).cuda(), wl.traj_off, SIG, 10)
+    ref = None
+    for extra in (0, 2, 4, 5, 8, 32):
+        gi, gd, st = tnn.tnn_knn(ix, 12, 0.0, extra=extra, defer_cells=0.4, stats=True)
+        assert st["warp_queries"] > 100
+        cur = (gi, gd, st)
+        if ref is None:
+            ref = cur
+        assert torch.equal(cur[0], ref[0]) and torch.equal(cur[1], ref[1])
+        assert cur[2] == ref[2], extra
