@@ -58,6 +58,7 @@ struct WarpSmem {
     int pre[32];
     int kend[32 * WQ_KEYS]; // key ranges of the present round: ends and offsets
     int krel[32 * WQ_KEYS];
+    unsigned long long count[4]; // bounds, distances, segments, FP64 distances
 };
 
 __host__ __device__ inline size_t fb_exact_smem_per_warp(int k_max)
@@ -152,7 +153,8 @@ __global__ void __launch_bounds__(TNN_WARPS_PER_CTA * 32, TNN_WARP_MINB)
     unsigned nfb = *(volatile unsigned *)&L.scr->n_fallback;
     if ((long long)nfb > L.fb_cap)
         nfb = (unsigned)L.fb_cap;
-    unsigned n_lb = 0, n_pairs = 0, n_segs = 0, n_fp = 0;
+    if (lane < 4)
+        S.count[lane] = 0;
     int2 ent = make_int2(0, 0);
     bool retry = false; // the same query again with the larger list
     float tau0 = INFINITY;
@@ -175,6 +177,7 @@ __global__ void __launch_bounds__(TNN_WARPS_PER_CTA * 32, TNN_WARP_MINB)
         }
         const bool unsettled = retry || ent.x < 0;
         const int wid = ent.x < 0 ? -1 - ent.x : ent.x;
+        unsigned n_lb = 0, n_pairs = 0, n_segs = 0, n_fp = 0; // this query's, of this lane
         const KnnWin *W = MANY ? L.wins + wid : &L.w0;
         const float4 q = W->q[ent.y];
         const QCtx c = make_qctx(W, q, true);
@@ -578,17 +581,18 @@ __global__ void __launch_bounds__(TNN_WARPS_PER_CTA * 32, TNN_WARP_MINB)
             else
                 atomicOr(&L.scr->status, 2u);
         }
+        const unsigned v[4] = {n_lb, n_pairs, n_segs, n_fp};
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            const unsigned x = __reduce_add_sync(FULLMASK, v[i]); // at most the index's points
+            if (lane == 0)
+                S.count[i] += x;
+        }
         __syncwarp();
     }
-    unsigned v[4] = {n_lb, n_pairs, n_segs, n_fp};
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-        unsigned long long x = v[i];
-        for (int o = 16; o > 0; o >>= 1)
-            x += __shfl_xor_sync(FULLMASK, x, o);
-        if (lane == 0 && x)
-            atomicAdd(&L.scr->stats[1 + i], x);
-    }
+    __syncwarp();
+    if (lane < 4 && S.count[lane])
+        atomicAdd(&L.scr->stats[1 + lane], S.count[lane]);
     if (blockIdx.x == 0 && threadIdx.x == 0)
         L.scr->stats[5] = nfb;
 }

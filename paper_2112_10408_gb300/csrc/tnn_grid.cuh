@@ -274,10 +274,10 @@ template <int NL> struct TileSmem {
 
 // Kept through all of it: the group's rectangle and the warp's counters
 // (queries, bounds, distances, segments, FP64 distances), which would take
-// registers from the lists.
+// registers from the lists.  A warp can take more than 2^32 distances.
 struct TileKeep {
     GroupBox box;
-    unsigned count[8];
+    unsigned long long count[6];
 };
 
 template <int NL> __host__ __device__ constexpr size_t tg_smem_per_warp()
@@ -387,7 +387,7 @@ __global__ void __launch_bounds__(TNN_WARPS_PER_CTA * 32, TileCtas<NL>::value)
     TileSmem<NL> &S = *(TileSmem<NL> *)ws;
     unsigned long long *Kw = (unsigned long long *)ws;
     TileKeep &KP = *(TileKeep *)(ws + tg_smem_per_warp<NL>() - sizeof(TileKeep));
-    if (lane < 8)
+    if (lane < 6)
         KP.count[lane] = 0;
     __syncwarp();
     pdl_trigger();
@@ -879,7 +879,7 @@ __global__ void __launch_bounds__(TNN_WARPS_PER_CTA * 32, TileCtas<NL>::value)
             if (settle && ok && r0 < r1) {
                 const unsigned r = tg_settle(W, q, Kw, lane, r0, r1);
                 ok = r & 1u;
-                atomicAdd(&KP.count[4], r >> 1);
+                atomicAdd(&KP.count[4], (unsigned long long)(r >> 1));
             }
         }
         if (settle && !ok) {
@@ -959,5 +959,5 @@ __global__ void __launch_bounds__(TNN_WARPS_PER_CTA * 32, TileCtas<NL>::value)
     }
     __syncwarp();
     if (lane < 5 && KP.count[lane])
-        atomicAdd(&L.scr->stats[lane], (unsigned long long)KP.count[lane]);
+        atomicAdd(&L.scr->stats[lane], KP.count[lane]);
 }
