@@ -99,10 +99,12 @@ __global__ void __launch_bounds__(VAL_THREADS)
             bad |= !(in[i].w >= in[i - 1].w);
         double dur = 0.0;
         int sg = seg_off[tr] + lane; // build id of the set
-        for (int f = b + lane * K; f < e; f += 32 * K, sg += 32) {
+        // by the points left: the first point's number may pass 2^31 at the end
+        for (int left = e - b - lane * K; left > 0; left -= 32 * K, sg += 32) {
+            const int f = e - left, cnt = min(K, left);
             const float tA = in[f].w;
-            dur += (double)in[min(f + K - 1, e - 1)].w - (double)tA;
-            range[sg] = make_int4(f, min(K, e - f), tr, 0);
+            dur += (double)in[f + cnt - 1].w - (double)tA;
+            range[sg] = make_int4(f, cnt, tr, 0);
             keys[sg] = ((unsigned long long)f2ord(tA) << 32) | (unsigned)sg;
         }
         for (int o = 16; o > 0; o >>= 1)
@@ -118,7 +120,7 @@ __global__ void __launch_bounds__(VAL_THREADS)
     __shared__ unsigned int s[VAL_THREADS / 32][9];
     unsigned int m[9] = {0u, 0xffffffffu, 0u, 0xffffffffu, 0u, 0xffffffffu, 0u, 0xffffffffu, 0u};
     bool bad = false;
-    for (int i = blockIdx.x * VAL_THREADS + threadIdx.x; i < n; i += pblocks * VAL_THREADS) {
+    for (int64_t i = blockIdx.x * VAL_THREADS + threadIdx.x; i < n; i += pblocks * VAL_THREADS) {
         const float4 v = in[i];
         out[i] = v;
         if (fabsf(v.x) <= 1e15f && fabsf(v.y) <= 1e15f && fabsf(v.z) <= 1e15f && fabsf(v.w) <= 1e15f)
