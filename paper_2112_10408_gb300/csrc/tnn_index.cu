@@ -87,9 +87,10 @@ __global__ void __launch_bounds__(VAL_THREADS)
 {
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     if ((int)blockIdx.x >= pblocks) {
-        for (int i = S + ((int)blockIdx.x - pblocks) * VAL_THREADS + threadIdx.x; i < S2;
-             i += ((int)gridDim.x - pblocks) * VAL_THREADS)
-            keys[i] = ~0ull; // the sort's padding
+        // the sort's padding (32 times the trajectories can pass 2^31)
+        for (int64_t i = S + (int64_t)(blockIdx.x - pblocks) * VAL_THREADS + threadIdx.x; i < S2;
+             i += (int64_t)(gridDim.x - pblocks) * VAL_THREADS)
+            keys[i] = ~0ull;
         const int tr = ((int)blockIdx.x - pblocks) * (VAL_THREADS / 32) + w;
         if (tr >= n_traj) // the same for the whole warp
             return;

@@ -65,3 +65,22 @@ def test_points_up_to_the_limit():
     ix.destroy()
     tnn.tnn_memory_trim()
     torch.cuda.empty_cache()
+
+
+def test_tens_of_millions_of_one_point_trajectories():
+    n = 65_700_000
+    _need(40, 8)
+    x = _points(n)
+    x[:, 3] = (torch.arange(n, device="cuda") * 7919 % (1 << 20)).float()  # in no order, with ties
+    off = np.arange(n + 1, dtype=np.int64)
+    ix = tnn.tnn_build_segments(x, off, (1.0, 1.0, 1.0, 1.0), 2)
+    assert ix.n_segments == n
+    seg, pm = tnn.tnn_index_export(ix)
+    t, first = torch.sort(x[:, 3], stable=True)
+    assert torch.equal(seg[:, 12].contiguous().view(torch.int32), first.int())
+    assert bool((seg[:, 13].contiguous().view(torch.int32) == 1).all())
+    assert torch.equal(seg[:, 3], t) and torch.equal(pm, t)
+    del x, seg, pm, t, first
+    ix.destroy()
+    tnn.tnn_memory_trim()
+    torch.cuda.empty_cache()
