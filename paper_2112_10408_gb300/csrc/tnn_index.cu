@@ -270,11 +270,11 @@ __global__ void __launch_bounds__(SF_THREADS)
         const double r = sqrt(r2) + 1e-12 * (1.0 + (double)mag);
         const float rf = __double2float_ru(r);
         rbits = __float_as_uint(rf); // rf >= 0: the bits order like the values
-        rec[4 * s + 0] = make_float4(Af[0], Af[1], Af[2], pa.w);
-        rec[4 * s + 1] = make_float4(Uf[0], Uf[1], Uf[2], pb.w);
-        rec[4 * s + 2] = make_float4(ABf[0], ABf[1], ABf[2], rf);
-        rec[4 * s + 3] = make_float4(__int_as_float(first), __int_as_float(count),
-                                     __int_as_float(tr), __int_as_float(s));
+        float4 *out = rec + 4 * (size_t)s;
+        out[0] = make_float4(Af[0], Af[1], Af[2], pa.w);
+        out[1] = make_float4(Uf[0], Uf[1], Uf[2], pb.w);
+        out[2] = make_float4(ABf[0], ABf[1], ABf[2], rf);
+        out[3] = make_float4(__int_as_float(first), __int_as_float(count), __int_as_float(tr), __int_as_float(s));
     }
     rbits = __reduce_max_sync(0xffffffffu, rbits); // one atomic per warp
     if ((threadIdx.x & 31) == 0 && rbits != 0u)
@@ -467,10 +467,10 @@ void tnn_bitonic_sort(unsigned long long *keys, int n2, cudaStream_t st)
         return;
     }
     k_bitonic_block<<<n2 / BS_BLOCK, BS_BLOCK / 4, 0, st>>>(keys);
-    for (int k = 2 * BS_BLOCK; k <= n2; k <<= 1) {
-        for (int j = k >> 1; j >= BS_BLOCK; j >>= 1)
-            k_bitonic_global<<<(n2 / 2 + 255) / 256, 256, 0, st>>>(keys, j, k);
-        k_bitonic_merge_local<<<n2 / BS_BLOCK, BS_BLOCK / 4, 0, st>>>(keys, k);
+    for (int64_t k = 2 * BS_BLOCK; k <= n2; k <<= 1) { // n2 is at most 2^30
+        for (int j = (int)(k >> 1); j >= BS_BLOCK; j >>= 1)
+            k_bitonic_global<<<(n2 / 2 + 255) / 256, 256, 0, st>>>(keys, j, (int)k);
+        k_bitonic_merge_local<<<n2 / BS_BLOCK, BS_BLOCK / 4, 0, st>>>(keys, (int)k);
     }
 }
 
@@ -635,11 +635,13 @@ __global__ void __launch_bounds__(1024)
     if (i < S) {
         const int s = (int)(keys[i] & 0xffffffffu);
         pos[s] = i;
-        const float4 a = rec[4 * s], u = rec[4 * s + 1];
-        out[4 * i + 0] = a;
-        out[4 * i + 1] = u;
-        out[4 * i + 2] = rec[4 * s + 2];
-        out[4 * i + 3] = rec[4 * s + 3];
+        const float4 *r = rec + 4 * (size_t)s;
+        float4 *o = out + 4 * (size_t)i;
+        const float4 a = r[0], u = r[1];
+        o[0] = a;
+        o[1] = u;
+        o[2] = r[2];
+        o[3] = r[3];
         tA[i] = a.w;
         tB = u.w;
     }
@@ -659,7 +661,7 @@ __global__ void __launch_bounds__(1024) k_pm_apply(const float4 *__restrict__ se
         c = fmaxf(c, bmax[b]);
     const float carry = block_max_1024(c, sh);
     const int i = blockIdx.x * 1024 + threadIdx.x;
-    float v = i < S ? seg[4 * i + 1].w : -INFINITY;
+    float v = i < S ? seg[4 * (size_t)i + 1].w : -INFINITY;
     for (int o = 1; o < 32; o <<= 1) {
         const float u = __shfl_up_sync(0xffffffffu, v, o);
         if (lane >= o)
@@ -752,7 +754,8 @@ __global__ void k_grid_extents(const float4 *__restrict__ seg, int S, const __gr
     const int p = blockIdx.x * blockDim.x + threadIdx.x; // build id
     if (p >= S)
         return;
-    const float4 a = seg[4 * p], u = seg[4 * p + 1], b = seg[4 * p + 2];
+    const float4 *r = seg + 4 * (size_t)p;
+    const float4 a = r[0], u = r[1], b = r[2];
     int bk, cx, cy;
     const int key = grid_key(g, a.w, a.x, a.y, b.x, b.y, bk, cx, cy);
     // every cylinder point is within |AB|/2 + r of the midpoint

@@ -41,9 +41,10 @@ def _check_search(ix, rows):
     assert d2.cpu().numpy().tolist() == [[0.3125, 0.8125, 1.8125, 2.3125]] * rows.size
 
 
-def test_points_up_to_the_limit():
-    n, K, length = (1 << 31) - 65, 64, 1 << 15
-    _need(130, 8)
+@pytest.mark.parametrize("n,K,length,device_gb", [((1 << 31) - 65, 64, 1 << 15, 130),
+                                                  ((1 << 30) + 4, 2, 1 << 10, 215)])  # 2^29 + 2 segments
+def test_points_up_to_the_limit(n, K, length, device_gb):
+    _need(device_gb, 8)
     x = _points(n)
     off = np.append(np.arange(0, n, length), n).astype(np.int64)
     ix = tnn.tnn_build_segments(x, off, (1.0, 1.0, 1.0, 1.0), K)
@@ -52,15 +53,15 @@ def test_points_up_to_the_limit():
     seg, pm = tnn.tnn_index_export(ix)
     s = torch.arange(S, device="cuda")
     first = seg[:, 12].contiguous().view(torch.int32)
-    # four segments begin with every second: t_A order is the build order
-    assert torch.equal(first, (64 * s).int())
+    # 256 / K segments begin with every second: t_A order is the build order
+    assert torch.equal(first, (K * s).int())
     count = seg[:, 13].contiguous().view(torch.int32)
     assert bool((count[:-1] == K).all()) and int(count[-1]) == n - K * (S - 1)
-    assert torch.equal(seg[:, 3], ((64 * s) >> 8).float()) and torch.equal(pm, seg[:, 7])
-    last = torch.clamp(64 * s + 63, max=n - 1)
+    assert torch.equal(seg[:, 3], ((K * s) >> 8).float()) and torch.equal(pm, seg[:, 7])
+    last = torch.clamp(K * s + K - 1, max=n - 1)
     assert torch.equal(seg[:, 7], (last >> 8).float())
-    assert torch.equal(seg[:, 0], ((64 * s) & 255).float())
-    _check_search(ix, [n - 10, n - 200, (1 << 30) + 77, (1 << 20) + 50, 130 * 256 + 5, 2 * 256 + 66])
+    assert torch.equal(seg[:, 0], ((K * s) & 255).float())
+    _check_search(ix, [n - 10, n - 200, (1 << 29) + 77, (1 << 20) + 50, 130 * 256 + 5, 2 * 256 + 66])
     del x, seg, pm, s, first, count, last
     ix.destroy()
     tnn.tnn_memory_trim()
