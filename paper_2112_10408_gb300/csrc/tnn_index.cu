@@ -1194,6 +1194,11 @@ extern "C" tnn_status tnn_build_segments(const float *d_xyzt, int64_t n,
         S += (uint32_t)(len + K - 1) / (uint32_t)K; // len < 2^31
         nt += (len + 31) >> 5;
     }
+    // the sorts take a power of two of keys in 32-bit places
+    if (S > (1ll << 30)) {
+        tnn_set_error("index allocation failed: %lld segments, at most 2^30 are possible", (long long)S);
+        return TNN_ERR_OOM;
+    }
     cudaStream_t st = (cudaStream_t)stream;
 
     tnn_index *ix = new tnn_index();
