@@ -7,7 +7,8 @@ self-query of all points of the medium trajectory workload (2,000 synthetic
 flights x 200 samples = 400,000 points, k = 32, 20-point segments, scales
 (1, 1, 10, 0.01), mask t_j < t_i).  Inputs are resident in HBM; L2 is
 flushed (256 MiB write) before every timed step.  The JSON line follows the
-repository's benchmark contract.
+repository's benchmark contract; everything else that is measured (work
+counters, rooflines by kernel, other workloads) goes to the file --details.
 
   python bench.py [--gpus N] [--steps K] [--warmup W] [--impl ours|reference]
 """
@@ -88,7 +89,38 @@ def _args():
                     help="skip the batched-window and nowcast measurements")
     ap.add_argument("--tuning", choices=["auto", "default"], default="auto",
                     help="autotune the seed/extra knobs (auto) or use the library defaults")
+    ap.add_argument("--details", default=os.path.join(ROOT, "build", "bench_details.json"),
+                    help="file for the measurements beside the printed line")
     return ap.parse_args()
+
+
+def _line(out):
+    """The printed line: the contract's keys and the head figures of the rest,
+    short enough for a reader of the output's last lines."""
+    def pick(d, *keys):
+        return {k: d[k] for k in keys if k in d} if d else None
+    line = pick(out, "metric", "value", "unit", "n_gpus", "steps", "warmup", "ms_per_step", "higher_is_better",
+                "scaling", "vs_baseline", "dtype", "data", "config", "impl", "clocks")
+    line["e2e"] = pick(out["e2e"], "value", "unit", "h2d_bytes_per_step", "d2h_bytes_per_step", "ms_per_step")
+    line["gpu_launches"] = out["gpu_launches"]
+    line["roofline"] = pick(out.get("roofline"), "bound", "achieved", "peak", "unit", "frac", "traffic", "kernel",
+                            "kernel_ms")
+    cpu = out.get("cpu_baseline")
+    line["cpu_baseline"] = pick(cpu, "value", "unit", "cores", "kind")
+    if cpu and "parity" in cpu:
+        line["cpu_baseline"].update(pick(cpu["parity"], "queries_checked", "identical_indices"))
+    line["comparator"] = {k: pick(v, "ms_per_step", "tnn_speedup", "identical_neighbours")
+                          for k, v in (out.get("comparator") or {}).items()}
+    return line
+
+
+def _write_details(out, path):
+    try:
+        os.makedirs(os.path.dirname(os.path.abspath(path)), exist_ok=True)
+        with open(path, "w") as f:
+            json.dump(out, f)
+    except OSError as e:
+        print(f"details not written: {e}", file=sys.stderr)
 
 
 def _workload(name, rank):
@@ -1011,7 +1043,8 @@ def run_ours(a):
                "stats_per_step": st, "e2e_breakdown": e2e_break, "tc_tiles": tc_tiles}
         if extras:
             out.update(extras)
-        print(json.dumps(out))
+        _write_details(out, a.details)
+        print(json.dumps(_line(out)))
     if world > 1:
         dist.destroy_process_group()
     return 0
