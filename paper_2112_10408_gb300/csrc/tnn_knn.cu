@@ -331,7 +331,12 @@ static tnn_status finish_search(const KnnLaunch &L, cudaStream_t st, bool prof, 
     }
     if (prof)
         TNN_CUDA_TRY(cudaEventRecord(pr.e[2], st));
-    TNN_CUDA_TRY(launch_dependent<KnnLaunch>(k_fallback_exact, (unsigned)g_num_sms, TNN_WARPS_PER_CTA * 32,
+    // Its CTAs take their places under the tail of the kernel before, on the
+    // SMs that fall free first: with one per SM they crowded on some of them
+    // (80,000 queries over as many points, each place 40 times: 155 ms, 136 ms
+    // when launched plainly, which costs every search 2.5 us), with two 78 ms,
+    // with four 40 ms.  Idle ones cost nothing measurable.
+    TNN_CUDA_TRY(launch_dependent<KnnLaunch>(k_fallback_exact, 4u * (unsigned)g_num_sms, TNN_WARPS_PER_CTA * 32,
                                              fb_exact_smem_per_warp(L.L_max) * TNN_WARPS_PER_CTA, st, L));
     if (prof) {
         TNN_CUDA_TRY(cudaEventRecord(pr.e[3], st));

@@ -151,3 +151,16 @@ def test_spare_slots_make_no_difference_to_the_grid_order():
             ref = cur
         assert torch.equal(cur[0], ref[0]) and torch.equal(cur[1], ref[1])
         assert cur[2] == ref[2], extra
+
+
+@pytest.mark.parametrize("k", [8, 16])
+def test_more_queries_by_the_definition_than_warps(k):
+    # every place 40 times: chains longer than the lists, so nearly every one
+    # of 6,000 queries is answered by the FP64 definition
+    rng = np.random.default_rng(k)
+    base = np.sort(rng.uniform(0.0, 60.0, (150, 4)), axis=0)
+    xyzt = np.repeat(base, 40, axis=0).astype(np.float32)
+    q = xyzt.copy()
+    q[:, 3] += 0.25
+    st = _run(xyzt, np.array([0, 2000, 6000], np.int64), q, k, SIG, K=10, what="copies")
+    assert st["exact_queries"] > 5000
