@@ -89,7 +89,7 @@ typedef struct {
  * bounding box and durations read back at the same time); the segment fit,
  * the sorts and the grid are enqueued after it and run on in stream order
  * after the call returns.  On success *out owns device memory until
- * tnn_index_destroy.
+ * tnn_index_destroy.  More than 2^30 segments are TNN_ERR_OOM.
  */
 tnn_status tnn_build_segments(const float *d_xyzt, int64_t n,
                               const int64_t *h_traj_off, int64_t n_traj,

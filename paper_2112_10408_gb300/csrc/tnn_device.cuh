@@ -26,8 +26,7 @@ __host__ __device__ inline size_t smem_per_warp(int L_max, int kseg_max, int mod
     size_t base = (size_t)L_max * 32 * 8;
     size_t rest = mode == SMEM_LINEAR
                       ? (32 * 16 + 32 * 4)
-                      : (2048 + (size_t)kseg_max * 16 +
-                         4 * (TNN_UCAP + (mode == SMEM_SWEEP ? TNN_WCAP : 0)));
+                      : (2048 + (size_t)kseg_max * 16 + 4 * (TNN_UCAP + TNN_WCAP));
     size_t cl = (size_t)CMAX * 32 * 12;
     if (rest < cl)
         rest = cl;

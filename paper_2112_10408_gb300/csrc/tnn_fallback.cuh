@@ -4,10 +4,11 @@
 //     neighbours are far away); Algorithm 2 puts such unfinished lines
 //     aside and carries on with the others -- they are finished here, where
 //     the whole warp works on one query (32, 64 or 128 candidates by k);
-//   - unsettled (window id stored as -1 - w): the chain of FP32 keys that FP32
-//     cannot order reached the last candidate; here the pruning key is that
-//     of a later rank (a deferred query that ends the same way is run again
-//     at once like that).
+//   - unsettled (window id stored as -1 - w): a point outside the tile's list
+//     could belong to the first k, or a chain of distances that FP32 cannot
+//     order was too long for the tile; here the pruning key is that of a later
+//     rank (a deferred query that ends the same way is run again at once like
+//     that).
 //
 // k_tnn_warp: the 32 lanes split the grid keys, the member segments and the
 // member points of one query.  Its candidates are sorted 32-bit keys (the

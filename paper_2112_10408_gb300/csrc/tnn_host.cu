@@ -155,10 +155,13 @@ static tnn_status run_copied(tnn_index *ix, int64_t n, const tnn_knn_params *kp,
     return TNN_OK;
 }
 
-// One window of all n self-queries: the tile kernel mirrors every finished
-// tile's rows into the mapped outputs m_idx, m_d2 as it goes, the per-query
-// kernels then finish the handed-over queries in the device lists, and
-// k_patch_rows writes those rows into the mapped outputs.  All on `st`.
+// One window of all n self-queries.  In grid order the tile kernel writes the
+// rows it settles to the mapped outputs m_idx, m_d2 only and leaves them out of
+// the device lists; the sweep's writes every row to the device lists and each
+// finished tile to the mapped outputs as well.  The per-query kernels finish
+// the handed-over queries in the device lists, and k_patch_rows copies those
+// rows, every one that a list of hand-overs names, into the mapped outputs.
+// All on `st`; only the mapped outputs are complete at the end.
 static tnn_status run_mapped(tnn_index *ix, int64_t n, const tnn_knn_params *kp, int32_t *d_idx,
                              float *d_d2, int32_t *m_idx, float *m_d2, cudaStream_t st)
 {

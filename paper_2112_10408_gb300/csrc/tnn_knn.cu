@@ -43,10 +43,13 @@
 //   A candidate enters a list iff its distance does not exceed the list's
 //   pruning key, so a segment whose bound exceeds that key cannot contribute.
 //   Settlement: if d32(b) > d32(a)(1 + 2^-17) + 2^-100 then d2(b) > d2(a);
-//   maximal chains of keys closer than that are re-ranked in FP64.  When the
-//   chain holding rank k reaches the last kept slot of a full candidate
-//   list, points outside the list could belong to it: that query is
-//   answered again by the warp scans of tnn_fallback.cuh.
+//   maximal chains of keys closer than that are re-ranked in FP64.  Points
+//   outside a full candidate list could belong to the first k when (sweep and
+//   linear search) the chain holding rank k reaches the last kept slot, or
+//   (grid order) the smallest distance outside is not beyond that margin of
+//   the largest among the first k listed: that query is answered again by the
+//   warp scans of tnn_fallback.cuh, whose list of 32, 64 or 128 follows the
+//   chain again, and by the FP64 definition if that fails too.
 #include <math.h>
 #include <string.h>
 

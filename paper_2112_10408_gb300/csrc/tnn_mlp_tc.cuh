@@ -18,7 +18,7 @@
 //   C of the hidden units, the partial heads are exchanged through distributed
 //   shared memory (summed in rank order) and each CTA goes on with its own
 //   columns.  4,096 rows, 192 -> 256 (cold caches): 27 us by 32 CTAs, 19 us by
-//   128; the gradient as a whole, back to back, 48 -> 38 us.
+//   128; the gradient as a whole, back to back, 48 -> 38 us (30.7 with what followed).
 //   (C is a power of two, used as a mask: a quotient per K step took a batch
 //   of 34,672 rows, 384 -> 128, where C is 1, from 107 to 115 us; the mask takes
 //   99.5.  An instantiation of its own for C = 1: 107.)

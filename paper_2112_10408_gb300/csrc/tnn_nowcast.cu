@@ -408,7 +408,9 @@ __global__ void k_adamw(const __grid_constant__ AdamArgs a)
     // flight (the order is fixed, so the result is deterministic).  The latency
     // of the column sums, one partial per 128 rows of the batch, bounds the
     // kernel: with eight loads in flight a gradient of 34,672 rows (384 -> 128)
-    // took 99.5 us and one of 4,096 (192 -> 256) 34.0, now 94.4 and 31.5.
+    // took 99.5 us and one of 4,096 (192 -> 256) 34.0, then 94.4 and 31.5 (30.7
+    // with the squared error as one more column instead of atomics behind a
+    // memset, whose order changed its last bits from call to call).
     const float *src;
     long long ld;
     int ns;
